@@ -29,160 +29,124 @@ using namespace bucket;
 #ifndef HT_BUCKET_MIN_BLOCKS
 #define HT_BUCKET_MIN_BLOCKS 3
 #endif
+#ifndef HT_BUCKET_LOOKUP_MIN_BLOCKS
+#define HT_BUCKET_LOOKUP_MIN_BLOCKS 3
+#endif
 
-// Plain find-or-put over one table.  The next tile's keys are loaded while
-// the current tile waits on the table.  (Pipelining tile i's claims with tile
-// i+1's bucket reads was measured slower on GB300: the extra live state costs
-// occupancy, and occupancy is what hides the table's latency here.)
+// find-or-put or lookup over one table.  A warp takes a fresh tile of 32 keys,
+// or 32 of its queued ones when that many wait (and the rest at the end), for
+// one pass over one bucket each (bucket_pass); the next two tiles' keys are
+// being loaded meanwhile.  A lookup in a table larger than L2 (ahead) also
+// touches the next tile's buckets, so that its reads hit L2.  Bound by random
+// 128-byte lines once the table is past L2 (40-46 G lines/s, 25 G/s where the
+// line is also written): find-or-put 22.8 G keys/s over a fill of 2^27 keys to
+// load 0.8 (19.2 with keys settled inside the tile), 41 on the successors of
+// 10^8 states (29); lookups 38 G/s (22; 31 without touching ahead, which gives
+// find-or-put nothing: its claims take the time).
+template <int KW, int BS, int G, bool VALUES, bool APPEND, bool LOOKUP>
+__device__ __forceinline__ void bucket_tiles(const DevTable& t, const void* keys, const uint32_t* vals, uint64_t n,
+                                             uint8_t* flags, uint32_t* out_val, typename Keys<KW>::T* new_out,
+                                             unsigned long long* new_count, uint64_t new_cap, bool ahead) {
+    using K = Keys<KW>;
+    using T = typename K::T;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
+    unsigned long long stored = 0;
+    __shared__ T s_new[APPEND ? kBlock / 32 : 1][APPEND ? kStageCap : 1];   // new keys awaiting the append
+    __shared__ PendEntry s_pend[kBlock / 32][kPend];
+    WarpStage<T, kStageCap> stage(s_new[APPEND ? warp : 0]);
+    Pending pend(s_pend[warp]);
+    uint64_t base = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) / 32 * 32;
+    // This tile's key and bucket, the next tile's key.
+    uint64_t key0 = 0, key1 = 0;
+    uint32_t val0 = 0, val1 = 0;
+    if (base + lane < n) {
+        key0 = K::load(keys, base + lane);
+        if (VALUES && !LOOKUP) val0 = vals[base + lane];
+    }
+    if (base + step + lane < n) {
+        key1 = K::load(keys, base + step + lane);
+        if (VALUES && !LOOKUP) val1 = vals[base + step + lane];
+    }
+    uint64_t bkt0 = hidx(key0, t.seed[0], t.nbuckets);
+    // Bounded: an iteration takes a tile or up to 32 queued keys, and a key is
+    // queued at most once for each slot of its k buckets.
+    for (;;) {
+        PendEntry d;
+        uint64_t bkt;
+        bool mine, ok;
+        if (pend.n >= 32 || (base >= n && pend.n)) {
+            d.key = d.pos = 0;
+            d.val = d.f = 0;
+            mine = ok = pend.pop(d);
+            bkt = hidx(d.key, t.seed[d.f], t.nbuckets);
+        } else if (base < n) {
+            d.key = key0;
+            d.pos = base + lane;
+            d.val = val0;
+            d.f = 0;
+            bkt = bkt0;
+            mine = d.pos < n;
+            ok = mine && !K::reserved(d.key);
+            if (mine && !ok) set_flag(t.ctr, kFlagInvalidKey);
+            key0 = key1;
+            val0 = val1;
+            bkt0 = hidx(key0, t.seed[0], t.nbuckets);
+            if (LOOKUP && ahead && base + step + lane < n) touch_l2(t.slots + bkt0 * BS);
+            if (base + 2 * step + lane < n) {
+                key1 = K::load(keys, base + 2 * step + lane);
+                if (VALUES && !LOOKUP) val1 = vals[base + 2 * step + lane];
+            }
+            base += step;
+        } else {
+            break;
+        }
+        uint32_t v = 0;
+        uint32_t st = bucket_pass<KW, BS, G, VALUES, LOOKUP>(t.slots, d.key, d.val, bkt, ok, &v);
+        bool waits;
+        if constexpr (LOOKUP) {
+            const bool next = st == kKeyFull;
+            if (next && ++d.f >= t.k) st = spill_find<KW>(t, d.key, &v);
+            waits = st == kKeyFull;
+            if (waits && ahead) touch_l2(t.slots + hidx(d.key, t.seed[d.f], t.nbuckets) * BS);
+            pend.push(waits, d.key, 0, d.pos, d.f);
+        } else {
+            st = settle_put<KW>(t, pend, st, d.key, d.val, d.pos, d.f, waits);
+            stored += st == kKeyHit;
+            if (APPEND) stage.push(st == kKeyHit, T(d.key), new_out, new_count, new_cap);
+        }
+        if (mine && !waits) {
+            if (flags) flags[d.pos] = uint8_t(st);
+            if (LOOKUP && VALUES) out_val[d.pos] = v;
+        }
+    }
+    if (APPEND) stage.flush(new_out, new_count, new_cap);
+    if (!LOOKUP) add_size<kBlock>(t, stored);
+}
+
 template <int KW, int BS, int G, bool VALUES, bool APPEND>
 __global__ void __launch_bounds__(kBlock, HT_BUCKET_MIN_BLOCKS)
-bucket_fop_kernel(const DevTable t, const void* __restrict__ keys, const uint32_t* __restrict__ vals,
+bucket_fop_kernel(const __grid_constant__ DevTable t, const void* __restrict__ keys, const uint32_t* __restrict__ vals,
                   uint64_t n, const unsigned long long* __restrict__ d_n, uint8_t* __restrict__ is_new,
                   typename Keys<KW>::T* __restrict__ new_out, unsigned long long* __restrict__ new_count,
                   uint64_t new_cap) {
     if (d_n) n = min(n, uint64_t(__ldcg(d_n)));        // batch size produced on the device
-    using K = Keys<KW>;
-    using T = typename K::T;
-    const int lane = threadIdx.x & 31;
-    const uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
-    const uint64_t step = nwarps * 32;
-    unsigned long long stored = 0;
-    __shared__ T s_new[APPEND ? kBlock / 32 : 1][APPEND ? kStageCap : 1];   // new keys awaiting the append
-    WarpStage<T, kStageCap> stage(s_new[APPEND ? (threadIdx.x >> 5) : 0]);
-    uint64_t base = ((uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * 32;
-    uint64_t next_key = 0;
-    uint32_t next_val = 0;
-    if (base + lane < n) {
-        next_key = K::load(keys, base + lane);
-        if (VALUES) next_val = vals[base + lane];
-    }
-    for (; base < n; base += step) {
-        const bool mine = base + lane < n;
-        const uint64_t mykey = next_key;
-        const uint32_t myval = next_val;
-        if (base + step + lane < n) {
-            next_key = K::load(keys, base + step + lane);
-            if (VALUES) next_val = vals[base + step + lane];
-        }
-        const bool myok = mine && !K::reserved(mykey);
-        if (mine && !myok) set_flag(t.ctr, kFlagInvalidKey);
-        const uint32_t my_new = bucket_tile<KW, BS, G>(t, mykey, myval, myok);
-        if (mine && is_new) is_new[base + lane] = uint8_t(my_new);
-        if (APPEND) stage.push(mine && my_new, T(mykey), new_out, new_count, new_cap);
-        stored += __popc(__ballot_sync(kFull, my_new != 0));
-    }
-    if (APPEND) stage.flush(new_out, new_count, new_cap);
-    if ((threadIdx.x & 31) == 0 && stored) atomicAdd(&t.ctr->size, stored);
+    bucket_tiles<KW, BS, G, VALUES, APPEND, false>(t, keys, vals, n, is_new, nullptr, new_out, new_count, new_cap,
+                                                   false);
 }
 
 // Lookup: like find-or-put without claims; a bucket with a free slot ends the
 // search (a key only moves on from a full bucket), all k full -> the spill.
-// One round at a time: a read-only probe gains more from the occupancy of a
-// small register footprint than from reading all rounds up front (measured:
-// 24.7 vs 20.1 G lookups/s on 2^27 keys at load 0.8).
-template <int KW, int BS, int G>
-__global__ void __launch_bounds__(kBlock)
-bucket_lookup_kernel(const DevTable t, const void* __restrict__ keys, uint64_t n,
-                     uint32_t* __restrict__ vals, uint8_t* __restrict__ found) {
-    using K = Keys<KW>;
-    constexpr int SPL = BS / G;
-    constexpr int GPW = 32 / G;
-    constexpr int PF = Prefetch<G, SPL>::kRounds;
-    constexpr uint32_t kGMask = (G == 32) ? 0xFFFFFFFFu : ((1u << G) - 1u);
-    const int lane = threadIdx.x & 31;
-    const int grp = lane / G, sub = lane % G, gbase = grp * G;
-    const uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
-    const uint32_t stash_used = __ldcg(&t.ctr->stash_used);
-    const uint32_t ovf_used = __ldcg(&t.ctr->ovf_used);
-
-    for (uint64_t base = ((uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * 32; base < n;
-         base += nwarps * 32) {
-        const bool mine = base + lane < n;
-        const uint64_t mykey = mine ? K::load(keys, base + lane) : 0;
-        const bool myok = mine && !K::reserved(mykey);
-        if (mine && !myok) set_flag(t.ctr, kFlagInvalidKey);
-        const uint64_t mybkt = hidx(mykey, t.seed[0], t.nbuckets);
-        uint32_t my_found = 0, my_val = 0;
-#pragma unroll 1
-        for (int r0 = 0; r0 < G; r0 += PF) {
-            uint64_t w[PF][SPL];
-#pragma unroll
-            for (int q = 0; q < PF; ++q) {
-                const int kidx = (r0 + q) * GPW + grp;
-                const uint64_t b = __shfl_sync(kFull, mybkt, kidx);
-                const bool ok = __shfl_sync(kFull, myok, kidx);
-                if (ok) {
-                    load_lane<SPL>(t.slots + b * BS + sub * SPL, w[q]);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < SPL; ++j) w[q][j] = kEmpty;
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < PF; ++q) {
-                const int kidx = (r0 + q) * GPW + grp;
-                const uint64_t key = __shfl_sync(kFull, mykey, kidx);
-                int state = __shfl_sync(kFull, myok, kidx) ? kRead : kDone;
-                uint64_t cur[SPL];
-#pragma unroll
-                for (int j = 0; j < SPL; ++j) cur[j] = w[q][j];
-                uint32_t lm, le;
-                scan_lane<KW, SPL>(cur, key, lm, le);
-                uint32_t f = 0, res_found = 0, res_val = 0;
-                while (__any_sync(kFull, state != kDone)) {
-                    const uint32_t Mb = __ballot_sync(kFull, state == kRead && lm != 0);
-                    const uint32_t M = (Mb >> gbase) & kGMask;
-                    const uint32_t E = (__ballot_sync(kFull, state == kRead && le != 0) >> gbase) & kGMask;
-                    uint32_t v = 0;
-                    if (lm) {
-                        const int j = __ffs(lm) - 1;
-#pragma unroll
-                        for (int jj = 0; jj < SPL; ++jj)
-                            if (jj == j) v = K::value(cur[jj]);
-                    }
-                    const int owner = M ? gbase + __ffs(M) - 1 : lane;
-                    v = __shfl_sync(kFull, v, owner);
-                    if (state == kRead) {
-                        if (M) {
-                            res_found = 1;
-                            res_val = v;
-                            state = kDone;
-                        } else if (E) {
-                            state = kDone;
-                        } else if (++f < t.k) {
-                            const uint64_t b = hidx(key, t.seed[f], t.nbuckets);
-                            load_lane<SPL>(t.slots + b * BS + sub * SPL, cur);
-                            scan_lane<KW, SPL>(cur, key, lm, le);
-                        } else {
-                            state = kSpill;
-                        }
-                    }
-                    if (state == kSpill) {
-                        if (sub == 0) {
-                            uint64_t sw;
-                            if (find_spill<KW>(t, key, stash_used, ovf_used, &sw)) {
-                                res_found = 1;
-                                res_val = K::value(sw);
-                            }
-                        }
-                        state = kDone;
-                    }
-                }
-                const int src = ((lane - (r0 + q) * GPW) & (GPW - 1)) * G;
-                const uint32_t gf = __shfl_sync(kFull, res_found, src);
-                const uint32_t gv = __shfl_sync(kFull, res_val, src);
-                if (lane / GPW == r0 + q) {
-                    my_found = gf;
-                    my_val = gv;
-                }
-            }
-        }
-        if (mine) {
-            if (found) found[base + lane] = uint8_t(my_found);
-            if (vals) vals[base + lane] = my_val;
-        }
-    }
+template <int KW, int BS, int G, bool VALUES>
+__global__ void __launch_bounds__(kBlock, HT_BUCKET_LOOKUP_MIN_BLOCKS)
+bucket_lookup_kernel(const __grid_constant__ DevTable t, const void* __restrict__ keys, uint64_t n,
+                     uint32_t* __restrict__ vals, uint8_t* __restrict__ found, bool ahead) {
+    bucket_tiles<KW, BS, G, VALUES, false, true>(t, keys, nullptr, n, found, vals, nullptr, nullptr, 0, ahead);
 }
+
+// A table larger than L2: a lookup touches its buckets one tile ahead.  Below
+// that the reads hit L2 anyway and this is one more L2 request per key.
+bool past_l2(const DevTable& t) { return t.nslots * 8 > l2_bytes(); }
 
 template <int KW, int BS, int G>
 cudaError_t launch_fop(const DevTable& t, const void* keys, const uint32_t* vals, uint64_t n,
@@ -190,40 +154,34 @@ cudaError_t launch_fop(const DevTable& t, const void* keys, const uint32_t* vals
                        unsigned long long* new_count, uint64_t new_cap, cudaStream_t s, const L2Window& w) {
     using T = typename Keys<KW>::T;
     ProfScope ps(kKBucketFop, s);
-    if (vals) {
-        auto k = bucket_fop_kernel<KW, BS, G, true, false>;
-        return launch_win(k, launch_blocks((const void*)k, kBlock), kBlock, s, w, t, keys, vals, n, d_n, is_new,
-                          (T*)nullptr, (unsigned long long*)nullptr, uint64_t(0));
-    } else if (new_out) {
-        auto k = bucket_fop_kernel<KW, BS, G, false, true>;
-        return launch_win(k, launch_blocks((const void*)k, kBlock), kBlock, s, w, t, keys, (const uint32_t*)nullptr, n,
-                          d_n, is_new, static_cast<T*>(new_out), new_count, new_cap);
-    }
-    auto k = bucket_fop_kernel<KW, BS, G, false, false>;
-    return launch_win(k, launch_blocks((const void*)k, kBlock), kBlock, s, w, t, keys, (const uint32_t*)nullptr, n, d_n,
-                      is_new, (T*)nullptr, (unsigned long long*)nullptr, uint64_t(0));
+    auto k = vals ? bucket_fop_kernel<KW, BS, G, KW == 32, false>
+             : new_out ? bucket_fop_kernel<KW, BS, G, false, true> : bucket_fop_kernel<KW, BS, G, false, false>;
+    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, keys, vals, n, d_n, is_new,
+                      static_cast<T*>(new_out), new_count, new_cap);
 }
 
 template <int KW, int BS, int G>
 cudaError_t launch_lookup(const DevTable& t, const void* keys, uint64_t n, uint32_t* vals,
                           uint8_t* found, cudaStream_t s, const L2Window& w) {
     ProfScope ps(kKBucketLookup, s);
-    auto k = bucket_lookup_kernel<KW, BS, G>;
-    return launch_win(k, launch_blocks((const void*)k, kBlock), kBlock, s, w, t, keys, n, vals, found);
+    auto k = vals ? bucket_lookup_kernel<KW, BS, G, true> : bucket_lookup_kernel<KW, BS, G, false>;
+    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, keys, n, vals, found,
+                      past_l2(t));
 }
 
 // Multi-table find-or-put of one step (the body is shared with the
 // persistent kernel, bucket::multi_find_or_put).
 template <int BS, int G>
 __global__ void __launch_bounds__(kBlock, HT_BUCKET_MIN_BLOCKS)
-multi_bucket_fop_kernel(const MultiDev m, uint64_t) {
+multi_bucket_fop_kernel(const __grid_constant__ MultiDev m, uint64_t) {
     __shared__ uint64_t s_new[kBlock / 32][kStageCap];
     __shared__ unsigned int s_first[multi::kExactTileExpl + 1];
     __shared__ unsigned long long s_scan[multi::kAdvShared];
+    __shared__ PendEntry s_pend[kBlock / 32][kPend];
     const multi::TileMap tm = multi::tile_map<kBlock>(m, s_first, s_scan);
     const uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
     const uint64_t gw = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    multi_find_or_put<BS, G>(m, tm, gw, nwarps, s_new[threadIdx.x >> 5]);
+    multi_find_or_put<BS, G>(m, tm, gw, nwarps, s_new[threadIdx.x >> 5], s_pend[threadIdx.x >> 5]);
 }
 
 // One warp per exploration: level 0 is the initial state.
@@ -235,8 +193,15 @@ __global__ void __launch_bounds__(kBlock) multi_bucket_init_kernel(const MultiDe
         const uint64_t key = m.s0[e];
         const bool ok = lane == 0 && !Keys<64>::reserved(key);
         const DevTable& t = m.tables[e];
-        const uint32_t my_new = bucket_tile<64, BS, G>(t, key, 0, ok);
-        __syncwarp();
+        uint32_t st = kKeyDone;
+        bool go = ok;
+        for (uint32_t f = 0; __any_sync(kFull, go);) {      // bounded: k buckets, each claim takes a slot
+            st = bucket_pass<64, BS, G, false, false>(t.slots, key, 0, hidx(key, t.seed[f], t.nbuckets), go);
+            if (st == kKeyFull && ++f >= t.k) st = spill_put<64>(t, key, 0);
+            go = st >= kKeyLost;
+            f = __shfl_sync(kFull, f, 0);
+        }
+        const bool my_new = st == kKeyHit;
         if (lane == 0) {
             if (ok && my_new) {
                 if (m.narrow[e]) static_cast<unsigned int*>(m.states[e])[0] = static_cast<unsigned int>(key);
@@ -295,27 +260,42 @@ packed_bucket_kernel(const DevTable* __restrict__ tables, const WorkDesc* __rest
     WorkDesc d = items[r];
     uint64_t next_off = r + 1 < nitems ? items[r + 1].tile_off : ~0ull;
     unsigned long long stored = 0;
-    for (uint64_t tile = t_begin; tile < t_end; ++tile) {
-        if (tile >= next_off) {                        // into a later item
-            if (lane == 0 && stored) atomicAdd(&tables[d.table].ctr->size, stored);
-            stored = 0;
-            do {
-                ++r;
-                next_off = r + 1 < nitems ? items[r + 1].tile_off : ~0ull;
-            } while (tile >= next_off);
-            d = items[r];
+    __shared__ PendEntry s_pend[kBlock / 32][kPend];
+    Pending pend(s_pend[threadIdx.x >> 5]);
+    // Bounded: an iteration takes a tile or up to 32 queued keys of the item.
+    for (uint64_t tile = t_begin;;) {
+        const bool moves = tile >= t_end || tile >= next_off;      // done with the item's tiles
+        PendEntry p;
+        p.key = p.pos = 0;
+        p.val = p.f = 0;
+        bool mine, ok;
+        if (pend.n >= 32 || (moves && pend.n)) {
+            mine = ok = pend.pop(p);
+        } else {
+            if (moves) {
+                if (lane == 0 && stored) atomicAdd(&tables[d.table].ctr->size, stored);
+                stored = 0;
+                if (tile >= t_end) break;
+                do {
+                    ++r;
+                    next_off = r + 1 < nitems ? items[r + 1].tile_off : ~0ull;
+                } while (tile >= next_off);
+                d = items[r];
+            }
+            p.pos = (tile - d.tile_off) * 32 + lane;
+            mine = p.pos < d.n;
+            p.key = mine ? K::load(d.keys, p.pos) : 0;
+            ok = mine && !K::reserved(p.key);
+            if (mine && !ok) set_flag(tables[d.table].ctr, kFlagInvalidKey);
+            ++tile;
         }
-        const uint64_t i = (tile - d.tile_off) * 32 + lane;
-        const bool mine = i < d.n;
-        const uint64_t key = mine ? K::load(d.keys, i) : 0;
-        const bool ok = mine && !K::reserved(key);
         const DevTable& t = tables[d.table];
-        if (mine && !ok) set_flag(t.ctr, kFlagInvalidKey);
-        const uint32_t my_new = bucket_tile<KW, BS, G>(t, key, 0, ok);
-        if (mine && d.flags) d.flags[i] = uint8_t(my_new);
-        stored += __popc(__ballot_sync(kFull, my_new != 0));
+        uint32_t st = bucket_pass<KW, BS, G, false, false>(t.slots, p.key, 0, hidx(p.key, t.seed[p.f], t.nbuckets), ok);
+        bool waits;
+        st = settle_put<KW>(t, pend, st, p.key, 0, p.pos, p.f, waits);
+        if (mine && !waits && d.flags) d.flags[p.pos] = uint8_t(st);
+        stored += __popc(__ballot_sync(kFull, st == kKeyHit));
     }
-    if (lane == 0 && stored) atomicAdd(&tables[d.table].ctr->size, stored);
 }
 
 // One BFS level with successor generation and find-or-put fused (the
@@ -330,13 +310,14 @@ constexpr int kFusedStage = 512;
 template <int KW, int BS, int G>
 __global__ void __launch_bounds__(kFusedBlock, HT_BUCKET_MIN_BLOCKS * 2)
 bfs_fused_kernel(const PreparedModel* __restrict__ model, const typename Keys<KW>::T* __restrict__ frontier,
-                 uint64_t n, const DevTable t, typename Keys<KW>::T* __restrict__ out,
+                 uint64_t n, const __grid_constant__ DevTable t, typename Keys<KW>::T* __restrict__ out,
                  unsigned long long* __restrict__ count, uint64_t cap, unsigned long long* __restrict__ gen) {
     using K = Keys<KW>;
     using T = typename K::T;
     __shared__ PreparedModel sm;
     __shared__ uint64_t s_succ[kFusedBlock / 32][kFusedStage];
     __shared__ T s_new[kFusedBlock / 32][kStageCap];
+    __shared__ PendEntry s_pend[kFusedBlock / 32][kPend];
     {
         const uint32_t* src = reinterpret_cast<const uint32_t*>(model);
         uint32_t* dst = reinterpret_cast<uint32_t*>(&sm);
@@ -350,6 +331,22 @@ bfs_fused_kernel(const PreparedModel* __restrict__ model, const typename Keys<KW
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     const uint64_t rounds = (n + stride - 1) / stride;       // warp-uniform trip count
     unsigned long long made = 0, stored = 0;
+    Pending pend(s_pend[warp]);
+    // One pass over a tile of fresh successors, or over queued keys.
+    auto step = [&](bool queued, uint64_t key, bool ok) {
+        PendEntry d;
+        d.key = key;
+        d.f = 0;
+        if (queued) {
+            d.key = 0;
+            ok = pend.pop(d);
+        }
+        uint32_t res = bucket_pass<KW, BS, G, false, false>(t.slots, d.key, 0, hidx(d.key, t.seed[d.f], t.nbuckets), ok);
+        bool waits;
+        res = settle_put<KW>(t, pend, res, d.key, 0, 0, d.f, waits);
+        stage.push(res == kKeyHit, T(d.key), out, count, cap);
+        stored += res == kKeyHit;
+    };
     for (uint64_t r = 0; r < rounds; ++r) {
         const uint64_t i = r * stride + uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
         const bool act = i < n;
@@ -373,23 +370,27 @@ bfs_fused_kernel(const PreparedModel* __restrict__ model, const typename Keys<KW
             }
             __syncwarp();
             const uint32_t m = min(uint32_t(kFusedStage), tot - chunk);
-            for (uint32_t j0 = 0; j0 < m; j0 += 32) {
-                const bool mine = j0 + lane < m;
-                const uint64_t key = mine ? buf[j0 + lane] : 0;
-                const bool ok = mine && !K::reserved(key);
-                if (mine && !ok) set_flag(t.ctr, kFlagInvalidKey);
-                const uint32_t my_new = bucket_tile<KW, BS, G>(t, key, 0, ok);
-                stage.push(mine && my_new, T(key), out, count, cap);
-                stored += __popc(__ballot_sync(kFull, my_new != 0));
+            for (uint32_t j0 = 0; j0 < m || pend.n >= 32;) {
+                if (pend.n >= 32) {
+                    step(true, 0, false);
+                } else {
+                    const bool mine = j0 + lane < m;
+                    const uint64_t key = mine ? buf[j0 + lane] : 0;
+                    const bool ok = mine && !K::reserved(key);
+                    if (mine && !ok) set_flag(t.ctr, kFlagInvalidKey);
+                    step(false, key, ok);
+                    j0 += 32;
+                }
             }
             __syncwarp();
         }
         made += cnt;
     }
+    while (pend.n) step(true, 0, false);
     stage.flush(out, count, cap);
     for (int o = 16; o; o >>= 1) made += __shfl_down_sync(kFull, made, o);
-    if (lane == 0 && stored) atomicAdd(&t.ctr->size, stored);
     if (lane == 0 && made) atomicAdd(gen, made);
+    add_size<kFusedBlock>(t, stored);
 }
 
 // (bucket_slots, lanes) pairs that are instantiated.

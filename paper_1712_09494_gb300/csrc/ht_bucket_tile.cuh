@@ -1,6 +1,7 @@
 // Warp-cooperative bucket probe and claim of the GPUexplore-style table
-// (Section 4.2 of the paper), shared by the kernels that find-or-put tiles
-// of 32 keys: the single-table, multi-table, packed and persistent kernels.
+// (Section 4.2 of the paper), shared by the kernels that find-or-put or look
+// up tiles of 32 keys: the single-table, multi-table, packed, fused and
+// persistent kernels.
 // The protocol and its exactly-once argument are described at the top of
 // ht_bucket.cu.
 #pragma once
@@ -38,257 +39,211 @@ __device__ __forceinline__ void load_lane(const uint64_t* p, uint64_t (&w)[SPL])
     }
 }
 
-enum : int { kDone = 0, kRead = 1, kSpill = 3 };
-
-// Per-lane view of its SPL slots: which hold the key, which are free.
-template <int KW, int SPL>
-__device__ __forceinline__ void scan_lane(const uint64_t (&w)[SPL], uint64_t key, uint32_t& m, uint32_t& e) {
-    using K = Keys<KW>;
-    m = 0;
-    e = 0;
-#pragma unroll
-    for (int j = 0; j < SPL; ++j) {
-        m |= uint32_t(K::keyof(w[j]) == key) << j;
-        e |= uint32_t(K::empty(w[j])) << j;
-    }
-}
-
-// Rounds whose first bucket reads are issued together: up to 128 bytes of
-// slot words per lane in flight.
+// Rounds of a tile whose buckets are read together: up to 128 bytes of slot
+// words per lane in flight.
 template <int G, int SPL>
-struct Prefetch {
+struct Rounds {
     static constexpr int kCap = (16 / SPL) < 8 ? (16 / SPL) : 8;   // <= 128 B of words per lane
-    static constexpr int kRounds = kCap < G ? kCap : G;
+    static constexpr int kN = kCap < G ? kCap : G;
 };
 
-// The general claim loop of one round, for the rare keys whose first claim
-// lost or whose first bucket was full.  `le` is this lane's view of its free
-// slots in bucket b (no match was seen there).  Returns the group's result
-// (1 = stored) on every lane of the group.
-template <int KW, int BS, int G>
-__device__ __noinline__ uint32_t claim_slow(const DevTable t, bool active, uint64_t key, uint64_t word,
-                                            uint64_t b, uint32_t le, int sub, int gbase, int lane) {
+// What one pass over its bucket leaves of a key.
+enum : uint32_t {
+    kKeyDone = 0,     // found by find-or-put; not stored, for a lookup
+    kKeyHit = 1,      // stored by this find-or-put; found by a lookup
+    kKeyLost = 2,     // its claim lost the slot to another key: the same bucket again
+    kKeyFull = 3,     // its bucket is full of other keys: the next hash function
+};
+
+// One pass of a tile of 32 keys over one bucket each: lane l holds key l
+// (ok false on lanes without one) and the index bkt of the bucket to try, and
+// gets back that key's status.  Group g (G lanes) serves key q*(32/G)+g in
+// round q.  The buckets of all rounds (of a chunk of rounds, for many lanes
+// per key) are read up front, each round is decided from two ballots, and a
+// find-or-put's claims go out together: the lowest lane of the group that
+// sees a free slot CASes its lowest one (slot-index order).  A pass is
+// straight-line code, at most one bucket read and one CAS per key; keys it
+// leaves unsettled go to the caller's queue (Pending below), which runs them
+// 32 at a time.  They are few (a full first bucket: 1 in 25 keys over a fill
+// to load 0.8, 1 in 7 at the end), so settling them inside the tile would
+// stall 32 keys on the round trips of one or two; done that way, out of
+// line, the calls' stack traffic alone (the table descriptor copied for each)
+// was 60% of all L1 sectors, and an L2-resident replay ran at 27 G keys/s
+// (now 60 and more).
+template <int KW, int BS, int G, bool VALUES, bool LOOKUP>
+__device__ __forceinline__ uint32_t bucket_pass(uint64_t* slots, uint64_t mykey, uint32_t myval, uint64_t mybkt,
+                                                bool myok, uint32_t* found_val = nullptr) {
     using K = Keys<KW>;
     constexpr int SPL = BS / G;
-    constexpr uint32_t kGMask = (G == 32) ? 0xFFFFFFFFu : ((1u << G) - 1u);
-    int state = active ? kRead : kDone;
-    uint32_t lm = 0, f = 0, res = 0;
-    // Bounded: every pass ends the key, takes one free slot out of the
-    // group's view (<= BS per bucket) or moves to the next of k buckets;
-    // after the last one the spill path ends it.
-    while (__any_sync(kFull, state != kDone)) {
-        const uint32_t M = (__ballot_sync(kFull, state == kRead && lm != 0) >> gbase) & kGMask;
-        const uint32_t E = (__ballot_sync(kFull, state == kRead && le != 0) >> gbase) & kGMask;
-        int owner = -1;
-        if (state == kRead) {
-            if (M) {
-                state = kDone;
-            } else if (E) {
-                owner = gbase + __ffs(E) - 1;
-            } else if (++f < t.k) {
-                b = hidx(key, t.seed[f], t.nbuckets);
-                uint64_t nw[SPL];
-                load_lane<SPL>(t.slots + b * BS + sub * SPL, nw);
-                scan_lane<KW, SPL>(nw, key, lm, le);
-            } else {
-                state = kSpill;
-            }
-        }
-        uint32_t code = 0;
-        if (lane == owner) {
-            const int j = __ffs(le) - 1;
-            const uint64_t old =
-                atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + b * BS + sub * SPL + j), kEmpty, word);
-            code = old == kEmpty ? 0u : (K::keyof(old) == key ? 1u : 2u);
-            le &= ~(1u << j);
-        }
-        code = __shfl_sync(kFull, code, owner >= 0 ? owner : lane);
-        if (owner >= 0 && code != 2u) {
-            state = kDone;
-            res = code == 0u;
-        }
-        if (state == kSpill) {
-            if (sub == 0) res = place_spill<KW>(t, key, word) == 1 ? 1u : 0u;
-            state = kDone;
-        }
-    }
-    return __shfl_sync(kFull, res, gbase);
-}
-
-// find-or-put / insert.  A warp takes 32 keys; lane l hashes key l once.  In
-// round r, group g (G lanes) serves key r*(32/G)+g.  The first bucket of
-// every round is read up front (chunk_read); the rounds' first claims are
-// then decided from those reads and all their CASes issued together
-// (chunk_claim); the CAS results are read and the rare leftovers finished
-// (chunk_resolve).  Claims go in slot-index order: the lowest lane of the
-// group holding a free slot (in the group's view) CASes its lowest free
-// slot; a failed CAS marks that slot taken and claim_slow tries the next one.
-
-// State of rounds [r0, r0 + R) of one tile between its phases: the claim
-// bookkeeping (TileClaims) and, when read into registers, the first bucket
-// of each round (TileWords).
-template <int KW, int BS, int G, int R>
-struct TileClaims {
-    static constexpr int SPL = BS / G;
-    uint64_t old[R];          // first CAS result (owner lanes)
-    uint64_t owner_pack;      // 5 bits per round: claiming lane within the group
-    uint32_t le_pack;         // SPL bits per round: free slots in this lane's share
-    uint32_t claim, slow;     // per round: first claim issued / needs claim_slow
-};
-
-template <int KW, int BS, int G>
-struct TileWords {
-    static constexpr int SPL = BS / G;
-    static constexpr int PF = Prefetch<G, SPL>::kRounds;
-    uint64_t w[PF][SPL];      // first bucket of each round, this lane's share
-};
-
-// The key of lane l (`mykey`, `myok`) is served in round l / GPW by group l % GPW.
-template <int KW, int BS, int G>
-__device__ __forceinline__ void chunk_read(const DevTable& t, TileWords<KW, BS, G>& c, int r0, uint64_t mybkt,
-                                           bool myok) {
-    using C = TileWords<KW, BS, G>;
     constexpr int GPW = 32 / G;
-    const int lane = threadIdx.x & 31;
-    const int grp = lane / G, sub = lane % G;
-#pragma unroll
-    for (int q = 0; q < C::PF; ++q) {
-        const int kidx = (r0 + q) * GPW + grp;
-        const uint64_t b = __shfl_sync(kFull, mybkt, kidx);
-        if (__shfl_sync(kFull, myok, kidx)) {
-            load_lane<C::SPL>(t.slots + b * BS + sub * C::SPL, c.w[q]);
-        } else {
-#pragma unroll
-            for (int j = 0; j < C::SPL; ++j) c.w[q][j] = kEmpty;
-        }
-    }
-}
-
-// Decides rounds r0..r0+R-1 from their first buckets (fetch(q, w) supplies
-// this lane's share of round r0+q's bucket) and issues their first CASes.
-template <int KW, int BS, int G, int R, class Fetch>
-__device__ __forceinline__ void chunk_claim(const DevTable& t, TileClaims<KW, BS, G, R>& c, int r0, uint64_t mykey,
-                                            uint64_t mybkt, uint64_t myword, bool myok, Fetch&& fetch) {
-    using C = TileClaims<KW, BS, G, R>;
-    constexpr int GPW = 32 / G;
+    constexpr int PF = Rounds<G, SPL>::kN;
     constexpr uint32_t kGMask = (G == 32) ? 0xFFFFFFFFu : ((1u << G) - 1u);
-    constexpr uint32_t kLMask = (1u << C::SPL) - 1u;
+    static_assert(SPL >= 1 && SPL <= 8 && BS % G == 0 && G % PF == 0, "bucket/lane split");
     const int lane = threadIdx.x & 31;
     const int grp = lane / G, sub = lane % G, gbase = grp * G;
-    c.le_pack = c.claim = c.slow = 0;
-    c.owner_pack = 0;
-    // Decide each round from its read: found, claim, or slow path.
-#pragma unroll
-    for (int q = 0; q < R; ++q) {
-        const int kidx = (r0 + q) * GPW + grp;
-        const uint64_t key = __shfl_sync(kFull, mykey, kidx);
-        const bool ok = __shfl_sync(kFull, myok, kidx);
-        uint64_t w[C::SPL];
-        fetch(q, w);
-        uint32_t lm, le;
-        scan_lane<KW, C::SPL>(w, key, lm, le);
-        const uint32_t M = (__ballot_sync(kFull, ok && lm != 0) >> gbase) & kGMask;
-        const uint32_t E = (__ballot_sync(kFull, ok && le != 0) >> gbase) & kGMask;
-        c.le_pack |= le << (q * C::SPL);
-        if (ok && !M) {
-            if (E) {
-                c.claim |= 1u << q;
-                c.owner_pack |= uint64_t(__ffs(E) - 1) << (5 * q);
-            } else {
-                c.slow |= 1u << q;
-            }
-        }
-    }
-    // Issue every round's first CAS; the results are read in chunk_resolve.
-#pragma unroll
-    for (int q = 0; q < R; ++q) {
-        const int kidx = (r0 + q) * GPW + grp;
-        const uint64_t b = __shfl_sync(kFull, mybkt, kidx);
-        const uint64_t word = __shfl_sync(kFull, myword, kidx);
-        c.old[q] = kEmpty;
-        if (((c.claim >> q) & 1u) && sub == int((c.owner_pack >> (5 * q)) & 31u)) {
-            const int j = __ffs((c.le_pack >> (q * C::SPL)) & kLMask) - 1;
-            c.old[q] = atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + b * BS + sub * C::SPL + j),
-                                 kEmpty, word);
-            c.le_pack &= ~(1u << (q * C::SPL + j));
-        }
-    }
-}
-
-// Returns bit q set (group-uniform) when the group's key of round r0 + q was stored.
-template <int KW, int BS, int G, int R>
-__device__ __forceinline__ uint32_t chunk_resolve(const DevTable& t, TileClaims<KW, BS, G, R>& c, int r0,
-                                                  uint64_t mykey, uint64_t mybkt, uint64_t myword) {
-    using K = Keys<KW>;
-    using C = TileClaims<KW, BS, G, R>;
-    constexpr int GPW = 32 / G;
-    constexpr uint32_t kLMask = (1u << C::SPL) - 1u;
-    const int lane = threadIdx.x & 31;
-    const int grp = lane / G, sub = lane % G, gbase = grp * G;
-    uint32_t res = 0;
-#pragma unroll
-    for (int q = 0; q < R; ++q) {
-        const int kidx = (r0 + q) * GPW + grp;
-        const uint64_t key = __shfl_sync(kFull, mykey, kidx);
-        const uint32_t code = c.old[q] == kEmpty ? 0u : (K::keyof(c.old[q]) == key ? 1u : 2u);
-        const int src = gbase + int((c.owner_pack >> (5 * q)) & 31u);
-        const uint32_t v = __shfl_sync(kFull, code, src);
-        if ((c.claim >> q) & 1u) {
-            if (v == 0u) res |= 1u << q;
-            else if (v == 2u) c.slow |= 1u << q;
-        }
-    }
-    // Rare: claims that lost to another key, and full first buckets.
-    if (__any_sync(kFull, c.slow != 0)) {
-#pragma unroll 1
-        for (int q = 0; q < R; ++q) {
-            if (!__any_sync(kFull, (c.slow >> q) & 1u)) continue;
-            const int kidx = (r0 + q) * GPW + grp;
-            const uint64_t key = __shfl_sync(kFull, mykey, kidx);
-            const uint64_t word = __shfl_sync(kFull, myword, kidx);
-            const uint64_t b = __shfl_sync(kFull, mybkt, kidx);
-            const uint32_t r = claim_slow<KW, BS, G>(t, (c.slow >> q) & 1u, key, word, b,
-                                                     (c.le_pack >> (q * C::SPL)) & kLMask, sub, gbase, lane);
-            if (r) res |= 1u << q;
-        }
-    }
-    return res;
-}
-
-// Lane l's key was served by group l % GPW in round l / GPW.
-template <int G>
-__device__ __forceinline__ uint32_t my_result(uint32_t res_all) {
-    constexpr int GPW = 32 / G;
-    const int lane = threadIdx.x & 31;
-    return (__shfl_sync(kFull, res_all, (lane % GPW) * G) >> (lane / GPW)) & 1u;
-}
-
-// One warp serves one tile of up to 32 keys: lane l holds key l (myok false
-// on lanes without a valid key).  Returns 1 on the lanes whose key this call
-// stored.  Used by the multi-table BFS step and the serving kernel, which
-// pass a different table per tile.
-template <int KW, int BS, int G>
-__device__ __forceinline__ uint32_t bucket_tile(const DevTable& t, uint64_t mykey, uint32_t myval, bool myok) {
-    using K = Keys<KW>;
-    using W = TileWords<KW, BS, G>;
-    constexpr int PF = W::PF;
-    static_assert(W::SPL >= 1 && W::SPL <= 8 && BS % G == 0 && G % PF == 0 && PF * W::SPL <= 32,
-                  "bucket/lane split");
-    const uint64_t mybkt = hidx(mykey, t.seed[0], t.nbuckets);
-    const uint64_t myword = K::word(mykey, myval);
-    uint32_t res_all = 0;            // bit r: the group's key of round r was stored
+    const int mysh = (lane % GPW) * G;              // lane l's key is served by group l % GPW ...
+    const int myround = lane / GPW;                 // ... in round l / GPW
+    const uint32_t okmask = __ballot_sync(kFull, myok);
+    const uint64_t mybase = mybkt * BS;
+    uint32_t status = kKeyDone;
 #pragma unroll 1
     for (int r0 = 0; r0 < G; r0 += PF) {
-        W words;
-        TileClaims<KW, BS, G, PF> c;
-        chunk_read<KW, BS, G>(t, words, r0, mybkt, myok);
-        chunk_claim<KW, BS, G, PF>(t, c, r0, mykey, mybkt, myword, myok, [&](int q, uint64_t (&w)[W::SPL]) {
+        uint64_t at[PF], key[PF], w[PF][SPL], old[PF];
+        bool ok[PF], own[PF], full[PF];
 #pragma unroll
-            for (int j = 0; j < W::SPL; ++j) w[j] = words.w[q][j];
-        });
-        res_all |= chunk_resolve<KW, BS, G, PF>(t, c, r0, mykey, mybkt, myword) << r0;
+        for (int q = 0; q < PF; ++q) {
+            const int kidx = (r0 + q) * GPW + grp;
+            at[q] = __shfl_sync(kFull, mybase, kidx) + uint32_t(sub * SPL);
+            ok[q] = (okmask >> kidx) & 1u;
+            if (ok[q]) {
+                load_lane<SPL>(slots + at[q], w[q]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < SPL; ++j) w[q][j] = 0;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < PF; ++q) {
+            const int kidx = (r0 + q) * GPW + grp;
+            key[q] = KW == 32 ? uint64_t(__shfl_sync(kFull, uint32_t(mykey), kidx)) : __shfl_sync(kFull, mykey, kidx);
+            bool hit = false;
+            uint32_t e = 0, v = 0;                  // e: free slots, the lane's first one in the highest bit set
+#pragma unroll
+            for (int j = 0; j < SPL; ++j) {
+                if constexpr (KW == 32) {
+                    const bool same = uint32_t(w[q][j]) == uint32_t(key[q]);
+                    hit |= same;
+                    if (LOOKUP && VALUES && same) v = K::value(w[q][j]);
+                    e = (e << 1) | uint32_t(uint32_t(w[q][j]) == 0xFFFFFFFFu);
+                } else {
+                    // Only EMPTY has the top bit set (keys reserve it).
+                    hit |= w[q][j] == key[q];
+                    e = __funnelshift_l(uint32_t(w[q][j] >> 32), e, 1);
+                }
+            }
+            const uint32_t M = __ballot_sync(kFull, hit && ok[q]);
+            const uint32_t E = __ballot_sync(kFull, e != 0 && ok[q]);
+            const uint32_t gm = (M >> gbase) & kGMask, ge = (E >> gbase) & kGMask;
+            full[q] = ok[q] && !gm && !ge;
+            own[q] = !LOOKUP && ok[q] && !gm && ge && sub == __ffs(ge) - 1;
+            old[q] = 0;
+            if constexpr (!LOOKUP) {
+                const uint32_t val = VALUES ? __shfl_sync(kFull, myval, kidx) : 0u;
+                if (own[q]) {
+                    const int j = SPL - 32 + __clz(e);
+                    old[q] = atomicCAS(reinterpret_cast<unsigned long long*>(slots + at[q] + j), kEmpty,
+                                       K::word(key[q], val));
+                }
+            } else {
+                if (myround == r0 + q) status = ((M >> mysh) & kGMask) ? kKeyHit : kKeyDone;
+                if (VALUES) {
+                    const uint32_t mm = (M >> mysh) & kGMask;
+                    const uint32_t x = __shfl_sync(kFull, v, mysh + (mm ? __ffs(mm) - 1 : 0));
+                    if (myround == r0 + q) *found_val = mm ? x : 0u;
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < PF; ++q) {
+            const uint32_t F = __ballot_sync(kFull, full[q]);
+            if constexpr (LOOKUP) {
+                if (myround == r0 + q && ((F >> mysh) & 1u)) status = kKeyFull;
+            } else {
+                const bool stored = own[q] && old[q] == kEmpty;
+                const bool lost = own[q] && !stored && K::keyof(old[q]) != key[q];
+                const uint32_t S = __ballot_sync(kFull, stored);
+                const uint32_t L = __ballot_sync(kFull, lost);
+                if (myround == r0 + q)
+                    status = ((S >> mysh) & kGMask) ? kKeyHit
+                             : ((L >> mysh) & kGMask) ? kKeyLost : ((F >> mysh) & 1u) ? kKeyFull : kKeyDone;
+            }
+        }
     }
-    return my_result<G>(res_all);
+    return status;
+}
+
+// A warp's queue of unsettled keys in shared memory: kPend entries, of which
+// at most 31 wait when a tile adds up to 32.  Taken back 32 at a time, last
+// first.
+constexpr int kPend = 64;
+struct PendEntry {
+    uint64_t key;
+    uint64_t pos;      // where its answer goes
+    uint32_t val;
+    uint32_t f;        // the hash function to try next
+};
+
+struct Pending {
+    PendEntry* q;
+    uint32_t n;
+    __device__ __forceinline__ explicit Pending(PendEntry* buf) : q(buf), n(0) {}
+    __device__ __forceinline__ void push(bool pred, uint64_t key, uint32_t val, uint64_t pos, uint32_t f) {
+        const uint32_t mask = __ballot_sync(kFull, pred);
+        if (!mask) return;
+        const int lane = threadIdx.x & 31;
+        if (pred) {
+            PendEntry& e = q[n + __popc(mask & ((1u << lane) - 1))];
+            e.key = key;
+            e.pos = pos;
+            e.val = val;
+            e.f = f;
+        }
+        n += __popc(mask);
+        __syncwarp();
+    }
+    // Lane l's entry of the last min(n, 32), if there is one.
+    __device__ __forceinline__ bool pop(PendEntry& e) {
+        const uint32_t m = n < 32u ? n : 32u;
+        const uint32_t lane = threadIdx.x & 31;
+        const bool have = lane < m;
+        if (have) e = q[n - m + lane];
+        n -= m;
+        __syncwarp();
+        return have;
+    }
+};
+
+// All k buckets full: the stash and the overflow set.  Out of line: rare.
+template <int KW>
+__device__ __noinline__ uint32_t spill_put(const DevTable& t, uint64_t key, uint32_t val) {
+    return place_spill<KW>(t, key, Keys<KW>::word(key, val)) == 1 ? uint32_t(kKeyHit) : uint32_t(kKeyDone);
+}
+
+template <int KW>
+__device__ __noinline__ uint32_t spill_find(const DevTable& t, uint64_t key, uint32_t* val) {
+    uint64_t w = 0;
+    const bool found = find_spill<KW>(t, key, __ldcg(&t.ctr->stash_used), __ldcg(&t.ctr->ovf_used), &w);
+    *val = found ? Keys<KW>::value(w) : 0u;
+    return found ? uint32_t(kKeyHit) : uint32_t(kKeyDone);
+}
+
+// Settles a pass's statuses: a key past its last bucket goes to the spill,
+// one with a bucket left to the queue.  Returns the status of the keys that
+// are done; `waits` on the lanes whose key was queued.
+template <int KW>
+__device__ __forceinline__ uint32_t settle_put(const DevTable& t, Pending& pend, uint32_t st, uint64_t key,
+                                               uint32_t val, uint64_t pos, uint32_t f, bool& waits) {
+    if (st == kKeyFull) ++f;
+    if (st == kKeyFull && f >= t.k) st = spill_put<KW>(t, key, val);
+    waits = st >= kKeyLost;
+    pend.push(waits, key, val, pos, f);
+    return st;
+}
+
+// Adds every warp's count (lane 0's) to a table's size with one atomic per
+// block: the last step of a kernel, reached by all its threads.
+template <int NT>
+__device__ __forceinline__ void add_size(const DevTable& t, unsigned long long stored) {
+    __shared__ unsigned long long s_sum[NT / 32];
+    for (int o = 16; o; o >>= 1) stored += __shfl_down_sync(kFull, stored, o);
+    if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = stored;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long total = 0;
+#pragma unroll
+        for (int j = 0; j < NT / 32; ++j) total += s_sum[j];
+        if (total) atomicAdd(&t.ctr->size, total);
+    }
 }
 
 // Multi-table find-or-put of warps [gw] of [nwarps]: the step's tiles (the
@@ -300,7 +255,7 @@ __device__ __forceinline__ uint32_t bucket_tile(const DevTable& t, uint64_t myke
 // are) and its new states are appended to e's states.
 template <int BS, int G>
 __device__ void multi_find_or_put(const MultiDev& m, const multi::TileMap& tm, uint64_t gw, uint64_t nwarps,
-                                  uint64_t* stage_buf) {
+                                  uint64_t* stage_buf, PendEntry* pend_buf) {
     using K = Keys<64>;
     const uint64_t tiles = tm.total(m);
     const int lane = threadIdx.x & 31;
@@ -311,42 +266,51 @@ __device__ void multi_find_or_put(const MultiDev& m, const multi::TileMap& tm, u
     // one atomic each when the warp moves to another exploration or the stage
     // is full: the large explorations' counters are shared by many warps.
     multi::StateStage<kStageCap> stage(stage_buf);
+    Pending pend(pend_buf);
     multi::TileCursor cur;
     cur.start(m, tm, t_begin);
     uint32_t e = cur.e;
     uint64_t cnt = multi::step_count(m, e);
     unsigned long long stored = 0;
-    auto settle = [&]() {
-        stage.flush(m, e);
-        if (lane == 0 && stored) atomicAdd(&m.tables[e].ctr->size, stored);
-        stored = 0;
-    };
     // The next tile's keys are loaded while this one is claimed.  Lanes past
     // an exploration's count read unused words of its segment.
     uint64_t next_key = __ldcg(reinterpret_cast<const unsigned long long*>(m.succ + cur.key_index(m, t_begin, lane)));
-    for (uint64_t tile = t_begin; tile < t_end; ++tile) {
-        const uint64_t cur_key = next_key;
-        if (tile >= cur.b1) {                          // into a later exploration's tiles
-            settle();
-            cur.seek(m, tm, tile);
-            e = cur.e;
-            cnt = multi::step_count(m, e);
+    // Bounded: an iteration takes a tile or up to 32 queued keys, and a key is
+    // queued at most once for each slot of its k buckets.
+    for (uint64_t tile = t_begin;;) {
+        const bool moves = tile >= t_end || tile >= cur.b1;    // done with exploration e's tiles
+        PendEntry d;
+        d.key = d.pos = 0;
+        d.val = d.f = 0;
+        bool ok;
+        if (pend.n >= 32 || (moves && pend.n)) {
+            ok = pend.pop(d);
+        } else {
+            if (moves) {
+                stage.flush(m, e);
+                if (lane == 0 && stored) atomicAdd(&m.tables[e].ctr->size, stored);
+                stored = 0;
+                if (tile >= t_end) break;
+                cur.seek(m, tm, tile);
+                e = cur.e;
+                cnt = multi::step_count(m, e);
+            }
+            d.key = next_key;
+            ok = 32 * (tile - cur.b0) + lane < cnt && !K::reserved(d.key);
+            if (++tile < t_end) {
+                multi::TileCursor nx = cur;
+                nx.seek(m, tm, tile);
+                next_key = __ldcg(reinterpret_cast<const unsigned long long*>(m.succ + nx.key_index(m, tile, lane)));
+            }
+            if (!__any_sync(kFull, ok)) continue;
         }
-        const uint64_t i = 32 * (tile - cur.b0) + lane;
-        if (tile + 1 < t_end) {
-            multi::TileCursor nx = cur;
-            nx.seek(m, tm, tile + 1);
-            next_key = __ldcg(reinterpret_cast<const unsigned long long*>(m.succ + nx.key_index(m, tile + 1, lane)));
-        }
-        const bool mine = i < cnt;
-        if (!__any_sync(kFull, mine)) continue;
-        const uint64_t key = mine ? cur_key : 0;
-        const bool ok = mine && !K::reserved(key);
-        const uint32_t my_new = bucket_tile<64, BS, G>(m.tables[e], key, 0, ok);
-        stage.push(mine && my_new, key, m, e);
-        stored += __popc(__ballot_sync(kFull, my_new != 0));
+        const DevTable& t = m.tables[e];
+        uint32_t st = bucket_pass<64, BS, G, false, false>(t.slots, d.key, 0, hidx(d.key, t.seed[d.f], t.nbuckets), ok);
+        bool waits;
+        st = settle_put<64>(t, pend, st, d.key, 0, 0, d.f, waits);
+        stage.push(st == kKeyHit, d.key, m, e);
+        stored += __popc(__ballot_sync(kFull, st == kKeyHit));
     }
-    settle();
 }
 
 }  // namespace bucket

@@ -1,6 +1,7 @@
 // Kernels shared by both schemes: export, fill, frontier compaction, the
 // random-read roofline probe; plus launch sizing and event timing.
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <unordered_map>
 #include <vector>
@@ -225,6 +226,25 @@ int launch_blocks(const void* kernel, int block, size_t smem) {
     const int grid = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
     c.emplace(kernel, grid);
     return grid;
+}
+
+int launch_grid(const void* kernel, int block, uint64_t items, uint64_t per_block) {
+    const uint64_t need = items / per_block + (items % per_block != 0);
+    return int(std::min<uint64_t>(uint64_t(launch_blocks(kernel, block)), std::max<uint64_t>(need, 1)));
+}
+
+uint64_t l2_bytes() {
+    static std::atomic<int64_t> cached[64];            // 0: not asked yet, -1: unknown
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int64_t b = cached[dev].load(std::memory_order_relaxed);
+    if (!b) {
+        int v = 0;
+        cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, dev);
+        b = v > 0 ? v : -1;
+        cached[dev].store(b, std::memory_order_relaxed);
+    }
+    return b > 0 ? uint64_t(b) : 0;
 }
 
 L2Window l2_window(const void* base, size_t bytes) {

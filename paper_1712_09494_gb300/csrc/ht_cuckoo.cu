@@ -565,21 +565,6 @@ cuckoo_insert_kernel(const DevTable t, const DevScratch sc, uint32_t parity, uin
 
 }  // namespace
 
-namespace {
-// The current device's L2 size in bytes (queried once per device).
-uint64_t l2_bytes() {
-    static int cached[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    if (!cached[dev]) {
-        int v = 0;
-        cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, dev);
-        cached[dev] = v > 0 ? v : -1;
-    }
-    return cached[dev] > 0 ? uint64_t(cached[dev]) : 0;
-}
-}  // namespace
-
 cudaError_t cuckoo_probe(int kw, const DevTable& t, const DevScratch& sc, uint32_t parity,
                          const void* keys, const uint32_t* vals, uint64_t n,
                          const unsigned long long* d_n, uint64_t off, uint8_t* is_new, cudaStream_t s,

@@ -403,6 +403,7 @@ multi_persistent_kernel(const __grid_constant__ MultiDev m, uint64_t budget, uin
     __shared__ unsigned long long sh[multi::kAdvShared];
     __shared__ unsigned int s_first[multi::kExactTileExpl + 1];
     __shared__ MultiWinner s_win[kBlock / 32][CUCKOO ? kWinStage : 1];
+    __shared__ bucket::PendEntry s_pend[CUCKOO ? 1 : kBlock / 32][CUCKOO ? 1 : bucket::kPend];
     __shared__ int s_ok;
     const uint64_t gtid = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const uint64_t nthreads = uint64_t(gridDim.x) * blockDim.x;
@@ -425,7 +426,7 @@ multi_persistent_kernel(const __grid_constant__ MultiDev m, uint64_t budget, uin
             if (!grid_sync(m, &s_ok)) return;
             cuckoo_insert_winners(m, gtid, nthreads);
         } else {
-            bucket::multi_find_or_put<BS, G>(m, tm, gw, nwarps, stage);
+            bucket::multi_find_or_put<BS, G>(m, tm, gw, nwarps, stage, s_pend[threadIdx.x >> 5]);
         }
         if (!grid_sync(m, &s_ok)) return;
     }

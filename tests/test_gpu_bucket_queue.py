@@ -1,0 +1,78 @@
+"""Bucket tables almost full: most keys find their first buckets full and go
+through the kernels' queues of unsettled keys, past the last bucket into the
+stash and the overflow set, at batch sizes around the 32-key tile and the
+queue's limits.  Every answer must equal the oracle's (exact)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_1712_09494_gb300 as ht
+from gpu_util import assert_flags_per_key, assert_same_set, to_dev, to_np
+from workloads import keys as wk
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(8, 2), (8, 8), (16, 2), (16, 4), (16, 16), (32, 4), (32, 32)]
+
+
+def _batches(keys, rng):
+    """Ragged batches over the keys, each with a third of repeats (also inside the batch)."""
+    out, at = [], 0
+    sizes = [1, 31, 32, 33, 63, 64, 65, 257]
+    i = 0
+    while at < len(keys):
+        m = min(sizes[i % len(sizes)], len(keys) - at)
+        fresh = keys[at:at + m]
+        rep = keys[rng.integers(0, at + m, size=m // 3)]
+        out.append(rng.permutation(np.concatenate([fresh, rep])))
+        at += m
+        i += 1
+    return out
+
+
+@pytest.mark.parametrize("kw", [32, 64])
+@pytest.mark.parametrize("bs,lanes", SHAPES)
+@pytest.mark.parametrize("k", [1, 3, 16])
+def test_nearly_full_table_settles_every_key(kw, bs, lanes, k):
+    slots = 2048
+    n = int(slots * (1.02 if k == 1 else 0.98))        # k = 1: past the table into the spill
+    keys = wk.distinct_keys(n, kw, seed=bs * 100 + lanes + k)
+    rng = np.random.default_rng(k)
+    t = ht.HashTable(slots, "bucket", kw, dict(bucket_slots=bs, lanes_per_key=lanes, num_hashes=k, max_rebuilds=1))
+    orc = oracle.OracleTable()
+    batches = _batches(keys, rng)
+    batches.append(rng.permutation(np.concatenate([keys, keys])))      # one large batch of repeats
+    for b in batches:
+        assert_flags_per_key(b, to_np(t.find_or_put(to_dev(b))), orc.find_or_put(b))
+    q = np.concatenate([keys, wk.distinct_keys(n, kw, seed=bs * 100 + lanes + k, start=n)])
+    found, _ = t.lookup(to_dev(q))
+    assert np.array_equal(to_np(found), np.repeat(np.array([1, 0], dtype=np.uint8), n))
+    got, _ = t.export()
+    assert_same_set(to_np(got, np.uint32 if kw == 32 else np.uint64), keys)
+
+
+def test_values_of_queued_keys():
+    n = 2000
+    keys = wk.distinct_keys(n, 32, seed=4)
+    t = ht.HashTable(2048, "bucket", 32)
+    vals = np.arange(n, dtype=np.uint32) * 7 + 1
+    t.insert(to_dev(keys), to_dev(vals))
+    found, v = t.lookup(to_dev(keys))
+    assert to_np(found).all() and np.array_equal(to_np(v, np.uint32), vals)
+
+
+def test_many_nearly_full_tables_in_one_call():
+    n, tables = 250, 40                                # 256-slot tables
+    tabs = [ht.HashTable(256, "bucket", 64) for _ in range(tables)]
+    keys = [wk.distinct_keys(n, 64, seed=50 + i) for i in range(tables)]
+    for lo, hi in ((0, 100), (50, n)):
+        items, flags = [], []
+        for i in range(tables):
+            flags.append(torch.zeros(hi - lo, dtype=torch.uint8, device="cuda"))
+            items.append((i, to_dev(keys[i][lo:hi]), flags[-1]))
+        ht.ht_multi_find_or_put([t.handle for t in tabs], items)
+        for i in range(tables):
+            new = np.arange(lo, hi) >= (0 if lo == 0 else 100)
+            assert np.array_equal(to_np(flags[i]), new.astype(np.uint8))
+    assert [t.size() for t in tabs] == [n] * tables
