@@ -74,13 +74,9 @@ struct DeviceGuard {
 
 ht_status clear_table(ht_table* t, cudaStream_t s) {
     // Words per slot: 2 for 128-bit keys and long-key Cuckoo entries.
-    const uint64_t w = (t->kw == 128 || (is_long(t->kw) && t->scheme == HT_CUCKOO)) ? 2 : 1;
-    const uint64_t wo = t->kw >= 128 ? 2 : 1;    // words per overflow entry
-    HT_TRY(fill_words(t->dt.slots, t->dt.nslots * w, kEmpty, s));
-    HT_TRY(fill_words(t->dt.stash, t->dt.stash_slots, kEmpty, s));
-    HT_TRY(fill_words(t->dt.ovf, t->dt.ovf_slots * wo, kEmpty, s));
-    HT_TRY(cudaMemsetAsync(t->dt.ctr, 0, sizeof(DevCounters), s));
-    return HT_OK;
+    const uint32_t w = (t->kw == 128 || (is_long(t->kw) && t->scheme == HT_CUCKOO)) ? 2 : 1;
+    const uint32_t wo = t->kw >= 128 ? 2 : 1;    // words per overflow entry
+    return cuda_status(clear_words(t->dt, w, wo, s));
 }
 
 // Every stored key (and value) to the caller's buffers, any key width.
@@ -726,8 +722,7 @@ ht_status ht_export(ht_table* t, void* d_keys_out, uint32_t* d_values_out, uint6
 ht_status ht_clear(ht_table* t, void* stream) {
     if (!t) return HT_ERR_INVALID;
     DeviceGuard g(t->device);
-    t->sticky = HT_OK;
-    t->rebuild_exhausted = false;
+    table_forget(t);
     return clear_table(t, as_stream(stream));
 }
 
@@ -827,6 +822,10 @@ uint64_t ht::model_max_successors(const ht_model* m, uint32_t key_width) {
 
 const DevTable& ht::table_dev(const ht_table* t) { return t->dt; }
 const DevScratch& ht::table_scratch(const ht_table* t) { return t->sc; }
+void ht::table_forget(ht_table* t) {
+    t->sticky = HT_OK;
+    t->rebuild_exhausted = false;
+}
 void ht::table_release(ht_table* t, cudaStream_t s) {
     if (!t) return;
     DeviceGuard g(t->device);

@@ -58,6 +58,38 @@ __global__ void __launch_bounds__(kBlock) fill_kernel(uint64_t* __restrict__ p, 
     if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) p[n - 1] = v;
 }
 
+// Words [0, n) of p to EMPTY by threads [tid] of [nthreads], 32 bytes a store
+// (p is 32-byte aligned).
+__device__ __forceinline__ void empty_words(uint64_t* p, uint64_t n, uint64_t tid, uint64_t nthreads) {
+    for (uint64_t i = tid; i < n / 4; i += nthreads)
+        asm volatile("st.global.v4.u64 [%0], {%1, %1, %1, %1};" ::"l"(p + 4 * i), "l"(kEmpty) : "memory");
+    if (tid < (n & 3)) p[n - 1 - tid] = kEmpty;
+}
+
+__device__ __forceinline__ void empty_table(const DevTable& t, uint32_t slot_words, uint32_t ovf_words, uint64_t tid,
+                                            uint64_t nthreads) {
+    empty_words(t.slots, t.nslots * slot_words, tid, nthreads);
+    empty_words(t.ovf, uint64_t(t.ovf_slots) * ovf_words, tid, nthreads);
+    empty_words(t.stash, t.stash_slots, tid, nthreads);
+    uint64_t* c = reinterpret_cast<uint64_t*>(t.ctr);
+    for (uint64_t i = tid; i < sizeof(DevCounters) / 8; i += nthreads) c[i] = 0;
+}
+
+// A table's slots, overflow set, stash and counters in one launch (they took
+// four, 9 us of a small call's clear; now 4): bound by its launch up to a few
+// MB, then by the stores.
+__global__ void __launch_bounds__(kBlock)
+clear_kernel(const __grid_constant__ DevTable t, uint32_t slot_words, uint32_t ovf_words) {
+    empty_table(t, slot_words, ovf_words, uint64_t(blockIdx.x) * blockDim.x + threadIdx.x,
+                uint64_t(gridDim.x) * blockDim.x);
+}
+
+// The same for n tables of 8-byte slots: row y of the grid takes table y.
+__global__ void __launch_bounds__(kBlock) clear_many_kernel(const DevTable* __restrict__ tables, uint32_t n) {
+    for (uint32_t e = blockIdx.y; e < n; e += gridDim.y)
+        empty_table(tables[e], 1, 1, uint64_t(blockIdx.x) * blockDim.x + threadIdx.x, uint64_t(gridDim.x) * blockDim.x);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kBlock)
 compact_kernel(const T* __restrict__ keys, const uint8_t* __restrict__ flags, uint64_t n,
@@ -286,6 +318,20 @@ cudaError_t fill_words(uint64_t* p, uint64_t n, uint64_t v, cudaStream_t s) {
     if (!n) return cudaSuccess;
     ProfScope ps(kKClear, s);
     fill_kernel<<<launch_blocks((const void*)fill_kernel, kBlock), kBlock, 0, s>>>(p, n, v);
+    return cudaGetLastError();
+}
+
+cudaError_t clear_words(const DevTable& t, uint32_t slot_words, uint32_t ovf_words, cudaStream_t s) {
+    ProfScope ps(kKClear, s);
+    auto k = clear_kernel;
+    // At least four 32-byte stores a thread: a 512 KB table takes 16 blocks.
+    k<<<launch_grid((const void*)k, kBlock, t.nslots * slot_words, 16 * kBlock), kBlock, 0, s>>>(t, slot_words, ovf_words);
+    return cudaGetLastError();
+}
+
+cudaError_t clear_many(const DevTable* tables, uint32_t n, cudaStream_t s) {
+    ProfScope ps(kKClear, s);
+    clear_many_kernel<<<dim3(16, std::min(n, 4096u)), kBlock, 0, s>>>(tables, n);
     return cudaGetLastError();
 }
 

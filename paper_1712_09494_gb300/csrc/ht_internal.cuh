@@ -412,6 +412,10 @@ cudaError_t cuckoo_lookup(int kw, const DevTable& t, const void* keys, uint64_t 
 cudaError_t table_export(int kw, const DevTable& t, void* keys_out, uint32_t* vals_out,
                          unsigned long long* count, uint64_t cap, cudaStream_t s);
 cudaError_t fill_words(uint64_t* p, uint64_t n, uint64_t v, cudaStream_t s);
+// Empties a table (its slots and overflow entries are of 1 or 2 words), or n
+// tables of one-word slots whose descriptors are in device memory.
+cudaError_t clear_words(const DevTable& t, uint32_t slot_words, uint32_t ovf_words, cudaStream_t s);
+cudaError_t clear_many(const DevTable* tables, uint32_t n, cudaStream_t s);
 cudaError_t compact(int kw, const void* keys, const uint8_t* flags, uint64_t n, void* out,
                     unsigned long long* count, cudaStream_t s);
 cudaError_t probe_random_read(const void* buf, uint64_t bytes, uint32_t gran, uint64_t n_access,
@@ -541,6 +545,9 @@ const DevScratch& table_scratch(const ht_table* t);
 BucketCfg table_bucket_cfg(const ht_table* t);
 ht_scheme table_scheme(const ht_table* t);
 uint32_t table_key_width(const ht_table* t);
+// ht_clear's host side: the table forgets a full or exhausted state (its
+// device words are emptied by the caller).
+void table_forget(ht_table* t);
 // Frees an idle table's memory in the order of stream s, without a device
 // synchronisation (the caller guarantees no work on the table is pending).
 void table_release(ht_table* t, cudaStream_t s);

@@ -152,12 +152,12 @@ ht_status step_launches(ht_multi* m) {
 }
 
 ht_status reset_multi(ht_multi* m) {
-    for (ht_table* t : m->tables) {
-        ht_status st = ht_clear(t, m->stream);
-        if (st != HT_OK) return st;
-    }
+    // All of a group's tables in one launch: one ht_clear each took 4.6 of
+    // 256 explorations' 50 ms.
+    for (ht_table* t : m->tables) table_forget(t);
     for (auto& g : m->groups) {
         const uint64_t n = g.members.size();
+        if (clear_many(g.dev.tables, uint32_t(n), m->stream) != cudaSuccess) return HT_ERR_CUDA;
         // Zero every counter array (they sit contiguously at the arena's start).
         const char* first = reinterpret_cast<const char*>(g.dev.total);
         const char* last = reinterpret_cast<const char*>(g.dev.steps) + 256;
