@@ -11,10 +11,11 @@
 // next bucket; after the last one the key goes to the stash.
 //
 // Exactly-once: a slot never returns to empty and never changes its key, and
-// every group claims in the same slot order.  A group that claims slot s saw
-// every earlier slot (by load or by a failed CAS) holding another key, so a
-// concurrent group with the same key either meets the claimed word first or
-// finds the bucket full only after the word was written there.  A key goes
+// all groups with one key claim in the same order of the slots (from a place
+// that the key gives, around the bucket).  A group that claims slot s saw
+// every slot before it in that order holding another key, so a concurrent
+// group with the same key either meets the claimed word first or finds the
+// bucket full only after the word was written there.  A key goes
 // to bucket f+1 only after bucket f was observed full without it, and
 // fullness is permanent, so lookups may stop at the first non-full bucket.
 #include <algorithm>

@@ -55,13 +55,32 @@ enum : uint32_t {
     kKeyFull = 3,     // its bucket is full of other keys: the next hash function
 };
 
+// Where a key's claims start in a bucket's slots: claims go from there on,
+// around the bucket.  Any order does that is the same for all copies of a key
+// (the argument in ht_bucket.cu).  When every key starts at slot 0, the keys of
+// a small table's batch that share a bucket all claim the same slot and all but
+// one lose and try again: 16,384 new keys into 62,500 slots took 22 us, of which
+// a batch of stored keys takes 4.
+template <int BS>
+__device__ __forceinline__ uint32_t claim_rot(uint64_t key) {
+    return ((uint32_t(key) ^ uint32_t(key >> 32)) * 0x9E3779B1u >> 16) % uint32_t(BS);
+}
+
+// The first bit set of an N-bit mask (N a power of two) from bit `from` on,
+// around its end.
+template <int N>
+__device__ __forceinline__ uint32_t first_from(uint32_t mask, uint32_t from) {
+    const uint32_t up = mask >> from;
+    return up ? from + __ffs(up) - 1 : __ffs(mask) - 1;
+}
+
 // One pass of a tile of 32 keys over one bucket each: lane l holds key l
 // (ok false on lanes without one) and the index bkt of the bucket to try, and
 // gets back that key's status.  Group g (G lanes) serves key q*(32/G)+g in
 // round q.  The buckets of all rounds (of a chunk of rounds, for many lanes
 // per key) are read up front, each round is decided from two ballots, and a
-// find-or-put's claims go out together: the lowest lane of the group that
-// sees a free slot CASes its lowest one (slot-index order).  A pass is
+// find-or-put's claims go out together: the lane of the group that sees the
+// first free slot in the key's order CASes it.  A pass is
 // straight-line code, at most one bucket read and one CAS per key; keys it
 // leaves unsettled go to the caller's queue (Pending below), which runs them
 // 32 at a time.  They are few (a full first bucket: 1 in 25 keys over a fill
@@ -107,7 +126,7 @@ __device__ __forceinline__ uint32_t bucket_pass(uint64_t* slots, uint64_t mykey,
             const int kidx = (r0 + q) * GPW + grp;
             key[q] = KW == 32 ? uint64_t(__shfl_sync(kFull, uint32_t(mykey), kidx)) : __shfl_sync(kFull, mykey, kidx);
             bool hit = false;
-            uint32_t e = 0, v = 0;                  // e: free slots, the lane's first one in the highest bit set
+            uint32_t e = 0, v = 0;                  // e: free slots, slot j of the lane's share in bit SPL - 1 - j
 #pragma unroll
             for (int j = 0; j < SPL; ++j) {
                 if constexpr (KW == 32) {
@@ -125,12 +144,13 @@ __device__ __forceinline__ uint32_t bucket_pass(uint64_t* slots, uint64_t mykey,
             const uint32_t E = __ballot_sync(kFull, e != 0 && ok[q]);
             const uint32_t gm = (M >> gbase) & kGMask, ge = (E >> gbase) & kGMask;
             full[q] = ok[q] && !gm && !ge;
-            own[q] = !LOOKUP && ok[q] && !gm && ge && sub == __ffs(ge) - 1;
             old[q] = 0;
             if constexpr (!LOOKUP) {
+                const uint32_t rot = claim_rot<BS>(key[q]);
+                own[q] = ok[q] && !gm && ge && uint32_t(sub) == first_from<G>(ge, rot / SPL);
                 const uint32_t val = VALUES ? __shfl_sync(kFull, myval, kidx) : 0u;
                 if (own[q]) {
-                    const int j = SPL - 32 + __clz(e);
+                    const uint32_t j = SPL - 1 - first_from<SPL>(e, rot % SPL);
                     old[q] = atomicCAS(reinterpret_cast<unsigned long long*>(slots + at[q] + j), kEmpty,
                                        K::word(key[q], val));
                 }

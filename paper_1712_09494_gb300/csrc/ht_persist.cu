@@ -85,8 +85,8 @@ __device__ bool grid_sync(const MultiDev& m, int* s_ok) {
 }
 
 // Level 0 of every exploration: its initial state placed in its (empty)
-// table -- bucket scheme: the first slot of bucket h_1, the lowest free slot
-// of the claim order; Cuckoo: slot h_1 -- and stored as the first state.
+// table -- bucket scheme: the first slot of bucket h_1 (nothing else claims
+// yet, so any free slot does); Cuckoo: slot h_1 -- and stored as the first state.
 // Tables are addressed as 64-bit key tables (a 32-bit set table's words are
 // the same), states are written in their exploration's width.
 template <bool CUCKOO, int BS>
