@@ -44,12 +44,21 @@ def _check(status, where):
         raise HtError(status, where)
 
 
+# Pointers and streams go to ctypes as plain integers (its argtypes convert
+# them), and the current stream comes from torch's raw accessor: a small call
+# is bound by the host, and building a Stream object and c_void_p's for each
+# took 4 of its 9 us.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) if hasattr(torch._C, "_cuda_getDevice") else None
+
+
 def _stream(stream):
     if stream is None:
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        if _raw_stream is None or not torch.cuda.is_initialized():
+            return torch.cuda.current_stream().cuda_stream
+        return _raw_stream(torch._C._cuda_getDevice())
     if isinstance(stream, torch.cuda.Stream):
-        return ctypes.c_void_p(stream.cuda_stream)
-    return ctypes.c_void_p(int(stream))
+        return stream.cuda_stream
+    return int(stream)
 
 
 def _dptr(t, what):
@@ -59,7 +68,7 @@ def _dptr(t, what):
         raise ValueError("%s must be a CUDA tensor" % what)
     if not t.is_contiguous():
         raise ValueError("%s must be contiguous" % what)
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _key_width(keys):
@@ -174,14 +183,16 @@ def ht_multi_find_or_put(tables, items, stream=None):
     import numpy as np
     n = len(tables)
     arr_t = (ctypes.c_void_p * max(1, n))(*[getattr(t, "value", t) for t in tables])
-    w = np.zeros(max(1, len(items)), dtype=_WORK_DTYPE)
+    rows = []
     for i, (ti, keys, is_new) in enumerate(items):
         if not (keys.is_cuda and keys.is_contiguous()):
             raise ValueError("keys of item %d must be a contiguous CUDA tensor" % i)
         if is_new is not None and not (is_new.is_cuda and is_new.is_contiguous()):
             raise ValueError("is_new of item %d must be a contiguous CUDA tensor" % i)
-        w[i] = (ti, 0, keys.data_ptr() if keys.numel() else 0, keys.numel(),
-                is_new.data_ptr() if is_new is not None and is_new.numel() else 0)
+        m = keys.numel()
+        rows.append((ti, 0, keys.data_ptr() if m else 0, m,
+                     is_new.data_ptr() if is_new is not None and is_new.numel() else 0))
+    w = np.array(rows, dtype=_WORK_DTYPE) if rows else np.zeros(1, dtype=_WORK_DTYPE)
     _check(load().ht_multi_find_or_put(arr_t, n, w.ctypes.data_as(ctypes.c_void_p), len(items), _stream(stream)),
            "ht_multi_find_or_put")
 
@@ -325,7 +336,7 @@ def ht_bfs(table, model, s0=0, max_levels=4096, states=None, states_cap=0, strea
     name = "ht_bfs_fused" if fused else "ht_bfs"
     _check(getattr(load(), name)(table, ctypes.byref(model), int(s0), int(max_levels), sizes,
                                  _dptr(states, "states"), cap, ctypes.byref(res), _stream(stream)), name)
-    return res, [int(sizes[i]) for i in range(res.levels)]
+    return res, sizes[:res.levels]
 
 
 class MultiExploration:
@@ -381,7 +392,7 @@ class MultiExploration:
         _check(load().ht_multi_result(self._h, int(i), ctypes.byref(lv), ctypes.byref(st), ctypes.byref(gen),
                                       ctypes.byref(comp), sizes, ctypes.byref(ptr), None, 0), "ht_multi_result")
         out = dict(levels=lv.value, states=st.value, successors=gen.value, complete=comp.value,
-                   level_sizes=[int(sizes[j]) for j in range(lv.value)], states_ptr=ptr.value)
+                   level_sizes=sizes[:lv.value], states_ptr=ptr.value)
         if with_states:
             arr = np.empty(st.value, dtype=np.uint32 if key_width == 32 else np.uint64)
             _check(load().ht_multi_result(self._h, int(i), None, None, None, None, None, None,
@@ -497,25 +508,29 @@ class HashTable:
             pass
 
     def _keys(self, keys):
-        if _key_width(keys) != self.key_width:
+        """The keys as a contiguous tensor, and how many there are."""
+        kw = _key_width(keys)
+        if kw != self.key_width:
             raise ValueError("table has %d-bit keys" % self.key_width)
-        return keys.contiguous()
+        return keys.contiguous(), (keys.shape[0] if kw >= 128 else keys.numel())
 
     def find_or_put(self, keys, stream=None):
-        keys = self._keys(keys)
-        is_new = torch.empty(_nkeys(keys), dtype=torch.uint8, device=keys.device)
-        ht_find_or_put(self._h, keys, is_new, stream)
+        keys, n = self._keys(keys)
+        is_new = keys.new_empty(n, dtype=torch.uint8)
+        _check(load().ht_find_or_put(self._h, _dptr(keys, "keys"), n, is_new.data_ptr() if n else None,
+                                     _stream(stream)), "ht_find_or_put")
         return is_new
 
     def insert(self, keys, values=None, stream=None):
-        keys = self._keys(keys)
+        keys, _ = self._keys(keys)
         ht_insert(self._h, keys, None if values is None else values.contiguous(), stream)
 
     def lookup(self, keys, stream=None):
-        keys = self._keys(keys)
-        found = torch.empty(_nkeys(keys), dtype=torch.uint8, device=keys.device)
-        values = torch.empty(keys.numel(), dtype=torch.int32, device=keys.device) if self.key_width == 32 else None
-        ht_lookup(self._h, keys, values, found, stream)
+        keys, n = self._keys(keys)
+        found = keys.new_empty(n, dtype=torch.uint8)
+        values = keys.new_empty(n, dtype=torch.int32) if self.key_width == 32 else None
+        _check(load().ht_lookup(self._h, _dptr(keys, "keys"), n, values.data_ptr() if values is not None else None,
+                                found.data_ptr(), _stream(stream)), "ht_lookup")
         return found, values
 
     def sync(self, stream=None):
