@@ -16,7 +16,7 @@
 // go in slot order over the candidates (the slot-order argument of the
 // 64-bit kernels: a key is claimed in at most one slot), and only the CAS
 // result decides, so stale or torn reads cannot duplicate a key.
-#include "ht_internal.cuh"
+#include "ht_bucket_tile.cuh"
 
 namespace ht {
 namespace {
@@ -71,130 +71,239 @@ __device__ bool wide_ovf_find(const DevTable& t, uint64_t lo, uint64_t hi) {
     return false;
 }
 
-// find-or-put: a warp takes 32 keys (lane l loads key l); in round q group
-// g (G lanes) serves key q*(32/G)+g through buckets h_1, h_2, ... until the
-// key is found, claimed, or (all k buckets full) placed in the overflow set.
-// APPEND: the keys new to the table also go to new_out at *new_count
-// (staged per warp in shared memory; entries past new_cap not written).
-// d_n (nullable): the batch size produced on the device, at most n.
-template <int G, bool LOOKUP, bool APPEND>
-__global__ void __launch_bounds__(kBlock)
-wide_kernel(const DevTable t, const ulonglong2* __restrict__ keys, uint64_t n,
-            const unsigned long long* __restrict__ d_n, uint8_t* __restrict__ out,
-            ulonglong2* __restrict__ new_out, unsigned long long* __restrict__ new_count, uint64_t new_cap) {
+// A warp's queue of keys whose bucket was full, as the 64-bit kernels' Pending:
+// at most 31 wait when a tile adds up to 32; taken back 32 at a time.
+constexpr int kWidePend = 64;
+struct WideEntry {
+    ulonglong2 key;
+    uint64_t pos;      // where its answer goes
+    uint32_t f;        // the hash function to try next
+    uint32_t pad_;
+};
+
+// All k buckets full: the overflow set.  Out of line: rare.  Returns 1 when
+// the key was stored there.
+__device__ __noinline__ uint32_t wide_spill_put(const DevTable& t, uint64_t lo, uint64_t hi) {
+    const int r = wide_ovf_insert(t, lo, hi);
+    if (r == 1) atomicAdd(&t.ctr->ovf_used, 1u);
+    if (r < 0) {
+        set_flag(t.ctr, kFlagDropped);
+        atomicAdd(&t.ctr->dropped, 1ull);
+    }
+    return r == 1;
+}
+
+__device__ __noinline__ uint32_t wide_spill_find(const DevTable& t, uint64_t lo, uint64_t hi) {
+    return wide_ovf_find(t, lo, hi);
+}
+
+// One pass of a tile of 32 keys over one bucket each (lane l holds key l and
+// its bucket's index; ok false without one): 0 found (lookup: absent), 1 stored
+// (lookup: found), 2 its bucket is full of other keys.  Group g (G lanes)
+// serves key q*(32/G)+g in round q; all rounds' buckets are read up front with
+// 256-bit loads and the first claims go out together.  A claim that another
+// key's won is followed by the next candidate slot's at once: a stored key
+// whose low word is all ones always reads as a candidate, so reading the bucket
+// again would not get past it.
+template <int G, bool LOOKUP>
+__device__ __forceinline__ uint32_t wide_pass(uint64_t* slots, ulonglong2 mykey, uint64_t mybkt, bool myok) {
     constexpr int SPL = kWideBS / G;
     constexpr int GPW = 32 / G;
     constexpr uint32_t kGMask = (1u << G) - 1u;
-    if (d_n) n = min(n, uint64_t(__ldcg(d_n)));
+    constexpr int PF = G < 4 ? G : 2;               // 16 words of buckets in flight per lane
     const int lane = threadIdx.x & 31;
     const int grp = lane / G, sub = lane % G, gbase = grp * G;
-    const uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
-    unsigned long long stored = 0;
-    __shared__ ulonglong2 s_new[APPEND ? kBlock / 32 : 1][APPEND ? kStageCap : 1];
-    WarpStage<ulonglong2, kStageCap> stage(s_new[APPEND ? (threadIdx.x >> 5) : 0]);
-    for (uint64_t base = ((uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * 32; base < n;
-         base += nwarps * 32) {
-        const bool mine = base + lane < n;
-        ulonglong2 mk = make_ulonglong2(0, 0);
-        if (mine) mk = keys[base + lane];
-        const bool myok = mine && !wide_reserved(mk.y);
-        if (mine && !myok) set_flag(t.ctr, kFlagInvalidKey);
-        uint32_t res_all = 0;                       // bit q: the group's key of round q was stored / found
-        for (int q = 0; q < G; ++q) {
-            const int kidx = q * GPW + grp;
-            const uint64_t lo = __shfl_sync(kFull, mk.x, kidx);
-            const uint64_t hi = __shfl_sync(kFull, mk.y, kidx);
-            const bool ok = __shfl_sync(kFull, myok, kidx);
-            const uint64_t fold = wide_fold(lo, hi);
-            uint32_t f = 0;
-            uint64_t b = hidx(fold, t.seed[0], t.nbuckets);
-            int state = ok ? 0 : 3;                 // 0 read, 1 decide, 2 spill, 3 done
-            uint32_t cand = 0, match = 0, res = 0;
-            // Bounded: each pass ends the key, spends a candidate slot of
-            // this bucket (<= 8) or moves to the next of k buckets.
-            while (__any_sync(kFull, state != 3)) {
-                if (state == 0) {
-                    cand = match = 0;
+    const int mysh = (lane % GPW) * G, myround = lane / GPW;
+    const uint32_t okmask = __ballot_sync(kFull, myok);
+    uint32_t status = 0;
+#pragma unroll 1
+    for (int r0 = 0; r0 < G; r0 += PF) {
+        uint64_t at[PF], lo[PF], hi[PF], w[PF][2 * SPL];
+        ulonglong2 old[PF];
+        uint32_t cand[PF], rot[PF];
+        int claim[PF];                              // the slot of the lane's share it claims (-1: none)
+        bool ok[PF], done[PF], stored[PF];
 #pragma unroll
-                    for (int j = 0; j < SPL; ++j) {
-                        const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(
-                            t.slots + 2 * (b * kWideBS + uint64_t(sub * SPL + j))));
-                        if (LOOKUP) {
-                            // No writer runs beside a lookup: reads are
-                            // complete, and only all ones is empty.
-                            if (v.x == lo && v.y == hi) match |= 1u << j;
-                            else if (v.x == kOnes && v.y == kOnes) cand |= 1u << j;
-                        } else if (slot_class(v.x, v.y) == 2) {
-                            if (v.x == lo && v.y == hi) match |= 1u << j;
-                        } else {
-                            cand |= 1u << j;
-                        }
-                    }
-                    state = 1;
-                }
-                const uint32_t M = (__ballot_sync(kFull, state == 1 && match != 0) >> gbase) & kGMask;
-                const uint32_t C = (__ballot_sync(kFull, state == 1 && cand != 0) >> gbase) & kGMask;
-                int owner = -1;
-                if (state == 1) {
-                    if (M) {
-                        state = 3;
-                        res = LOOKUP ? 1u : 0u;
-                    } else if (C) {
-                        if (LOOKUP) {
-                            // An empty slot: a key moves on to its next
-                            // bucket only from a full one, so it is absent.
-                            state = 3;
-                            res = 0;
-                        } else {
-                            owner = gbase + __ffs(C) - 1;
-                        }
-                    } else if (++f < t.k) {
-                        b = hidx(fold, t.seed[f], t.nbuckets);
-                        state = 0;
-                    } else {
-                        state = 2;
-                    }
-                }
-                uint32_t code = 0;
-                if (!LOOKUP && lane == owner) {
-                    const int j = __ffs(cand) - 1;
-                    uint64_t ol, oh;
-                    cas128(t.slots + 2 * (b * kWideBS + uint64_t(sub * SPL + j)), lo, hi, ol, oh);
-                    code = (ol == kOnes && oh == kOnes) ? 0u : ((ol == lo && oh == hi) ? 1u : 2u);
-                    cand &= ~(1u << j);
-                }
-                code = __shfl_sync(kFull, code, owner >= 0 ? owner : lane);
-                if (owner >= 0 && code != 2u) {
-                    state = 3;
-                    res = code == 0u;
-                }
-                if (state == 2) {
-                    if (sub == 0) {
-                        if (LOOKUP) {
-                            res = wide_ovf_find(t, lo, hi) ? 1u : 0u;
-                        } else {
-                            const int r = wide_ovf_insert(t, lo, hi);
-                            res = r == 1;
-                            if (r == 1) atomicAdd(&t.ctr->ovf_used, 1u);
-                            if (r < 0) {
-                                set_flag(t.ctr, kFlagDropped);
-                                atomicAdd(&t.ctr->dropped, 1ull);
-                            }
-                        }
-                    }
-                    state = 3;
-                }
+        for (int q = 0; q < PF; ++q) {
+            const int kidx = (r0 + q) * GPW + grp;
+            at[q] = 2 * (__shfl_sync(kFull, mybkt, kidx) * kWideBS + uint32_t(sub * SPL));
+            ok[q] = (okmask >> kidx) & 1u;
+#pragma unroll
+            for (int j = 0; j < 2 * SPL; j += 4) {
+                unsigned long long a = 0, b = 0, c = 0, d = 0;
+                if (ok[q])
+                    asm volatile("ld.global.cg.v4.u64 {%0,%1,%2,%3}, [%4];"
+                                 : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(slots + at[q] + j));
+                w[q][j] = a;
+                w[q][j + 1] = b;
+                w[q][j + 2] = c;
+                w[q][j + 3] = d;
             }
-            res = __shfl_sync(kFull, res, gbase);
-            res_all |= res << q;
         }
-        const uint32_t my = (__shfl_sync(kFull, res_all, (lane % GPW) * G) >> (lane / GPW)) & 1u;
-        if (mine && out) out[base + lane] = uint8_t(my);
-        if (APPEND) stage.push(mine && my, mk, new_out, new_count, new_cap);
-        if (!LOOKUP) stored += __popc(__ballot_sync(kFull, my != 0));
+        bool more = false;
+#pragma unroll
+        for (int q = 0; q < PF; ++q) {
+            const int kidx = (r0 + q) * GPW + grp;
+            lo[q] = __shfl_sync(kFull, mykey.x, kidx);
+            hi[q] = __shfl_sync(kFull, mykey.y, kidx);
+            bool hit = false;
+            uint32_t e = 0;
+#pragma unroll
+            for (int j = 0; j < SPL; ++j) {
+                const uint64_t x = w[q][2 * j], y = w[q][2 * j + 1];
+                // The top bit of a complete high word is 0.  A lookup runs with
+                // no writer: its reads are complete and only EMPTY sets it.
+                const bool part = LOOKUP ? (y >> 63) != 0 : ((y >> 63) != 0 || x == kOnes);
+                hit |= x == lo[q] && y == hi[q] && (LOOKUP || !part);
+                e |= uint32_t(part) << j;
+            }
+            const uint32_t M = __ballot_sync(kFull, hit && ok[q]);
+            const uint32_t gm = (M >> gbase) & kGMask;
+            cand[q] = ok[q] && !gm ? e : 0u;
+            done[q] = !ok[q] || gm != 0;
+            stored[q] = false;
+            claim[q] = -1;
+            if constexpr (LOOKUP) {
+                const uint32_t ge = (__ballot_sync(kFull, cand[q] != 0) >> gbase) & kGMask;
+                done[q] |= ge != 0;                 // a key moves on only from a full bucket
+                if (myround == r0 + q && ((M >> mysh) & kGMask)) status = 1;
+            } else {
+                rot[q] = bucket::claim_rot<kWideBS>(lo[q] ^ hi[q]);
+                const uint32_t ge = (__ballot_sync(kFull, cand[q] != 0) >> gbase) & kGMask;
+                if (cand[q] && uint32_t(sub) == bucket::first_from<G>(ge, rot[q] / SPL)) {
+                    claim[q] = int(bucket::first_from<SPL>(cand[q], rot[q] % SPL));
+                    uint64_t ol, oh;
+                    cas128(slots + at[q] + 2 * claim[q], lo[q], hi[q], ol, oh);
+                    old[q] = make_ulonglong2(ol, oh);
+                }
+                more |= ge != 0;
+            }
+        }
+        // Bounded: every pass of the loop ends the key of each claim made or
+        // spends its candidate slot.
+        while (!LOOKUP && __any_sync(kFull, more)) {
+            more = false;
+#pragma unroll
+            for (int q = 0; q < PF; ++q) {
+                bool won = false, same = false;
+                if (claim[q] >= 0) {
+                    won = old[q].x == kOnes && old[q].y == kOnes;
+                    same = old[q].x == lo[q] && old[q].y == hi[q];
+                    cand[q] &= ~(1u << claim[q]);
+                    claim[q] = -1;
+                }
+                const uint32_t W = __ballot_sync(kFull, won), S = __ballot_sync(kFull, same);
+                if ((W >> gbase) & kGMask) stored[q] = done[q] = true;
+                if ((S >> gbase) & kGMask) done[q] = true;
+                if (done[q]) cand[q] = 0;
+                const uint32_t ge = (__ballot_sync(kFull, cand[q] != 0) >> gbase) & kGMask;
+                if (cand[q] && uint32_t(sub) == bucket::first_from<G>(ge, rot[q] / SPL)) {
+                    claim[q] = int(bucket::first_from<SPL>(cand[q], rot[q] % SPL));
+                    uint64_t ol, oh;
+                    cas128(slots + at[q] + 2 * claim[q], lo[q], hi[q], ol, oh);
+                    old[q] = make_ulonglong2(ol, oh);
+                }
+                more |= ge != 0;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < PF; ++q) {
+            const uint32_t D = __ballot_sync(kFull, !done[q]), S = __ballot_sync(kFull, stored[q]);
+            if (myround == r0 + q) {
+                if ((D >> mysh) & 1u) status = 2;
+                else if (!LOOKUP) status = (S >> mysh) & 1u;
+            }
+        }
+    }
+    return status;
+}
+
+// find-or-put or lookup: a warp takes a fresh tile of 32 keys, or 32 queued
+// ones, for one pass over one bucket each, as the 64-bit kernel does
+// (bucket_tiles in ht_bucket.cu).  Bound by random 128-byte lines.
+// APPEND: the keys new to the table also go to new_out at *new_count
+// (staged per warp in shared memory; entries past new_cap not written).
+// d_n (nullable): the batch size produced on the device, at most n.
+// ahead: a lookup in a table larger than L2 touches the next tile's buckets.
+#ifndef HT_WIDE_MIN_BLOCKS
+#define HT_WIDE_MIN_BLOCKS 3
+#endif
+template <int G, bool LOOKUP, bool APPEND>
+__global__ void __launch_bounds__(kBlock, HT_WIDE_MIN_BLOCKS)
+wide_kernel(const __grid_constant__ DevTable t, const ulonglong2* __restrict__ keys, uint64_t n,
+            const unsigned long long* __restrict__ d_n, uint8_t* __restrict__ out,
+            ulonglong2* __restrict__ new_out, unsigned long long* __restrict__ new_count, uint64_t new_cap, bool ahead) {
+    if (d_n) n = min(n, uint64_t(__ldcg(d_n)));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
+    unsigned long long stored = 0;
+    constexpr int kStage = kStageCap / 2;              // with the queues, under 48 KB a block
+    __shared__ ulonglong2 s_new[APPEND ? kBlock / 32 : 1][APPEND ? kStage : 1];
+    __shared__ WideEntry s_pend[kBlock / 32][kWidePend];
+    WideEntry* pend = s_pend[warp];
+    uint32_t waiting = 0;
+    WarpStage<ulonglong2, kStage> stage(s_new[APPEND ? warp : 0]);
+    uint64_t base = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) / 32 * 32;
+    ulonglong2 key0 = make_ulonglong2(0, 0), key1 = key0;
+    if (base + lane < n) key0 = keys[base + lane];
+    if (base + step + lane < n) key1 = keys[base + step + lane];
+    // Bounded: an iteration takes a tile or up to 32 queued keys, and a key is
+    // queued at most once for each of its k buckets.
+    for (;;) {
+        ulonglong2 key = make_ulonglong2(0, 0);
+        uint64_t pos = 0;
+        uint32_t f = 0;
+        bool mine, ok;
+        if (waiting >= 32 || (base >= n && waiting)) {
+            const uint32_t m = min(waiting, 32u);
+            mine = ok = uint32_t(lane) < m;
+            if (ok) {
+                const WideEntry e = pend[waiting - m + lane];
+                key = e.key;
+                pos = e.pos;
+                f = e.f;
+            }
+            waiting -= m;
+            __syncwarp();
+        } else if (base < n) {
+            key = key0;
+            pos = base + lane;
+            mine = pos < n;
+            ok = mine && !wide_reserved(key.y);
+            if (mine && !ok) set_flag(t.ctr, kFlagInvalidKey);
+            key0 = key1;
+            if (LOOKUP && ahead && base + step + lane < n)
+                touch_l2(t.slots + 2 * kWideBS * hidx(wide_fold(key0.x, key0.y), t.seed[0], t.nbuckets));
+            if (base + 2 * step + lane < n) key1 = keys[base + 2 * step + lane];
+            base += step;
+        } else {
+            break;
+        }
+        const uint64_t fold = wide_fold(key.x, key.y);
+        uint32_t st = wide_pass<G, LOOKUP>(t.slots, key, hidx(fold, t.seed[f], t.nbuckets), ok);
+        bool waits = st == 2;
+        if (waits && ++f >= t.k) {
+            st = LOOKUP ? wide_spill_find(t, key.x, key.y) : wide_spill_put(t, key.x, key.y);
+            waits = false;
+        }
+        const uint32_t wm = __ballot_sync(kFull, waits);
+        if (wm) {
+            if (waits) {
+                WideEntry& e = pend[waiting + __popc(wm & ((1u << lane) - 1))];
+                e.key = key;
+                e.pos = pos;
+                e.f = f;
+                if (LOOKUP && ahead) touch_l2(t.slots + 2 * kWideBS * hidx(fold, t.seed[f], t.nbuckets));
+            }
+            waiting += __popc(wm);
+            __syncwarp();
+        }
+        if (mine && !waits && out) out[pos] = uint8_t(st);
+        if (APPEND) stage.push(st == 1, key, new_out, new_count, new_cap);
+        if (!LOOKUP) stored += st == 1;
     }
     if (APPEND) stage.flush(new_out, new_count, new_cap);
-    if (!LOOKUP && lane == 0 && stored) atomicAdd(&t.ctr->size, stored);
+    if (!LOOKUP) bucket::add_size<kBlock>(t, stored);
 }
 
 // Every stored key (table, then overflow set) to out[2 * i .. 2 * i + 1].
@@ -588,8 +697,9 @@ cudaError_t launch_wide(const DevTable& t, const void* keys, uint64_t n, const u
                         uint8_t* out, void* new_out, unsigned long long* new_count, uint64_t new_cap,
                         cudaStream_t s) {
     auto k = wide_kernel<G, LOOKUP, APPEND>;
-    k<<<launch_blocks((const void*)k, kBlock), kBlock, 0, s>>>(t, static_cast<const ulonglong2*>(keys), n, d_n, out,
-                                                              static_cast<ulonglong2*>(new_out), new_count, new_cap);
+    k<<<launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s>>>(
+        t, static_cast<const ulonglong2*>(keys), n, d_n, out, static_cast<ulonglong2*>(new_out), new_count, new_cap,
+        t.nslots * 16 > l2_bytes());
     return cudaGetLastError();
 }
 

@@ -76,3 +76,22 @@ def test_many_nearly_full_tables_in_one_call():
             new = np.arange(lo, hi) >= (0 if lo == 0 else 100)
             assert np.array_equal(to_np(flags[i]), new.astype(np.uint8))
     assert [t.size() for t in tabs] == [n] * tables
+
+
+@pytest.mark.parametrize("lanes", [2, 4])
+@pytest.mark.parametrize("ones", [False, True])
+def test_nearly_full_table_of_128_bit_keys(lanes, ones):
+    """ones: every low word all ones, so that every stored key reads as a claim candidate."""
+    n = 1000
+    hi = wk.distinct_keys(2 * n, 64, seed=lanes)
+    lo = np.full(2 * n, 2 ** 64 - 1, dtype=np.uint64) if ones else wk.distinct_keys(2 * n, 64, seed=9)
+    keys = np.stack([lo, hi], axis=1)
+    rng = np.random.default_rng(lanes)
+    t = ht.HashTable(1024, "bucket", 128, dict(bucket_slots=8, lanes_per_key=lanes))
+    orc = oracle.OracleTable128()
+    for idx in _batches(np.arange(n), rng) + [rng.permutation(np.tile(np.arange(n), 2))]:
+        got = to_np(t.find_or_put(to_dev(keys[idx])))
+        assert_flags_per_key(idx, got, orc.find_or_put(keys[idx]))
+    found, _ = t.lookup(to_dev(keys))
+    assert np.array_equal(to_np(found), np.repeat(np.array([1, 0], dtype=np.uint8), n))
+    assert t.sync() == 0 and t.size() == n
