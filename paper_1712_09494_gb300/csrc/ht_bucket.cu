@@ -1,21 +1,23 @@
 // GPUexplore-style bucket table (Section 4.2 of the paper).
 //
 // A key hashes to a bucket of BS 8-byte slots (BS*8 = 64/128/256 bytes,
-// aligned so one group's read is a single coalesced request).  A group of G
-// lanes reads the bucket, each lane BS/G consecutive slots; ballots give
-// every lane the bucket-wide "matches" and "free" masks (Fig. 4, steps 1-2).
-// If the key is present the group stops.  Otherwise the group CASes the free
-// slots in a fixed order until one CAS succeeds or returns the key itself
-// (step 3: another group may take a slot between the read and the CAS).
-// When the bucket has no free slot left, the next hash function picks the
-// next bucket; after the last one the key goes to the stash.
+// aligned).  The bucket is read whole by BS/8 lanes, whose ballots give the
+// "matches" and "free" masks (Fig. 4, steps 1-2), or a 32-byte sector at a time
+// by one lane (ht_bucket_tile.cuh).  If the key is present the search stops.
+// Otherwise the first free slot in the key's order of the bucket's slots is
+// CASed until a CAS succeeds or returns the key itself (step 3: another key may
+// take a slot between the read and the CAS).  When the bucket has no free slot
+// left, the next hash function picks the next bucket; after the last one the
+// key goes to the stash.
 //
 // Exactly-once: a slot never returns to empty and never changes its key, and
-// all groups with one key claim in the same order of the slots (from a place
-// that the key gives, around the bucket).  A group that claims slot s saw
-// every slot before it in that order holding another key, so a concurrent
-// group with the same key either meets the claimed word first or finds the
-// bucket full only after the word was written there.  A key goes
+// all copies of a key claim in the same order of the slots (sector after sector
+// from one that the key gives, around the bucket; in each sector from a slot
+// that the key gives).  A copy that claims slot s saw every slot before it in
+// that order holding another key, so a concurrent copy either meets the claimed
+// word first or finds the sector (the bucket) full only after the word was
+// written there; and a sector with a free slot shows the key in no sector after
+// it.  A key goes
 // to bucket f+1 only after bucket f was observed full without it, and
 // fullness is permanent, so lookups may stop at the first non-full bucket.
 #include <algorithm>
@@ -27,27 +29,25 @@ namespace {
 
 using namespace bucket;
 
-#ifndef HT_BUCKET_MIN_BLOCKS
-#define HT_BUCKET_MIN_BLOCKS 3
-#endif
-#ifndef HT_BUCKET_LOOKUP_MIN_BLOCKS
-#define HT_BUCKET_LOOKUP_MIN_BLOCKS 3
-#endif
+// Resident blocks per SM that the kernels are compiled for: 3 for whole
+// buckets (the fill of 2^27 keys takes 8.1 ms; 8.3 at 4), 5 for sectors
+// (a replay of 10^8 keys 0.99 ms; 1.05 at 3 and 4, 0.98 at 6).
+constexpr int kWholeBlocks = 3;
+constexpr int kSectorBlocks = 5;
 
 // find-or-put or lookup over one table.  A warp takes a fresh tile of 32 keys,
 // or 32 of its queued ones when that many wait (and the rest at the end), for
-// one pass over one bucket each (bucket_pass); the next two tiles' keys are
-// being loaded meanwhile.  A lookup in a table larger than L2 (ahead) also
-// touches the next tile's buckets, so that its reads hit L2.  Bound by random
-// 128-byte lines once the table is past L2 (40-46 G lines/s, 25 G/s where the
-// line is also written): find-or-put 22.8 G keys/s over a fill of 2^27 keys to
-// load 0.8 (19.2 with keys settled inside the tile), 41 on the successors of
-// 10^8 states (29); lookups 38 G/s (22; 31 without touching ahead, which gives
-// find-or-put nothing: its claims take the time).
-template <int KW, int BS, int G, bool VALUES, bool APPEND, bool LOOKUP>
+// one pass; the next two tiles' keys are being loaded meanwhile.  A lookup in a
+// table past L2 (WHOLE) also touches the next tile's buckets, so that its reads
+// hit L2.  Past L2 bound by random 128-byte lines (40-46 G lines/s, 25 G/s where
+// the line is also written): find-or-put 23 G keys/s over a fill of 2^27 keys to
+// load 0.8 (19 with whole tiles settled in place), 41 on the successors of 10^8
+// states (29); lookups 39 G/s (22; 31 without touching ahead, which gives
+// find-or-put nothing: its claims take the time).  In L2 100 G/s (27).
+template <int KW, int BS, bool VALUES, bool APPEND, bool LOOKUP, bool WHOLE>
 __device__ __forceinline__ void bucket_tiles(const DevTable& t, const void* keys, const uint32_t* vals, uint64_t n,
                                              uint8_t* flags, uint32_t* out_val, typename Keys<KW>::T* new_out,
-                                             unsigned long long* new_count, uint64_t new_cap, bool ahead) {
+                                             unsigned long long* new_count, uint64_t new_cap) {
     using K = Keys<KW>;
     using T = typename K::T;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -58,7 +58,7 @@ __device__ __forceinline__ void bucket_tiles(const DevTable& t, const void* keys
     WarpStage<T, kStageCap> stage(s_new[APPEND ? warp : 0]);
     Pending pend(s_pend[warp]);
     uint64_t base = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) / 32 * 32;
-    // This tile's key and bucket, the next tile's key.
+    // This tile's key and sector, the next tile's key.
     uint64_t key0 = 0, key1 = 0;
     uint32_t val0 = 0, val1 = 0;
     if (base + lane < n) {
@@ -69,31 +69,30 @@ __device__ __forceinline__ void bucket_tiles(const DevTable& t, const void* keys
         key1 = K::load(keys, base + step + lane);
         if (VALUES && !LOOKUP) val1 = vals[base + step + lane];
     }
-    uint64_t bkt0 = hidx(key0, t.seed[0], t.nbuckets);
+    auto start = [&](uint64_t key) { return first_sector<BS / kSec>(key, hidx(key, t.seed[0], t.nbuckets)); };
+    uint64_t sec0 = start(key0);
     // Bounded: an iteration takes a tile or up to 32 queued keys, and a key is
-    // queued at most once for each slot of its k buckets.
+    // queued at most once for each sector and slot of its k buckets.
     for (;;) {
         PendEntry d;
-        uint64_t bkt;
         bool mine, ok;
         if (pend.n >= 32 || (base >= n && pend.n)) {
-            d.key = d.pos = 0;
-            d.val = d.f = 0;
+            d.key = d.pos = d.sec = 0;
+            d.val = d.probe = 0;
             mine = ok = pend.pop(d);
-            bkt = hidx(d.key, t.seed[d.f], t.nbuckets);
         } else if (base < n) {
             d.key = key0;
             d.pos = base + lane;
+            d.sec = sec0;
             d.val = val0;
-            d.f = 0;
-            bkt = bkt0;
+            d.probe = 0;
             mine = d.pos < n;
             ok = mine && !K::reserved(d.key);
             if (mine && !ok) set_flag(t.ctr, kFlagInvalidKey);
             key0 = key1;
             val0 = val1;
-            bkt0 = hidx(key0, t.seed[0], t.nbuckets);
-            if (LOOKUP && ahead && base + step + lane < n) touch_l2(t.slots + bkt0 * BS);
+            sec0 = start(key0);
+            if (LOOKUP && WHOLE && base + step + lane < n) touch_l2(t.slots + sec0 / (BS / kSec) * BS);
             if (base + 2 * step + lane < n) {
                 key1 = K::load(keys, base + 2 * step + lane);
                 if (VALUES && !LOOKUP) val1 = vals[base + 2 * step + lane];
@@ -102,17 +101,12 @@ __device__ __forceinline__ void bucket_tiles(const DevTable& t, const void* keys
         } else {
             break;
         }
-        uint32_t v = 0;
-        uint32_t st = bucket_pass<KW, BS, G, VALUES, LOOKUP>(t.slots, d.key, d.val, bkt, ok, &v);
+        uint32_t v = 0, st;
         bool waits;
         if constexpr (LOOKUP) {
-            const bool next = st == kKeyFull;
-            if (next && ++d.f >= t.k) st = spill_find<KW>(t, d.key, &v);
-            waits = st == kKeyFull;
-            if (waits && ahead) touch_l2(t.slots + hidx(d.key, t.seed[d.f], t.nbuckets) * BS);
-            pend.push(waits, d.key, 0, d.pos, d.f);
+            st = find_pass<KW, BS, WHOLE>(t, pend, d, ok, waits, &v);
         } else {
-            st = settle_put<KW>(t, pend, st, d.key, d.val, d.pos, d.f, waits);
+            st = put_pass<KW, BS, WHOLE, APPEND>(t, pend, d, ok, waits);
             stored += st == kKeyHit;
             if (APPEND) stage.push(st == kKeyHit, T(d.key), new_out, new_count, new_cap);
         }
@@ -125,68 +119,64 @@ __device__ __forceinline__ void bucket_tiles(const DevTable& t, const void* keys
     if (!LOOKUP) add_size<kBlock>(t, stored);
 }
 
-template <int KW, int BS, int G, bool VALUES, bool APPEND>
-__global__ void __launch_bounds__(kBlock, HT_BUCKET_MIN_BLOCKS)
+template <int KW, int BS, bool VALUES, bool APPEND, bool WHOLE>
+__global__ void __launch_bounds__(kBlock, WHOLE ? kWholeBlocks : kSectorBlocks)
 bucket_fop_kernel(const __grid_constant__ DevTable t, const void* __restrict__ keys, const uint32_t* __restrict__ vals,
                   uint64_t n, const unsigned long long* __restrict__ d_n, uint8_t* __restrict__ is_new,
                   typename Keys<KW>::T* __restrict__ new_out, unsigned long long* __restrict__ new_count,
                   uint64_t new_cap) {
     if (d_n) n = min(n, uint64_t(__ldcg(d_n)));        // batch size produced on the device
-    bucket_tiles<KW, BS, G, VALUES, APPEND, false>(t, keys, vals, n, is_new, nullptr, new_out, new_count, new_cap,
-                                                   false);
+    bucket_tiles<KW, BS, VALUES, APPEND, false, WHOLE>(t, keys, vals, n, is_new, nullptr, new_out, new_count, new_cap);
 }
 
 // Lookup: like find-or-put without claims; a bucket with a free slot ends the
 // search (a key only moves on from a full bucket), all k full -> the spill.
-template <int KW, int BS, int G, bool VALUES>
-__global__ void __launch_bounds__(kBlock, HT_BUCKET_LOOKUP_MIN_BLOCKS)
+template <int KW, int BS, bool VALUES, bool WHOLE>
+__global__ void __launch_bounds__(kBlock, WHOLE ? kWholeBlocks : kSectorBlocks)
 bucket_lookup_kernel(const __grid_constant__ DevTable t, const void* __restrict__ keys, uint64_t n,
-                     uint32_t* __restrict__ vals, uint8_t* __restrict__ found, bool ahead) {
-    bucket_tiles<KW, BS, G, VALUES, false, true>(t, keys, nullptr, n, found, vals, nullptr, nullptr, 0, ahead);
+                     uint32_t* __restrict__ vals, uint8_t* __restrict__ found) {
+    bucket_tiles<KW, BS, VALUES, false, true, WHOLE>(t, keys, nullptr, n, found, vals, nullptr, nullptr, 0);
 }
 
-// A table larger than L2: a lookup touches its buckets one tile ahead.  Below
-// that the reads hit L2 anyway and this is one more L2 request per key.
+// Tables past L2 have their buckets read whole, smaller ones a sector at a time
+// (the reason and both sides' times are at the passes, ht_bucket_tile.cuh).
 bool past_l2(const DevTable& t) { return t.nslots * 8 > l2_bytes(); }
 
-template <int KW, int BS, int G>
+template <int KW, int BS, bool WHOLE>
 cudaError_t launch_fop(const DevTable& t, const void* keys, const uint32_t* vals, uint64_t n,
                        const unsigned long long* d_n, uint8_t* is_new, void* new_out,
                        unsigned long long* new_count, uint64_t new_cap, cudaStream_t s, const L2Window& w) {
     using T = typename Keys<KW>::T;
-    ProfScope ps(kKBucketFop, s);
-    auto k = vals ? bucket_fop_kernel<KW, BS, G, KW == 32, false>
-             : new_out ? bucket_fop_kernel<KW, BS, G, false, true> : bucket_fop_kernel<KW, BS, G, false, false>;
+    auto k = vals ? bucket_fop_kernel<KW, BS, KW == 32, false, WHOLE>
+             : new_out ? bucket_fop_kernel<KW, BS, false, true, WHOLE> : bucket_fop_kernel<KW, BS, false, false, WHOLE>;
     return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, keys, vals, n, d_n, is_new,
                       static_cast<T*>(new_out), new_count, new_cap);
 }
 
-template <int KW, int BS, int G>
+template <int KW, int BS, bool WHOLE>
 cudaError_t launch_lookup(const DevTable& t, const void* keys, uint64_t n, uint32_t* vals,
                           uint8_t* found, cudaStream_t s, const L2Window& w) {
-    ProfScope ps(kKBucketLookup, s);
-    auto k = vals ? bucket_lookup_kernel<KW, BS, G, true> : bucket_lookup_kernel<KW, BS, G, false>;
-    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, keys, n, vals, found,
-                      past_l2(t));
+    auto k = vals ? bucket_lookup_kernel<KW, BS, true, WHOLE> : bucket_lookup_kernel<KW, BS, false, WHOLE>;
+    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, keys, n, vals, found);
 }
 
 // Multi-table find-or-put of one step (the body is shared with the
 // persistent kernel, bucket::multi_find_or_put).
-template <int BS, int G>
-__global__ void __launch_bounds__(kBlock, HT_BUCKET_MIN_BLOCKS)
+template <int BS>
+__global__ void __launch_bounds__(kBlock, 4)
 multi_bucket_fop_kernel(const __grid_constant__ MultiDev m, uint64_t) {
-    __shared__ uint64_t s_new[kBlock / 32][kStageCap];
+    __shared__ uint64_t s_new[kBlock / 32][kMultiStage];
     __shared__ unsigned int s_first[multi::kExactTileExpl + 1];
     __shared__ unsigned long long s_scan[multi::kAdvShared];
     __shared__ PendEntry s_pend[kBlock / 32][kPend];
     const multi::TileMap tm = multi::tile_map<kBlock>(m, s_first, s_scan);
     const uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
     const uint64_t gw = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    multi_find_or_put<BS, G>(m, tm, gw, nwarps, s_new[threadIdx.x >> 5], s_pend[threadIdx.x >> 5]);
+    multi_find_or_put<BS>(m, tm, gw, nwarps, s_new[threadIdx.x >> 5], s_pend[threadIdx.x >> 5]);
 }
 
 // One warp per exploration: level 0 is the initial state.
-template <int BS, int G>
+template <int BS>
 __global__ void __launch_bounds__(kBlock) multi_bucket_init_kernel(const MultiDev m) {
     const int lane = threadIdx.x & 31;
     const uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
@@ -195,13 +185,19 @@ __global__ void __launch_bounds__(kBlock) multi_bucket_init_kernel(const MultiDe
         const bool ok = lane == 0 && !Keys<64>::reserved(key);
         const DevTable& t = m.tables[e];
         uint32_t st = kKeyDone;
-        bool go = ok;
-        for (uint32_t f = 0; __any_sync(kFull, go);) {      // bounded: k buckets, each claim takes a slot
-            st = bucket_pass<64, BS, G, false, false>(t.slots, key, 0, hidx(key, t.seed[f], t.nbuckets), go);
-            if (st == kKeyFull && ++f >= t.k) st = spill_put<64>(t, key, 0);
+        PendEntry d;
+        d.key = key;
+        d.val = d.probe = 0;
+        d.sec = first_sector<BS / kSec>(key, hidx(key, t.seed[0], t.nbuckets));
+        for (bool go = ok; go;) {               // bounded: the sectors of k buckets, each lost claim takes a slot
+            st = sector_pass<64, false>(t.slots, key, 0, d.sec, true);
             go = st >= kKeyLost;
-            f = __shfl_sync(kFull, f, 0);
+            if (st == kKeyFull && !advance<BS / kSec, false>(t, d)) {
+                st = spill_put<64>(t, key, 0);
+                go = false;
+            }
         }
+        __syncwarp();
         const bool my_new = st == kKeyHit;
         if (lane == 0) {
             if (ok && my_new) {
@@ -223,15 +219,15 @@ __global__ void __launch_bounds__(kBlock) multi_bucket_init_kernel(const MultiDe
     }
 }
 
-template <int BS, int G>
+template <int BS>
 cudaError_t launch_multi(const MultiDev& m, uint64_t max_tiles, bool init, cudaStream_t s) {
     if (init) {
-        auto k = multi_bucket_init_kernel<BS, G>;
+        auto k = multi_bucket_init_kernel<BS>;
         const int grid = int(std::min<uint64_t>(launch_blocks((const void*)k, kBlock), (m.count + 7) / 8));
         k<<<grid, kBlock, 0, s>>>(m);
     } else {
         ProfScope ps(kKBucketFop, s);
-        auto k = multi_bucket_fop_kernel<BS, G>;
+        auto k = multi_bucket_fop_kernel<BS>;
         k<<<launch_blocks((const void*)k, kBlock), kBlock, 0, s>>>(m, max_tiles);
     }
     return cudaGetLastError();
@@ -242,8 +238,8 @@ cudaError_t launch_multi(const MultiDev& m, uint64_t max_tiles, bool init, cudaS
 // items and each warp takes a contiguous range of them, finds its first
 // tile's item once and walks the items in order, keeping the item's
 // descriptor in registers and its table's size count until it moves on.
-template <int KW, int BS, int G>
-__global__ void __launch_bounds__(kBlock, HT_BUCKET_MIN_BLOCKS)
+template <int KW, int BS>
+__global__ void __launch_bounds__(kBlock, 4)
 packed_bucket_kernel(const DevTable* __restrict__ tables, const WorkDesc* __restrict__ items, uint32_t nitems,
                      uint64_t ntiles) {
     using K = Keys<KW>;
@@ -267,8 +263,8 @@ packed_bucket_kernel(const DevTable* __restrict__ tables, const WorkDesc* __rest
     for (uint64_t tile = t_begin;;) {
         const bool moves = tile >= t_end || tile >= next_off;      // done with the item's tiles
         PendEntry p;
-        p.key = p.pos = 0;
-        p.val = p.f = 0;
+        p.key = p.pos = p.sec = 0;
+        p.val = p.probe = 0;
         bool mine, ok;
         if (pend.n >= 32 || (moves && pend.n)) {
             mine = ok = pend.pop(p);
@@ -289,11 +285,11 @@ packed_bucket_kernel(const DevTable* __restrict__ tables, const WorkDesc* __rest
             ok = mine && !K::reserved(p.key);
             if (mine && !ok) set_flag(tables[d.table].ctr, kFlagInvalidKey);
             ++tile;
+            const DevTable& t = tables[d.table];
+            p.sec = first_sector<BS / kSec>(p.key, hidx(p.key, t.seed[0], t.nbuckets));
         }
-        const DevTable& t = tables[d.table];
-        uint32_t st = bucket_pass<KW, BS, G, false, false>(t.slots, p.key, 0, hidx(p.key, t.seed[p.f], t.nbuckets), ok);
         bool waits;
-        st = settle_put<KW>(t, pend, st, p.key, 0, p.pos, p.f, waits);
+        const uint32_t st = put_pass<KW, BS, false, false>(tables[d.table], pend, p, ok, waits);
         if (mine && !waits && d.flags) d.flags[p.pos] = uint8_t(st);
         stored += __popc(__ballot_sync(kFull, st == kKeyHit));
     }
@@ -308,8 +304,8 @@ packed_bucket_kernel(const DevTable* __restrict__ tables, const WorkDesc* __rest
 constexpr int kFusedBlock = 128;
 constexpr int kFusedStage = 512;
 
-template <int KW, int BS, int G>
-__global__ void __launch_bounds__(kFusedBlock, HT_BUCKET_MIN_BLOCKS * 2)
+template <int KW, int BS, bool WHOLE>
+__global__ void __launch_bounds__(kFusedBlock, kWholeBlocks * 2)
 bfs_fused_kernel(const PreparedModel* __restrict__ model, const typename Keys<KW>::T* __restrict__ frontier,
                  uint64_t n, const __grid_constant__ DevTable t, typename Keys<KW>::T* __restrict__ out,
                  unsigned long long* __restrict__ count, uint64_t cap, unsigned long long* __restrict__ gen) {
@@ -337,14 +333,12 @@ bfs_fused_kernel(const PreparedModel* __restrict__ model, const typename Keys<KW
     auto step = [&](bool queued, uint64_t key, bool ok) {
         PendEntry d;
         d.key = key;
-        d.f = 0;
-        if (queued) {
-            d.key = 0;
-            ok = pend.pop(d);
-        }
-        uint32_t res = bucket_pass<KW, BS, G, false, false>(t.slots, d.key, 0, hidx(d.key, t.seed[d.f], t.nbuckets), ok);
+        d.pos = d.sec = 0;
+        d.val = d.probe = 0;
+        if (queued) ok = pend.pop(d);
+        else d.sec = first_sector<BS / kSec>(key, hidx(key, t.seed[0], t.nbuckets));
         bool waits;
-        res = settle_put<KW>(t, pend, res, d.key, 0, 0, d.f, waits);
+        const uint32_t res = put_pass<KW, BS, WHOLE, true>(t, pend, d, ok, waits);
         stage.push(res == kKeyHit, T(d.key), out, count, cap);
         stored += res == kKeyHit;
     };
@@ -394,9 +388,8 @@ bfs_fused_kernel(const PreparedModel* __restrict__ model, const typename Keys<KW
     add_size<kFusedBlock>(t, stored);
 }
 
-// (bucket_slots, lanes) pairs that are instantiated.
-#define HT_BUCKET_CONFIGS(X) \
-    X(8, 2) X(8, 4) X(8, 8) X(16, 2) X(16, 4) X(16, 8) X(16, 16) X(32, 4) X(32, 8) X(32, 16) X(32, 32)
+// The bucket sizes that are instantiated.
+#define HT_BUCKET_CONFIGS(X) X(8) X(16) X(32)
 
 }  // namespace
 
@@ -404,28 +397,34 @@ cudaError_t bucket_find_or_put(const BucketCfg& c, const DevTable& t, const void
                                const uint32_t* vals, uint64_t n, const unsigned long long* d_n,
                                uint8_t* is_new, void* new_out, unsigned long long* new_count,
                                uint64_t new_cap, cudaStream_t s, const L2Window& w) {
-#define X(BS, G)                                                                                  \
-    if (c.bucket_slots == BS && c.lanes == G)                                                     \
-        return c.kw == 32 ? launch_fop<32, BS, G>(t, keys, vals, n, d_n, is_new, new_out, new_count, new_cap, s, w) \
-                          : launch_fop<64, BS, G>(t, keys, vals, n, d_n, is_new, new_out, new_count, new_cap, s, w);
+    ProfScope ps(kKBucketFop, s);
+#define L(KW, BS)                                                                                                    \
+    return past_l2(t) ? launch_fop<KW, BS, true>(t, keys, vals, n, d_n, is_new, new_out, new_count, new_cap, s, w)   \
+                      : launch_fop<KW, BS, false>(t, keys, vals, n, d_n, is_new, new_out, new_count, new_cap, s, w);
+#define X(BS)                                                                                                        \
+    if (c.bucket_slots == BS) {                                                                                      \
+        if (c.kw == 32) L(32, BS)                                                                                    \
+        L(64, BS)                                                                                                    \
+    }
     HT_BUCKET_CONFIGS(X)
 #undef X
+#undef L
     return cudaErrorInvalidValue;
 }
 
 cudaError_t multi_bucket_find_or_put(const BucketCfg& c, const MultiDev& m, uint64_t max_tiles, cudaStream_t s) {
-#define X(BS, G)                                                                       \
-    if (c.bucket_slots == BS && c.lanes == G)                                          \
-        return launch_multi<BS, G>(m, max_tiles, false, s);
+#define X(BS)                                                                       \
+    if (c.bucket_slots == BS)                                          \
+        return launch_multi<BS>(m, max_tiles, false, s);
     HT_BUCKET_CONFIGS(X)
 #undef X
     return cudaErrorInvalidValue;
 }
 
 cudaError_t multi_bucket_init(const BucketCfg& c, const MultiDev& m, cudaStream_t s) {
-#define X(BS, G)                                                                       \
-    if (c.bucket_slots == BS && c.lanes == G)                                          \
-        return launch_multi<BS, G>(m, 0, true, s);
+#define X(BS)                                                                       \
+    if (c.bucket_slots == BS)                                          \
+        return launch_multi<BS>(m, 0, true, s);
     HT_BUCKET_CONFIGS(X)
 #undef X
     return cudaErrorInvalidValue;
@@ -435,17 +434,17 @@ cudaError_t packed_bucket_find_or_put(const BucketCfg& c, const DevTable* tables
                                       uint32_t nitems, uint64_t ntiles, cudaStream_t s) {
     if (!nitems || !ntiles) return cudaSuccess;
     ProfScope ps(kKBucketFop, s);
-#define L(KW, BS, G)                                                                                      \
+#define L(KW, BS)                                                                                      \
     {                                                                                                     \
-        auto k = packed_bucket_kernel<KW, BS, G>;                                                         \
+        auto k = packed_bucket_kernel<KW, BS>;                                                         \
         const int grid = int(std::min<uint64_t>(launch_blocks((const void*)k, kBlock), (ntiles + 7) / 8)); \
         k<<<grid, kBlock, 0, s>>>(tables, items, nitems, ntiles);                                         \
         return cudaGetLastError();                                                                        \
     }
-#define X(BS, G)                                                                                          \
-    if (c.bucket_slots == BS && c.lanes == G) {                                                           \
-        if (c.kw == 32) L(32, BS, G)                                                                      \
-        L(64, BS, G)                                                                                      \
+#define X(BS)                                                                                          \
+    if (c.bucket_slots == BS) {                                                           \
+        if (c.kw == 32) L(32, BS)                                                                      \
+        L(64, BS)                                                                                      \
     }
     HT_BUCKET_CONFIGS(X)
 #undef X
@@ -458,18 +457,18 @@ cudaError_t bfs_fused_level(const BucketCfg& c, const PreparedModel* model, cons
                             unsigned long long* gen, cudaStream_t s) {
     if (!n) return cudaSuccess;
     ProfScope ps(kKBucketFop, s);
-#define L(KW, BS, G)                                                                                     \
+#define L(KW, BS)                                                                                     \
     {                                                                                                    \
         using T = typename Keys<KW>::T;                                                                  \
-        auto k = bfs_fused_kernel<KW, BS, G>;                                                            \
+        auto k = past_l2(t) ? bfs_fused_kernel<KW, BS, true> : bfs_fused_kernel<KW, BS, false>;                                                            \
         k<<<launch_blocks((const void*)k, kFusedBlock), kFusedBlock, 0, s>>>(                            \
             model, static_cast<const T*>(frontier), n, t, static_cast<T*>(out), count, cap, gen);        \
         return cudaGetLastError();                                                                       \
     }
-#define X(BS, G)                                                                                         \
-    if (c.bucket_slots == BS && c.lanes == G) {                                                          \
-        if (c.kw == 32) L(32, BS, G)                                                                     \
-        L(64, BS, G)                                                                                     \
+#define X(BS)                                                                                         \
+    if (c.bucket_slots == BS) {                                                          \
+        if (c.kw == 32) L(32, BS)                                                                     \
+        L(64, BS)                                                                                     \
     }
     HT_BUCKET_CONFIGS(X)
 #undef X
@@ -479,12 +478,18 @@ cudaError_t bfs_fused_level(const BucketCfg& c, const PreparedModel* model, cons
 
 cudaError_t bucket_lookup(const BucketCfg& c, const DevTable& t, const void* keys, uint64_t n,
                           uint32_t* vals, uint8_t* found, cudaStream_t s, const L2Window& w) {
-#define X(BS, G)                                                                    \
-    if (c.bucket_slots == BS && c.lanes == G)                                       \
-        return c.kw == 32 ? launch_lookup<32, BS, G>(t, keys, n, vals, found, s, w)   \
-                          : launch_lookup<64, BS, G>(t, keys, n, vals, found, s, w);
+    ProfScope ps(kKBucketLookup, s);
+#define L(KW, BS)                                                                       \
+    return past_l2(t) ? launch_lookup<KW, BS, true>(t, keys, n, vals, found, s, w)      \
+                      : launch_lookup<KW, BS, false>(t, keys, n, vals, found, s, w);
+#define X(BS)                                                                           \
+    if (c.bucket_slots == BS) {                                                         \
+        if (c.kw == 32) L(32, BS)                                                       \
+        L(64, BS)                                                                       \
+    }
     HT_BUCKET_CONFIGS(X)
 #undef X
+#undef L
     return cudaErrorInvalidValue;
 }
 

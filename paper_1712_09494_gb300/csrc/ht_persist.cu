@@ -85,8 +85,9 @@ __device__ bool grid_sync(const MultiDev& m, int* s_ok) {
 }
 
 // Level 0 of every exploration: its initial state placed in its (empty)
-// table -- bucket scheme: the first slot of bucket h_1 (nothing else claims
-// yet, so any free slot does); Cuckoo: slot h_1 -- and stored as the first state.
+// table -- bucket scheme: in the sector of bucket h_1 where its search starts
+// (nothing else claims yet, so any slot of it does); Cuckoo: slot h_1 -- and
+// stored as the first state.
 // Tables are addressed as 64-bit key tables (a 32-bit set table's words are
 // the same), states are written in their exploration's width.
 template <bool CUCKOO, int BS>
@@ -94,7 +95,9 @@ __device__ void place_initial_states(const MultiDev& m, uint64_t gtid, uint64_t 
     for (uint64_t e = gtid; e < m.count; e += nthreads) {
         const uint64_t key = m.s0[e];
         const DevTable& t = m.tables[e];
-        const uint64_t pos = CUCKOO ? hidx(key, t.seed[0], t.nslots) : hidx(key, t.seed[0], t.nbuckets) * BS;
+        uint64_t pos = hidx(key, t.seed[0], t.nslots);
+        if (!CUCKOO)
+            pos = bucket::first_sector<BS / bucket::kSec>(key, hidx(key, t.seed[0], t.nbuckets)) * bucket::kSec;
         const uint64_t old = atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + pos), kEmpty, key);
         if (old != kEmpty) atomicOr(m.status, kMultiBadInit);
         if (m.narrow[e]) static_cast<unsigned int*>(m.states[e])[0] = static_cast<unsigned int>(key);
@@ -385,21 +388,21 @@ __device__ void cuckoo_insert_winners(const MultiDev& m, uint64_t gtid, uint64_t
     if (run_n) atomicAdd(&m.tables[run_e].ctr->size, run_n);
 }
 
-// Resident blocks per SM the kernel is compiled for (registers): measured
-// on config 4, the bucket kernel is fastest at 2 (no spills), the Cuckoo
-// kernel at 3.
+// Resident blocks per SM the kernel is compiled for (registers): measured on
+// 256 explorations of 38 M states, the bucket kernel is fastest at 4 (20.0 ms;
+// 22.5 at 3, 28.7 at 2), the Cuckoo kernel at 3.
 #ifndef HT_PERSIST_MIN_BLOCKS_BUCKET
-#define HT_PERSIST_MIN_BLOCKS_BUCKET 2
+#define HT_PERSIST_MIN_BLOCKS_BUCKET 4
 #endif
 #ifndef HT_PERSIST_MIN_BLOCKS_CUCKOO
 #define HT_PERSIST_MIN_BLOCKS_CUCKOO 3
 #endif
 
-template <bool CUCKOO, int BS, int G>
+template <bool CUCKOO, int BS>
 __global__ void __launch_bounds__(kBlock, CUCKOO ? HT_PERSIST_MIN_BLOCKS_CUCKOO : HT_PERSIST_MIN_BLOCKS_BUCKET)
 multi_persistent_kernel(const __grid_constant__ MultiDev m, uint64_t budget, uint64_t max_steps, uint64_t max_work,
                         uint64_t max_tiles) {
-    __shared__ uint64_t s_new[kBlock / 32][kStageCap];
+    __shared__ uint64_t s_new[kBlock / 32][CUCKOO ? kStageCap : bucket::kMultiStage];
     __shared__ unsigned long long sh[multi::kAdvShared];
     __shared__ unsigned int s_first[multi::kExactTileExpl + 1];
     __shared__ MultiWinner s_win[kBlock / 32][CUCKOO ? kWinStage : 1];
@@ -426,17 +429,17 @@ multi_persistent_kernel(const __grid_constant__ MultiDev m, uint64_t budget, uin
             if (!grid_sync(m, &s_ok)) return;
             cuckoo_insert_winners(m, gtid, nthreads);
         } else {
-            bucket::multi_find_or_put<BS, G>(m, tm, gw, nwarps, stage, s_pend[threadIdx.x >> 5]);
+            bucket::multi_find_or_put<BS>(m, tm, gw, nwarps, stage, s_pend[threadIdx.x >> 5]);
         }
         if (!grid_sync(m, &s_ok)) return;
     }
     if (gtid == 0) *m.steps = step;
 }
 
-template <bool CUCKOO, int BS, int G>
+template <bool CUCKOO, int BS>
 cudaError_t launch_persistent(const MultiDev& m, uint64_t budget, uint64_t max_steps, uint64_t max_work,
                               uint64_t max_tiles, cudaStream_t s) {
-    auto k = multi_persistent_kernel<CUCKOO, BS, G>;
+    auto k = multi_persistent_kernel<CUCKOO, BS>;
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -456,11 +459,10 @@ cudaError_t launch_persistent(const MultiDev& m, uint64_t budget, uint64_t max_s
 
 cudaError_t multi_persistent(ht_scheme scheme, const BucketCfg& c, const MultiDev& m, uint64_t budget,
                              uint64_t max_steps, uint64_t max_work, uint64_t max_tiles, cudaStream_t s) {
-    if (scheme == HT_CUCKOO) return launch_persistent<true, 16, 2>(m, budget, max_steps, max_work, max_tiles, s);
-#define P(BS, G)                                                                                           \
-    if (c.bucket_slots == BS && c.lanes == G)                                                              \
-        return launch_persistent<false, BS, G>(m, budget, max_steps, max_work, max_tiles, s);
-    P(16, 2) P(16, 4) P(16, 8) P(16, 16) P(8, 2) P(8, 4) P(8, 8) P(32, 4) P(32, 8) P(32, 16) P(32, 32)
+    if (scheme == HT_CUCKOO) return launch_persistent<true, 16>(m, budget, max_steps, max_work, max_tiles, s);
+#define P(BS) \
+    if (c.bucket_slots == BS) return launch_persistent<false, BS>(m, budget, max_steps, max_work, max_tiles, s);
+    P(8) P(16) P(32)
 #undef P
     return cudaErrorInvalidValue;
 }

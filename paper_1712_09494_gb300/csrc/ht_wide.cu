@@ -128,17 +128,7 @@ __device__ __forceinline__ uint32_t wide_pass(uint64_t* slots, ulonglong2 mykey,
             const int kidx = (r0 + q) * GPW + grp;
             at[q] = 2 * (__shfl_sync(kFull, mybkt, kidx) * kWideBS + uint32_t(sub * SPL));
             ok[q] = (okmask >> kidx) & 1u;
-#pragma unroll
-            for (int j = 0; j < 2 * SPL; j += 4) {
-                unsigned long long a = 0, b = 0, c = 0, d = 0;
-                if (ok[q])
-                    asm volatile("ld.global.cg.v4.u64 {%0,%1,%2,%3}, [%4];"
-                                 : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(slots + at[q] + j));
-                w[q][j] = a;
-                w[q][j + 1] = b;
-                w[q][j + 2] = c;
-                w[q][j + 3] = d;
-            }
+            bucket::load_sectors<2 * SPL>(slots + at[q], ok[q], w[q]);
         }
         bool more = false;
 #pragma unroll
@@ -168,7 +158,7 @@ __device__ __forceinline__ uint32_t wide_pass(uint64_t* slots, ulonglong2 mykey,
                 done[q] |= ge != 0;                 // a key moves on only from a full bucket
                 if (myround == r0 + q && ((M >> mysh) & kGMask)) status = 1;
             } else {
-                rot[q] = bucket::claim_rot<kWideBS>(lo[q] ^ hi[q]);
+                rot[q] = (bucket::claim_rot(lo[q] ^ hi[q]) % kWideBS);
                 const uint32_t ge = (__ballot_sync(kFull, cand[q] != 0) >> gbase) & kGMask;
                 if (cand[q] && uint32_t(sub) == bucket::first_from<G>(ge, rot[q] / SPL)) {
                     claim[q] = int(bucket::first_from<SPL>(cand[q], rot[q] % SPL));

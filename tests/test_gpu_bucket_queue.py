@@ -95,3 +95,41 @@ def test_nearly_full_table_of_128_bit_keys(lanes, ones):
     found, _ = t.lookup(to_dev(keys))
     assert np.array_equal(to_np(found), np.repeat(np.array([1, 0], dtype=np.uint8), n))
     assert t.sync() == 0 and t.size() == n
+
+
+@pytest.mark.parametrize("bs,lanes", [(8, 2), (16, 2), (32, 4)])
+@pytest.mark.parametrize("kw", [32, 64])
+def test_table_past_l2_at_high_load(kw, bs, lanes):
+    """Tables larger than L2 (other kernels than small ones) at load 0.95: every batch's fresh keys are new and its
+    repeats are not, all stored keys are found with their values and no other key is."""
+    from workloads import device_keys as dk
+    slots = 24_000_000                                  # 192 MB
+    n = int(slots * 0.95)
+    idx = torch.arange(2 * n, dtype=torch.int64, device="cuda")
+    if kw == 64:
+        keys = dk.mix63_perm_dev(idx, bs)
+    else:
+        k = dk.mix32_perm_dev(idx, bs)
+        keys = (k - ((k >> 31) << 32)).to(torch.int32)
+    t = ht.HashTable(slots, "bucket", kw, dict(bucket_slots=bs, lanes_per_key=lanes))
+    vals = (idx[:n] * 3 + 1).to(torch.int32)
+    at = 0
+    for m in (n // 2 + 7, n // 4 + 13, 1, 31, n):
+        m = min(m, n - at)
+        rep = torch.randint(0, at, (m // 4,), device="cuda") if at else idx[:0]
+        if at == 0 and kw == 32:
+            t.insert(keys[:m], vals[:m])                # the rest of the keys get value 0
+        else:
+            order = torch.randperm(m + len(rep), device="cuda")
+            batch = torch.cat([keys[at:at + m], keys[rep]])[order]
+            assert torch.equal(t.find_or_put(batch), (order < m).to(torch.uint8))
+        if at == 0:
+            first = m
+        at += m
+    found, v = t.lookup(keys)
+    assert torch.equal(found, (idx < n).to(torch.uint8))
+    if kw == 32:
+        want = torch.zeros(2 * n, dtype=torch.int32, device="cuda")
+        want[:first] = vals[:first]
+        assert torch.equal(v, want)
+    assert t.sync() == 0 and t.size() == n
