@@ -38,13 +38,13 @@ constexpr int kSectorBlocks = 5;
 // find-or-put or lookup over one table.  A warp takes a fresh tile of 32 keys,
 // or 32 of its queued ones when that many wait (and the rest at the end), for
 // one pass; the next two tiles' keys are being loaded meanwhile.  A lookup in a
-// table past L2 (WHOLE) also touches the next tile's buckets, so that its reads
+// table past L2 (AHEAD) also touches the next tile's buckets, so that its reads
 // hit L2.  Past L2 bound by random 128-byte lines (40-46 G lines/s, 25 G/s where
 // the line is also written): find-or-put 23 G keys/s over a fill of 2^27 keys to
 // load 0.8 (19 with whole tiles settled in place), 41 on the successors of 10^8
 // states (29); lookups 39 G/s (22; 31 without touching ahead, which gives
 // find-or-put nothing: its claims take the time).  In L2 100 G/s (27).
-template <int KW, int BS, bool VALUES, bool APPEND, bool LOOKUP, bool WHOLE>
+template <int KW, int BS, bool VALUES, bool APPEND, bool LOOKUP, bool WHOLE, bool AHEAD>
 __device__ __forceinline__ void bucket_tiles(const DevTable& t, const void* keys, const uint32_t* vals, uint64_t n,
                                              uint8_t* flags, uint32_t* out_val, typename Keys<KW>::T* new_out,
                                              unsigned long long* new_count, uint64_t new_cap) {
@@ -92,7 +92,7 @@ __device__ __forceinline__ void bucket_tiles(const DevTable& t, const void* keys
             key0 = key1;
             val0 = val1;
             sec0 = start(key0);
-            if (LOOKUP && WHOLE && base + step + lane < n) touch_l2(t.slots + sec0 / (BS / kSec) * BS);
+            if (AHEAD && base + step + lane < n) touch_l2(t.slots + sec0 / (BS / kSec) * BS);
             if (base + 2 * step + lane < n) {
                 key1 = K::load(keys, base + 2 * step + lane);
                 if (VALUES && !LOOKUP) val1 = vals[base + 2 * step + lane];
@@ -104,7 +104,7 @@ __device__ __forceinline__ void bucket_tiles(const DevTable& t, const void* keys
         uint32_t v = 0, st;
         bool waits;
         if constexpr (LOOKUP) {
-            st = find_pass<KW, BS, WHOLE>(t, pend, d, ok, waits, &v);
+            st = find_pass<KW, BS, AHEAD>(t, pend, d, ok, waits, &v);
         } else {
             st = put_pass<KW, BS, WHOLE, APPEND>(t, pend, d, ok, waits);
             stored += st == kKeyHit;
@@ -126,21 +126,30 @@ bucket_fop_kernel(const __grid_constant__ DevTable t, const void* __restrict__ k
                   typename Keys<KW>::T* __restrict__ new_out, unsigned long long* __restrict__ new_count,
                   uint64_t new_cap) {
     if (d_n) n = min(n, uint64_t(__ldcg(d_n)));        // batch size produced on the device
-    bucket_tiles<KW, BS, VALUES, APPEND, false, WHOLE>(t, keys, vals, n, is_new, nullptr, new_out, new_count, new_cap);
+    bucket_tiles<KW, BS, VALUES, APPEND, false, WHOLE, false>(t, keys, vals, n, is_new, nullptr, new_out, new_count, new_cap);
 }
 
 // Lookup: like find-or-put without claims; a bucket with a free slot ends the
 // search (a key only moves on from a full bucket), all k full -> the spill.
-template <int KW, int BS, bool VALUES, bool WHOLE>
-__global__ void __launch_bounds__(kBlock, WHOLE ? kWholeBlocks : kSectorBlocks)
+// Buckets are read whole at every size: an absent key takes 3.1 sectors at load
+// 0.8 (2^22 lookups, half absent, in L2: 78 us by sectors, 74 whole; 2^14: 17, 12).
+template <int KW, int BS, bool VALUES, bool AHEAD>
+__global__ void __launch_bounds__(kBlock, kWholeBlocks)
 bucket_lookup_kernel(const __grid_constant__ DevTable t, const void* __restrict__ keys, uint64_t n,
                      uint32_t* __restrict__ vals, uint8_t* __restrict__ found) {
-    bucket_tiles<KW, BS, VALUES, false, true, WHOLE>(t, keys, nullptr, n, found, vals, nullptr, nullptr, 0);
+    bucket_tiles<KW, BS, VALUES, false, true, true, AHEAD>(t, keys, nullptr, n, found, vals, nullptr, nullptr, 0);
 }
 
-// Tables past L2 have their buckets read whole, smaller ones a sector at a time
-// (the reason and both sides' times are at the passes, ht_bucket_tile.cuh).
+// Tables past L2 have their buckets read whole (the reason and both sides' times
+// are at the passes, ht_bucket_tile.cuh).
 bool past_l2(const DevTable& t) { return t.nslots * 8 > l2_bytes(); }
+
+// So have small batches in smaller tables: a warp then has one tile, and its
+// unsettled keys' passes come one after another, more of them by sectors.  New
+// keys to load 0.8 and stored keys, us a batch by sectors / whole: 2^14 keys
+// 10.6 / 9.2 and 7.8 / 6.8, 2^18 19.9 / 17.3 and 8.8 / 10.9, 2^20 35.9 / 35.9 and
+// 12.9 / 23.2, 2^22 103 / 101 and 37 / 85.
+constexpr uint64_t kSectorKeys = 1ull << 19;
 
 template <int KW, int BS, bool WHOLE>
 cudaError_t launch_fop(const DevTable& t, const void* keys, const uint32_t* vals, uint64_t n,
@@ -153,10 +162,11 @@ cudaError_t launch_fop(const DevTable& t, const void* keys, const uint32_t* vals
                       static_cast<T*>(new_out), new_count, new_cap);
 }
 
-template <int KW, int BS, bool WHOLE>
+template <int KW, int BS>
 cudaError_t launch_lookup(const DevTable& t, const void* keys, uint64_t n, uint32_t* vals,
                           uint8_t* found, cudaStream_t s, const L2Window& w) {
-    auto k = vals ? bucket_lookup_kernel<KW, BS, true, WHOLE> : bucket_lookup_kernel<KW, BS, false, WHOLE>;
+    auto k = past_l2(t) ? (vals ? bucket_lookup_kernel<KW, BS, true, true> : bucket_lookup_kernel<KW, BS, false, true>)
+                        : (vals ? bucket_lookup_kernel<KW, BS, true, false> : bucket_lookup_kernel<KW, BS, false, false>);
     return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, keys, n, vals, found);
 }
 
@@ -190,7 +200,7 @@ __global__ void __launch_bounds__(kBlock) multi_bucket_init_kernel(const MultiDe
         d.val = d.probe = 0;
         d.sec = first_sector<BS / kSec>(key, hidx(key, t.seed[0], t.nbuckets));
         for (bool go = ok; go;) {               // bounded: the sectors of k buckets, each lost claim takes a slot
-            st = sector_pass<64, false>(t.slots, key, 0, d.sec, true);
+            st = sector_pass<64>(t.slots, key, 0, d.sec, true);
             go = st >= kKeyLost;
             if (st == kKeyFull && !advance<BS / kSec, false>(t, d)) {
                 st = spill_put<64>(t, key, 0);
@@ -398,9 +408,10 @@ cudaError_t bucket_find_or_put(const BucketCfg& c, const DevTable& t, const void
                                uint8_t* is_new, void* new_out, unsigned long long* new_count,
                                uint64_t new_cap, cudaStream_t s, const L2Window& w) {
     ProfScope ps(kKBucketFop, s);
+    const bool whole = past_l2(t) || n < kSectorKeys;
 #define L(KW, BS)                                                                                                    \
-    return past_l2(t) ? launch_fop<KW, BS, true>(t, keys, vals, n, d_n, is_new, new_out, new_count, new_cap, s, w)   \
-                      : launch_fop<KW, BS, false>(t, keys, vals, n, d_n, is_new, new_out, new_count, new_cap, s, w);
+    return whole ? launch_fop<KW, BS, true>(t, keys, vals, n, d_n, is_new, new_out, new_count, new_cap, s, w)        \
+                 : launch_fop<KW, BS, false>(t, keys, vals, n, d_n, is_new, new_out, new_count, new_cap, s, w);
 #define X(BS)                                                                                                        \
     if (c.bucket_slots == BS) {                                                                                      \
         if (c.kw == 32) L(32, BS)                                                                                    \
@@ -479,17 +490,12 @@ cudaError_t bfs_fused_level(const BucketCfg& c, const PreparedModel* model, cons
 cudaError_t bucket_lookup(const BucketCfg& c, const DevTable& t, const void* keys, uint64_t n,
                           uint32_t* vals, uint8_t* found, cudaStream_t s, const L2Window& w) {
     ProfScope ps(kKBucketLookup, s);
-#define L(KW, BS)                                                                       \
-    return past_l2(t) ? launch_lookup<KW, BS, true>(t, keys, n, vals, found, s, w)      \
-                      : launch_lookup<KW, BS, false>(t, keys, n, vals, found, s, w);
-#define X(BS)                                                                           \
-    if (c.bucket_slots == BS) {                                                         \
-        if (c.kw == 32) L(32, BS)                                                       \
-        L(64, BS)                                                                       \
-    }
+#define X(BS)                                                                  \
+    if (c.bucket_slots == BS)                                                  \
+        return c.kw == 32 ? launch_lookup<32, BS>(t, keys, n, vals, found, s, w) \
+                          : launch_lookup<64, BS>(t, keys, n, vals, found, s, w);
     HT_BUCKET_CONFIGS(X)
 #undef X
-#undef L
     return cudaErrorInvalidValue;
 }
 

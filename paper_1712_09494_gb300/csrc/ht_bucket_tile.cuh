@@ -75,7 +75,7 @@ __device__ __forceinline__ void load_sectors(const uint64_t* p, bool ok, uint64_
 // trips of one or two (done so, out of line, an L2-resident replay of 10^8 keys
 // took 3.7 ms; now 1.0).
 //
-// sector_pass: one lane per key reads one sector of the key's bucket with one
+// sector_pass: find-or-put; one lane per key reads one sector of the key's bucket with one
 // 256-bit load.  A free slot in a sector ends the search: the key is in no later
 // one.  At load 0.8 a stored key is found after 1.35 sectors on average, so a key
 // costs a third of the words and instructions of a bucket read whole.  Bound by
@@ -86,9 +86,8 @@ __device__ __forceinline__ void load_sectors(const uint64_t* p, bool ok, uint64_
 // for a line), and a second sector is another request that crosses to the other
 // die's L2: fill of 2^27 keys 8.1 ms instead of 8.8, 20 M lookups in 500 MB 522 us
 // instead of 875, BFS of 10^8 states 63 ms instead of 67.
-template <int KW, bool LOOKUP>
-__device__ __forceinline__ uint32_t sector_pass(uint64_t* slots, uint64_t key, uint32_t val, uint64_t sec, bool ok,
-                                                uint32_t* found_val = nullptr) {
+template <int KW>
+__device__ __forceinline__ uint32_t sector_pass(uint64_t* slots, uint64_t key, uint32_t val, uint64_t sec, bool ok) {
     using K = Keys<KW>;
     if (!ok) return kKeyDone;
     uint64_t* p = slots + sec * kSec;
@@ -98,13 +97,10 @@ __device__ __forceinline__ uint32_t sector_pass(uint64_t* slots, uint64_t key, u
     uint32_t e = 0;                         // free slots, slot j in bit j
 #pragma unroll
     for (int j = 0; j < kSec; ++j) {
-        const bool same = K::keyof(w[j]) == key;
-        hit |= same;
-        if (LOOKUP && KW == 32 && same) *found_val = K::value(w[j]);
+        hit |= K::keyof(w[j]) == key;
         // 64-bit keys: only EMPTY has the top bit set.
         e |= (KW == 32 ? uint32_t(K::empty(w[j])) : uint32_t(w[j] >> 63)) << j;
     }
-    if (LOOKUP) return hit ? kKeyHit : e ? kKeyDone : kKeyFull;
     if (hit) return kKeyDone;
     if (!e) return kKeyFull;
     const uint64_t old =
@@ -287,7 +283,7 @@ template <int KW, int BS, bool WHOLE, bool ALL>
 __device__ __forceinline__ uint32_t put_pass(const DevTable& t, Pending& pend, PendEntry& d, bool ok, bool& waits) {
     constexpr int NS = BS / kSec;
     uint32_t st = WHOLE ? bucket_pass<KW, BS, false, ALL>(t.slots, d.key, d.val, d.sec / NS, ok)
-                        : sector_pass<KW, false>(t.slots, d.key, d.val, d.sec, ok);
+                        : sector_pass<KW>(t.slots, d.key, d.val, d.sec, ok);
     waits = st >= kKeyLost;
     if (st == kKeyFull && !advance<NS, WHOLE>(t, d)) {
         st = spill_put<KW>(t, d.key, d.val);
@@ -297,20 +293,19 @@ __device__ __forceinline__ uint32_t put_pass(const DevTable& t, Pending& pend, P
     return st;
 }
 
-// The same for a lookup.  A whole-bucket lookup's next bucket is touched when
-// its key is queued.
-template <int KW, int BS, bool WHOLE>
+// The same for a lookup, a whole bucket a pass; AHEAD: a queued key's next bucket
+// is touched.
+template <int KW, int BS, bool AHEAD>
 __device__ __forceinline__ uint32_t find_pass(const DevTable& t, Pending& pend, PendEntry& d, bool ok, bool& waits,
                                               uint32_t* val) {
     constexpr int NS = BS / kSec;
-    uint32_t st = WHOLE ? bucket_pass<KW, BS, true, false>(t.slots, d.key, 0, d.sec / NS, ok, val)
-                        : sector_pass<KW, true>(t.slots, d.key, 0, d.sec, ok, val);
+    uint32_t st = bucket_pass<KW, BS, true, false>(t.slots, d.key, 0, d.sec / NS, ok, val);
     waits = st == kKeyFull;
-    if (waits && !advance<NS, WHOLE>(t, d)) {
+    if (waits && !advance<NS, true>(t, d)) {
         st = spill_find<KW>(t, d.key, val);
         waits = false;
     }
-    if (WHOLE && waits) touch_l2(t.slots + d.sec / NS * BS);
+    if (AHEAD && waits) touch_l2(t.slots + d.sec / NS * BS);
     pend.push(waits, d);
     return st;
 }

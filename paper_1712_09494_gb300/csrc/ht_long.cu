@@ -15,8 +15,8 @@
 // writes the key's words between its two steps and waits on nothing there.
 // A reader whose tag matches a header waits (bounded) until the header is
 // published, reads it with acquire semantics and then compares the whole
-// key.  Claims go in slot order over the slots read as EMPTY, and a claim's
-// compare-and-swap returns the header's true state, so the slot-order
+// key.  Claims go over the slots read as EMPTY in an order that the digest
+// gives, and a claim's compare-and-swap returns the header's true state, so the
 // argument of the one-word kernels carries over unchanged: a key is claimed
 // in at most one slot, and it sits in bucket h_f only if h_1 .. h_{f-1} were
 // full.
@@ -31,7 +31,7 @@
 // Key-store rows hold the key's words and, for an odd word count, a zero
 // word, so every row is 16-byte aligned and is read and written with 16-byte
 // accesses.
-#include "ht_internal.cuh"
+#include "ht_bucket_tile.cuh"
 
 namespace ht {
 namespace {
@@ -89,20 +89,6 @@ __device__ __forceinline__ bool row_equals(const uint64_t* row, const uint64_t (
     return eq;
 }
 
-__device__ __forceinline__ void write_row(uint64_t* row, const uint64_t (&k)[kLongMaxWords], uint32_t RW) {
-#pragma unroll
-    for (uint32_t j = 0; j < kLongMaxWords; j += 2)
-        if (j < RW) *reinterpret_cast<ulonglong2*>(row + j) = make_ulonglong2(k[j], k[j + 1]);
-}
-
-// Bit p of x (p < 8) to bit 2p.
-__device__ __forceinline__ uint32_t spread8(uint32_t x) {
-    x = (x | (x << 4)) & 0x0F0Fu;
-    x = (x | (x << 2)) & 0x3333u;
-    x = (x | (x << 1)) & 0x5555u;
-    return x;
-}
-
 __device__ __forceinline__ uint64_t ld_acquire(const uint64_t* p) {
     uint64_t v;
     asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
@@ -113,11 +99,34 @@ __device__ __forceinline__ void st_release(uint64_t* p, uint64_t v) {
     asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// The digest of the W words at p, without keeping them.
+__device__ __forceinline__ uint64_t digest_at(const uint64_t* __restrict__ p, uint32_t W, uint64_t mask) {
+    uint64_t h = mix64(0x9E3779B97F4A7C15ull * (W + 1));
+#pragma unroll
+    for (uint32_t j = 0; j < kLongMaxWords; ++j)
+        if (j < W) h = mix64(h ^ __ldg(p + j));
+    return h & mask;
+}
+
+// A key-store row against the W words of an input key, with 16-byte loads of
+// the row (a padding word is not compared).
+__device__ __forceinline__ bool row_is(const uint64_t* row, const uint64_t* __restrict__ key, uint32_t W) {
+    bool eq = true;
+#pragma unroll
+    for (uint32_t j = 0; j < kLongMaxWords; j += 2)
+        if (j < W) {
+            const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(row + j));
+            eq &= v.x == __ldg(key + j);
+            if (j + 1 < W) eq &= v.y == __ldg(key + j + 1);
+        }
+    return eq;
+}
+
 // Bucket scheme: does slot `slot`, whose header carries the key's tag, hold
 // the key?  Waits until the header is published (bounded: after
 // t.spin_limit polls the timeout flag is set and the slot is taken as
 // another key's).
-__device__ bool slot_holds(const DevTable& t, uint64_t slot, const uint64_t (&k)[kLongMaxWords], uint32_t RW) {
+__device__ bool slot_holds(const DevTable& t, uint64_t slot, const uint64_t* __restrict__ key, uint32_t W, uint32_t RW) {
     uint64_t h = ld_acquire(t.slots + slot);
     uint32_t spins = 0;
     while (h & kBusy) {
@@ -128,117 +137,186 @@ __device__ bool slot_holds(const DevTable& t, uint64_t slot, const uint64_t (&k)
         __nanosleep(100);
         h = ld_acquire(t.slots + slot);
     }
-    return row_equals(t.kstore + slot * RW, k, RW);
+    return row_is(t.kstore + slot * RW, key, W);
 }
 
-// Bucket-scheme find-or-put (LOOKUP: lookup).  A warp takes 32 keys, one
-// per lane.  Each round every lane still searching names its bucket h_f, and
-// the warp reads those buckets together: in load j, lanes 8g .. 8g+7 read the
-// eight 16-byte pieces of the bucket of lane 4j+g, so a bucket is one
-// coalesced 128-byte access; ballots hand each owner its 16-bit masks of
-// slots whose tag matches and of EMPTY slots.  The owner then checks the
-// matching slots and, if the key is not there and the bucket has EMPTY
-// slots, claims them in slot order until one claim succeeds or another copy
-// of the key turns up.  A lookup stops at the first bucket with an EMPTY
-// slot.
-enum : int { kSearching = 0, kClaimed = 1, kFound = 2, kAbsent = 3, kIdle = 4 };
+__device__ __forceinline__ void store_sector(uint64_t* p, uint64_t a, uint64_t b, uint64_t c, uint64_t d) {
+    asm volatile("st.global.v4.u64 [%0], {%1,%2,%3,%4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
+}
 
+// The words of an input key to a key-store row (a zero padding word for an
+// odd W), a whole 32-byte sector a store where the row covers one: a sector
+// written in two halves is missed, filled and written twice (fill of 2^25
+// 256-bit keys 4.3 ms; 3.3 with whole sectors).  Rows are 4, 6 or 8 words, those
+// of 6 start in the middle of a sector every second time.
+__device__ __forceinline__ void copy_row(uint64_t* row, const uint64_t* __restrict__ key, uint32_t W, uint32_t RW) {
+    uint64_t k[kLongMaxWords];
+#pragma unroll
+    for (uint32_t j = 0; j < kLongMaxWords; ++j) k[j] = j < W ? __ldg(key + j) : 0;
+    if (reinterpret_cast<uintptr_t>(row) & 31) {
+        *reinterpret_cast<ulonglong2*>(row) = make_ulonglong2(k[0], k[1]);
+        store_sector(row + 2, k[2], k[3], k[4], k[5]);
+    } else {
+        store_sector(row, k[0], k[1], k[2], k[3]);
+        if (RW == 6) *reinterpret_cast<ulonglong2*>(row + 4) = make_ulonglong2(k[4], k[5]);
+        if (RW == 8) store_sector(row + 4, k[4], k[5], k[6], k[7]);
+    }
+}
+
+// The headers of 32 buckets, one per lane (bkt; ok false without one): lane l
+// gets its bucket's slots whose tag matches in bits 0-15 and its EMPTY slots
+// in bits 16-31.  Two lanes read a bucket, 8 headers each with two 256-bit
+// loads, 16 buckets a round; both rounds' reads go out together.
+__device__ __forceinline__ uint32_t read_headers(const uint64_t* slots, uint64_t bkt, uint64_t tag, bool ok) {
+    const int lane = threadIdx.x & 31, grp = lane >> 1, sub = lane & 1;
+    const uint32_t okmask = __ballot_sync(kFullMask, ok);
+    uint64_t w[2][8];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const uint64_t b = __shfl_sync(kFullMask, bkt, q * 16 + grp);
+        bucket::load_sectors<8>(slots + b * kLBS + sub * 8, (okmask >> (q * 16 + grp)) & 1u, w[q]);
+    }
+    uint32_t mine = 0;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const uint64_t ot = __shfl_sync(kFullMask, tag, q * 16 + grp);
+        uint32_t m = 0, e = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            m |= uint32_t((w[q][j] & ~kBusy) == ot) << j;
+            e |= uint32_t(w[q][j] >> 63) << j;             // only EMPTY has the top bit set
+        }
+        const uint32_t x = m | (e << 16);
+        const uint32_t lo = __shfl_sync(kFullMask, x, (lane & 15) * 2), hi = __shfl_sync(kFullMask, x, (lane & 15) * 2 + 1);
+        if ((lane >> 4) == q) mine = lo | (hi << 8);
+    }
+    return ok ? mine : 0u;
+}
+
+// Bucket-scheme find-or-put (LOOKUP: lookup).  A warp takes a fresh tile of 32
+// keys, one per lane, or 32 queued ones, reads one bucket of headers for each
+// and settles what that bucket settles: the owner lane checks the slots whose
+// tag matches, and if the key is not there and the bucket has EMPTY slots claims
+// them, from one that the digest gives around the bucket, until a claim succeeds
+// or another copy of the key turns up.  Keys whose bucket is full wait in the
+// warp's queue for a tile of their own.  A lookup stops at the first bucket with
+// an EMPTY slot, and in a table past L2 (ahead) touches the next tile's headers.
+// A key's words are not kept: only a claim and a tag match read them again (from
+// L1 or L2).  Bound by random lines: the headers', and the row's written or compared.
+constexpr int kLongPend = 64;
+struct LongEntry {
+    uint64_t digest;
+    uint64_t i;        // batch index
+    uint32_t f;        // the hash function to try next
+    uint32_t pad_;
+};
+// (3 blocks per SM: 3.32 ms per fill of 2^25 256-bit keys; 3.36 at 4, 4.33 with
+// eight-lane reads of the buckets and the key's words held in registers, whose
+// lookups ran at 8.4 G/s; now 23.)
 template <bool LOOKUP>
-__global__ void __launch_bounds__(kBlock)
-long_bucket_kernel(const DevTable t, const uint64_t* __restrict__ keys, uint64_t n, uint8_t* __restrict__ out) {
+__global__ void __launch_bounds__(kBlock, 3)
+long_bucket_kernel(const __grid_constant__ DevTable t, const uint64_t* __restrict__ keys, uint64_t n,
+                   uint8_t* __restrict__ out, bool ahead) {
     const uint32_t W = t.words, RW = t.row_words;
     const int lane = threadIdx.x & 31;
-    const uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
-    const uint64_t ntiles = (n + 31) >> 5;
+    const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
+    __shared__ LongEntry s_pend[kBlock / 32][kLongPend];
+    LongEntry* pend = s_pend[threadIdx.x >> 5];
+    uint32_t waiting = 0;
     unsigned long long added = 0;
-    for (uint64_t tile = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; tile < ntiles; tile += nwarps) {
-        const uint64_t i = tile * 32 + lane;
-        const bool act = i < n;
-        uint64_t k[kLongMaxWords];
-        if (act) {
-            load_key(keys, i, W, k);
+    uint64_t base = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) / 32 * 32;
+    // The next tile's digest, ready a tile ahead.
+    uint64_t next_d = base + lane < n ? digest_at(keys + (base + lane) * W, W, t.digest_mask) : 0;
+    // Bounded: an iteration takes a tile or up to 32 queued keys, and a key is
+    // queued at most once for each of its k buckets.
+    for (;;) {
+        LongEntry d;
+        d.digest = d.i = 0;
+        d.f = d.pad_ = 0;
+        bool act;
+        if (waiting >= 32 || (base >= n && waiting)) {
+            const uint32_t m = min(waiting, 32u);
+            act = uint32_t(lane) < m;
+            if (act) d = pend[waiting - m + lane];
+            waiting -= m;
+            __syncwarp();
+        } else if (base < n) {
+            d.i = base + lane;
+            d.digest = next_d;
+            act = d.i < n;
+            base += step;
+            if (base + lane < n) {
+                next_d = digest_at(keys + (base + lane) * W, W, t.digest_mask);
+                if (LOOKUP && ahead) touch_l2(t.slots + hidx(next_d, t.seed[0], t.nbuckets) * kLBS);
+            }
         } else {
-#pragma unroll
-            for (uint32_t j = 0; j < kLongMaxWords; ++j) k[j] = 0;
+            break;
         }
-        const uint64_t d = digest_of(k, W, t.digest_mask);
-        const uint64_t tag = d & kTagMask;
-        int res = act ? kSearching : kIdle;
-        uint32_t f = 0;
-        // Bounded: a searching lane moves to its next function or settles
-        // every round, and there are k functions.
-        while (__any_sync(kFullMask, res == kSearching)) {
-            const int need = res == kSearching;
-            const uint64_t base = need ? hidx(d, t.seed[f], t.nbuckets) * kLBS : 0;
-            ulonglong2 v[8];
-            int on[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int owner = 4 * j + (lane >> 3);
-                const uint64_t ob = __shfl_sync(kFullMask, base, owner);
-                on[j] = __shfl_sync(kFullMask, need, owner);
-                v[j] = make_ulonglong2(0, 0);
-                if (on[j]) v[j] = __ldcg(reinterpret_cast<const ulonglong2*>(t.slots + ob) + (lane & 7));
-            }
-            uint32_t match = 0, empty = 0;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const uint64_t ot = __shfl_sync(kFullMask, tag, 4 * j + (lane >> 3));
-                const bool m0 = on[j] && (v[j].x & ~kBusy) == ot, m1 = on[j] && (v[j].y & ~kBusy) == ot;
-                const bool e0 = on[j] && v[j].x == kEmpty, e1 = on[j] && v[j].y == kEmpty;
-                const uint32_t bm0 = __ballot_sync(kFullMask, m0), bm1 = __ballot_sync(kFullMask, m1);
-                const uint32_t be0 = __ballot_sync(kFullMask, e0), be1 = __ballot_sync(kFullMask, e1);
-                if ((lane >> 2) == j) {
-                    const int sh = 8 * (lane & 3);
-                    match = spread8((bm0 >> sh) & 0xFFu) | (spread8((bm1 >> sh) & 0xFFu) << 1);
-                    empty = spread8((be0 >> sh) & 0xFFu) | (spread8((be1 >> sh) & 0xFFu) << 1);
-                }
-            }
-            if (!need) continue;
-            while (match && res == kSearching) {
-                const int sl = __ffs(match) - 1;
-                match &= match - 1;
-                if (slot_holds(t, base + sl, k, RW)) res = kFound;
-            }
-            if (res == kSearching && empty) {
-                if (LOOKUP) {
-                    res = kAbsent;        // an EMPTY slot: the key would sit in this bucket
-                } else {
-                    while (empty && res == kSearching) {
-                        const int sl = __ffs(empty) - 1;
-                        empty &= empty - 1;
-                        uint64_t* hdr = t.slots + base + sl;
-                        const uint64_t old =
-                            atomicCAS(reinterpret_cast<unsigned long long*>(hdr), kEmpty, tag | kBusy);
-                        if (old == kEmpty) {
-                            write_row(t.kstore + (base + sl) * RW, k, RW);
-                            st_release(hdr, tag);
-                            res = kClaimed;
-                        } else if ((old & ~kBusy) == tag && slot_holds(t, base + sl, k, RW)) {
-                            res = kFound;
-                        }
-                    }
-                }
-            }
-            // Still searching: the bucket is full; the next function, if any.
-            if (res == kSearching && ++f >= t.k) res = kAbsent;
+        const uint64_t tag = d.digest & kTagMask;
+        const uint64_t bkt = hidx(d.digest, t.seed[d.f], t.nbuckets);
+        const uint32_t x = read_headers(t.slots, bkt, tag, act);
+        const uint64_t slot0 = bkt * kLBS;
+        const uint64_t* key = keys + d.i * W;
+        uint32_t match = x & 0xFFFFu, empty = x >> 16;
+        bool found = false, claimed = false;
+        // The first claim of a key without a match goes out before the others'
+        // matches are checked, and these rows' lines are asked for at once.
+        uint64_t old = 0;
+        uint32_t sl = 0;
+        bool sent = !LOOKUP && !match && empty;
+        if (sent) {
+            sl = bucket::first_from<kLBS>(empty, uint32_t(d.digest >> 7) % kLBS);
+            old = atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + slot0 + sl), kEmpty, tag | kBusy);
         }
-        if (!act) continue;
+        if (match) touch_l2(t.kstore + (slot0 + __ffs(match) - 1) * RW);
+        while (match && !found) {
+            const int ms = __ffs(match) - 1;
+            match &= match - 1;
+            found = slot_holds(t, slot0 + ms, key, W, RW);
+        }
+        bool full = act && !found;
         if (LOOKUP) {
-            if (out) out[i] = uint8_t(res == kFound);
+            full &= empty == 0;                    // an EMPTY slot: the key would sit in this bucket
         } else {
-            if (res == kAbsent) {         // all k buckets full
+            while (empty && full) {
+                uint64_t* hdr = t.slots + slot0 + sl;
+                if (!sent) {
+                    sl = bucket::first_from<kLBS>(empty, uint32_t(d.digest >> 7) % kLBS);
+                    hdr = t.slots + slot0 + sl;
+                    old = atomicCAS(reinterpret_cast<unsigned long long*>(hdr), kEmpty, tag | kBusy);
+                }
+                sent = false;
+                empty &= ~(1u << sl);
+                if (old == kEmpty) {
+                    copy_row(t.kstore + (slot0 + sl) * RW, key, W, RW);
+                    st_release(hdr, tag);
+                    claimed = true;
+                    full = false;
+                } else if ((old & ~kBusy) == tag && slot_holds(t, slot0 + sl, key, W, RW)) {
+                    full = false;
+                }
+            }
+        }
+        __syncwarp();
+        // Still searching: the bucket is full; the next function, if any.
+        bool waits = full;
+        if (full && ++d.f >= t.k) {
+            waits = false;
+            if (!LOOKUP) {                         // all k buckets full
                 set_flag(t.ctr, kFlagDropped);
                 atomicAdd(&t.ctr->dropped, 1ull);
             }
-            added += res == kClaimed;
-            if (out) out[i] = uint8_t(res == kClaimed);
         }
+        const uint32_t wm = __ballot_sync(kFullMask, waits);
+        if (wm) {
+            if (waits) pend[waiting + __popc(wm & ((1u << lane) - 1))] = d;
+            waiting += __popc(wm);
+            __syncwarp();
+        }
+        added += claimed;
+        if (act && !waits && out) out[d.i] = uint8_t(LOOKUP ? found : claimed);
     }
-    if (!LOOKUP) {
-        for (int o = 16; o; o >>= 1) added += __shfl_down_sync(kFullMask, added, o);
-        if (lane == 0 && added) atomicAdd(&t.ctr->size, added);
-    }
+    if (!LOOKUP) bucket::add_size<kBlock>(t, added);
 }
 
 // Cuckoo overflow set: linear probing over 16-byte (digest, row) entries.
@@ -286,18 +364,6 @@ struct LongStaged {
     uint64_t spos;
     uint64_t start;
 };
-
-// The words of batch key i to key-store row `row` (a zero padding word for
-// an odd W), with 16-byte stores.
-__device__ __forceinline__ void copy_row(uint64_t* row, const uint64_t* __restrict__ key, uint32_t W, uint32_t RW) {
-#pragma unroll
-    for (uint32_t j = 0; j < kLongMaxWords; j += 2)
-        if (j < RW) {
-            const uint64_t a = __ldg(key + j);
-            const uint64_t b = j + 1 < W ? __ldg(key + j + 1) : 0;
-            *reinterpret_cast<ulonglong2*>(row + j) = make_ulonglong2(a, b);
-        }
-}
 
 template <bool LOOKUP>
 __global__ void __launch_bounds__(kBlock)
@@ -571,7 +637,8 @@ cudaError_t long_find_or_put(const DevTable& t, const void* keys, uint64_t n, ui
     if (!n) return cudaSuccess;
     ProfScope ps(kKBucketFop, s);
     auto k = long_bucket_kernel<false>;
-    k<<<launch_blocks((const void*)k, kBlock), kBlock, 0, s>>>(t, static_cast<const uint64_t*>(keys), n, is_new);
+    k<<<launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s>>>(t, static_cast<const uint64_t*>(keys), n, is_new,
+                                                                       false);
     return cudaGetLastError();
 }
 
@@ -579,7 +646,8 @@ cudaError_t long_lookup(const DevTable& t, const void* keys, uint64_t n, uint8_t
     if (!n) return cudaSuccess;
     ProfScope ps(kKBucketLookup, s);
     auto k = long_bucket_kernel<true>;
-    k<<<launch_blocks((const void*)k, kBlock), kBlock, 0, s>>>(t, static_cast<const uint64_t*>(keys), n, found);
+    k<<<launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s>>>(t, static_cast<const uint64_t*>(keys), n, found,
+                                                                       t.nslots * 8 > l2_bytes());
     return cudaGetLastError();
 }
 

@@ -133,3 +133,22 @@ def test_table_past_l2_at_high_load(kw, bs, lanes):
         want[:first] = vals[:first]
         assert torch.equal(v, want)
     assert t.sync() == 0 and t.size() == n
+
+
+@pytest.mark.parametrize("w", [3, 4, 5, 6, 7, 8])
+@pytest.mark.parametrize("digest_bits", [0, 6])
+def test_nearly_full_table_of_long_keys(w, digest_bits):
+    """Rows of every word count; few digest bits make most matching tags another key's."""
+    n = 960
+    keys = wk.distinct_keys(2 * n, 64 * w, seed=w, shared_prefix=True)
+    rng = np.random.default_rng(w)
+    t = ht.HashTable(1024 if not digest_bits else 4096, "bucket", 64 * w, dict(digest_bits=digest_bits))
+    orc = oracle.OracleTableLong(w)
+    for idx in _batches(np.arange(n), rng) + [rng.permutation(np.tile(np.arange(n), 2))]:
+        got = to_np(t.find_or_put(to_dev(keys[idx])))
+        assert_flags_per_key(idx, got, orc.find_or_put(keys[idx]))
+    found, _ = t.lookup(to_dev(keys))
+    assert np.array_equal(to_np(found), np.repeat(np.array([1, 0], dtype=np.uint8), n))
+    assert t.sync() == 0 and t.size() == n
+    got, _ = t.export()
+    assert set(map(tuple, to_np(got, np.uint64).tolist())) == set(map(tuple, keys[:n].tolist()))
