@@ -23,6 +23,8 @@ struct ht_table {
     ht_status sticky;            // HT_ERR_FULL once a key was dropped
     uint64_t seed_base;
     L2Window win;                // l2_persist: the slots (or the Cuckoo claim set)
+    void* part;                  // scratch of a reordered batch (keys, positions, counters), made on first use
+    size_t part_bytes;
 };
 
 namespace {
@@ -87,10 +89,79 @@ cudaError_t export_any(ht_table* t, void* keys, uint32_t* vals, unsigned long lo
     return table_export(int(t->kw), t->dt, keys, vals, cnt, cap, s);
 }
 
+// Whether a batch of n keys is first reordered by table region, and in how many
+// regions (as bits; 0: no).  Tables past L2 whose 128-byte lines get more than
+// 1.25 keys each from the batch: fewer, and the lines touched twice do not pay
+// for the two passes over the keys (at 0.8 keys per line a 2^22-key batch takes
+// 134 instead of 167 us in region order, and 40 to reorder; at 1.6 a 2^24-key
+// batch 400 instead of 730, and 120 to reorder).  Regions of at most 24 MB: all
+// blocks work on two or three of them at a time.
+int region_bits(const ht_table* t, uint64_t n) {
+    const uint64_t bytes = t->dt.nslots * 8, l2 = l2_bytes();
+    if (!l2 || bytes <= l2 || t->win.bytes || n / 5 * 4 < bytes / 128) return 0;
+    int bits = 1;
+    while (bits < 8 && (bytes >> bits) > (24u << 20)) ++bits;
+    return bits;
+}
+
+// What reordering n keys of ksz bytes needs: counters, the keys, and with
+// answers to bring back (flags) these, the keys' places in their tiles and the
+// tiles' runs.
+struct PartScratch {
+    unsigned int* ctl;
+    char* keys;
+    uint8_t* flags;
+    uint16_t* loc;
+    void* runs;
+    size_t bytes;
+    PartScratch(void* base, uint64_t n, size_t ksz, bool with_flags, int bits) {
+        size_t at = 0;
+        auto carve = [&](size_t sz) {
+            char* p = static_cast<char*>(base) + at;
+            at += (sz + 255) / 256 * 256;
+            return p;
+        };
+        ctl = reinterpret_cast<unsigned int*>(carve(2 * kMaxRegions * sizeof(unsigned int)));
+        keys = carve(n * ksz);
+        flags = nullptr;
+        loc = nullptr;
+        runs = nullptr;
+        if (with_flags) {
+            flags = reinterpret_cast<uint8_t*>(carve(n));
+            loc = reinterpret_cast<uint16_t*>(carve(n * 2));
+            runs = carve(((n + kPartTile - 1) / kPartTile * 8) << bits);
+        }
+        bytes = at;
+    }
+};
+
+// The table keeps one block of that scratch, freed with it, that grows to the
+// largest piece seen.  Null when it cannot be had (no memory, or a stream
+// capture, which must not allocate): the batch then goes in its own order.
+void* part_scratch(ht_table* t, size_t need, cudaStream_t s) {
+    if (t->part_bytes >= need) return t->part;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return nullptr;
+    if (t->part) cudaFreeAsync(t->part, s);
+    t->part = nullptr;
+    t->part_bytes = 0;
+    if (cudaMallocAsync(&t->part, need, s) != cudaSuccess) {
+        cudaGetLastError();                          // not an error of this call
+        t->part = nullptr;
+        return nullptr;
+    }
+    t->part_bytes = need;
+    return t->part;
+}
+
+// Keys of one reordered piece: counters fit 32 bits, and its scratch (190 MB
+// with flags) stays a fraction of a table that wants it.
+constexpr uint64_t kPartPiece = 1ull << 24;
+
 // Runs find-or-put / insert over a batch without touching rebuild state.
 ht_status run_put(ht_table* t, const void* keys, const uint32_t* vals, uint64_t n, uint8_t* is_new,
                   void* new_out, unsigned long long* new_count, cudaStream_t s,
-                  const unsigned long long* d_n = nullptr, uint64_t new_cap = ~0ull) {
+                  const unsigned long long* d_n = nullptr, uint64_t new_cap = ~0ull, uint64_t part_cap = 0) {
     if (n == 0) return HT_OK;
     if (is_long(t->kw)) {
         if (vals || new_out || d_n) return HT_ERR_INVALID;
@@ -120,21 +191,45 @@ ht_status run_put(ht_table* t, const void* keys, const uint32_t* vals, uint64_t 
         }
         return HT_OK;
     }
-    if (t->scheme == HT_BUCKET) {
-        return cuda_status(bucket_find_or_put(bucket_cfg(t), t->dt, keys, vals, n, d_n, is_new, new_out,
-                                              new_count, new_cap, s, t->win));
-    }
     const size_t ksz = t->kw / 8;
-    for (uint64_t off = 0; off < n; off += t->chunk) {
-        const uint64_t m = std::min(t->chunk, n - off);
-        const void* k = static_cast<const char*>(keys) + off * ksz;
-        HT_TRY(cuckoo_probe(int(t->kw), t->dt, t->sc, t->parity, k, vals ? vals + off : nullptr, m, d_n,
-                            off, is_new ? is_new + off : nullptr, s, t->win, new_out != nullptr));
-        HT_TRY(cuckoo_insert(int(t->kw), t->dt, t->sc, t->parity, new_out, new_count, new_cap,
-                             std::min<uint64_t>(m, t->sc.win_cap), s, t->win));
-        t->parity ^= 1u;
+    // One piece in table order: bucket scheme in one launch, Cuckoo in chunks.
+    auto put = [&](const void* k, uint64_t m, const unsigned long long* dn, uint8_t* flags, const uint32_t* v,
+                   bool local) -> ht_status {
+        if (t->scheme == HT_BUCKET)
+            return cuda_status(bucket_find_or_put(bucket_cfg(t), t->dt, k, v, m, dn, flags, new_out, new_count, new_cap,
+                                                  s, t->win, local));
+        for (uint64_t off = 0; off < m; off += t->chunk) {
+            const uint64_t c = std::min(t->chunk, m - off);
+            HT_TRY(cuckoo_probe(int(t->kw), t->dt, t->sc, t->parity, static_cast<const char*>(k) + off * ksz,
+                                v ? v + off : nullptr, c, dn, off, flags ? flags + off : nullptr, s, t->win,
+                                new_out != nullptr, local));
+            HT_TRY(cuckoo_insert(int(t->kw), t->dt, t->sc, t->parity, new_out, new_count, new_cap,
+                                 std::min<uint64_t>(c, t->sc.win_cap), s, t->win));
+            t->parity ^= 1u;
+        }
+        return HT_OK;
+    };
+    if (!vals && (!d_n || n <= part_cap)) {
+        const uint64_t piece = d_n ? n : std::min(n, kPartPiece);
+        const int bits = region_bits(t, d_n ? piece / 2 : piece);   // d_n: about half of the bound
+        void* p = bits ? part_scratch(t, PartScratch(nullptr, piece, ksz, is_new != nullptr, bits).bytes, s) : nullptr;
+        if (p) {
+            const PartScratch ps(p, piece, ksz, is_new != nullptr, bits);
+            uint64_t off = 0;
+            for (; off < n && (d_n || region_bits(t, std::min(piece, n - off))); off += piece) {
+                const uint64_t m = std::min(piece, n - off);
+                HT_TRY(partition_keys(int(t->kw), static_cast<const char*>(keys) + off * ksz, m, d_n, t->dt.seed[0], bits,
+                                      ps.ctl, ps.keys, ps.loc, ps.runs, s));
+                const ht_status st = put(ps.keys, m, d_n, ps.flags, nullptr, true);
+                if (st != HT_OK) return st;
+                if (is_new) HT_TRY(partition_back(ps.flags, ps.loc, ps.runs, bits, m, is_new + off, s));
+            }
+            if (off >= n) return HT_OK;
+            return put(static_cast<const char*>(keys) + off * ksz, n - off, nullptr, is_new ? is_new + off : nullptr,
+                       nullptr, false);              // a last piece too small to be worth it
+        }
     }
-    return HT_OK;
+    return put(keys, n, d_n, is_new, vals, false);
 }
 
 ht_status read_counters(ht_table* t, DevCounters* c, cudaStream_t s) {
@@ -319,7 +414,8 @@ void window_release(int dev) {
 void free_table(ht_table* t, cudaStream_t s) {
     if (!t) return;
     if (t->win.base) window_release(t->device);
-    void* ptrs[] = {t->dt.slots, t->dt.stash, t->dt.ovf, t->dt.ctr, t->sc.set, t->sc.win, t->dt.kstore};
+    void* ptrs[] = {t->dt.slots, t->dt.stash, t->dt.ovf, t->dt.ctr, t->sc.set, t->sc.win, t->dt.kstore,
+                    t->part};
     for (void* p : ptrs)
         if (p) cudaFreeAsync(p, s);
     delete t;
@@ -944,7 +1040,7 @@ static ht_status bfs_common(ht_table* t, const ht_model* h_model, uint64_t s0, u
             HT_TRY(successors(int(t->kw), static_cast<const PreparedModel*>(dm.p), states + c0 * ksz, m, nullptr, 0, succ.p,
                               succ_cap, c + 1, c + 2, s));
             st = run_put(t, succ.p, nullptr, std::min<uint64_t>(succ_cap, m * msucc), nullptr, d_states, c, s, c + 1,
-                         states_cap);
+                         states_cap, succ_cap);
             if (st != HT_OK) return st;
         }
         lo = hi;

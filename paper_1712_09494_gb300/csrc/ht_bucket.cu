@@ -61,14 +61,13 @@ __device__ __forceinline__ void bucket_tiles(const DevTable& t, const void* keys
     // This tile's key and sector, the next tile's key.
     uint64_t key0 = 0, key1 = 0;
     uint32_t val0 = 0, val1 = 0;
-    if (base + lane < n) {
-        key0 = K::load(keys, base + lane);
-        if (VALUES && !LOOKUP) val0 = vals[base + lane];
-    }
-    if (base + step + lane < n) {
-        key1 = K::load(keys, base + step + lane);
-        if (VALUES && !LOOKUP) val1 = vals[base + step + lane];
-    }
+    auto load = [&](uint64_t i, uint64_t& key, uint32_t& val) {
+        if (i >= n) return;
+        key = K::load(keys, i);
+        if (VALUES && !LOOKUP) val = vals[i];
+    };
+    load(base + lane, key0, val0);
+    load(base + step + lane, key1, val1);
     auto start = [&](uint64_t key) { return first_sector<BS / kSec>(key, hidx(key, t.seed[0], t.nbuckets)); };
     uint64_t sec0 = start(key0);
     // Bounded: an iteration takes a tile or up to 32 queued keys, and a key is
@@ -82,21 +81,18 @@ __device__ __forceinline__ void bucket_tiles(const DevTable& t, const void* keys
             mine = ok = pend.pop(d);
         } else if (base < n) {
             d.key = key0;
+            mine = base + lane < n;
             d.pos = base + lane;
             d.sec = sec0;
             d.val = val0;
             d.probe = 0;
-            mine = d.pos < n;
             ok = mine && !K::reserved(d.key);
             if (mine && !ok) set_flag(t.ctr, kFlagInvalidKey);
             key0 = key1;
             val0 = val1;
             sec0 = start(key0);
             if (AHEAD && base + step + lane < n) touch_l2(t.slots + sec0 / (BS / kSec) * BS);
-            if (base + 2 * step + lane < n) {
-                key1 = K::load(keys, base + 2 * step + lane);
-                if (VALUES && !LOOKUP) val1 = vals[base + 2 * step + lane];
-            }
+            load(base + 2 * step + lane, key1, val1);
             base += step;
         } else {
             break;
@@ -158,8 +154,8 @@ cudaError_t launch_fop(const DevTable& t, const void* keys, const uint32_t* vals
     using T = typename Keys<KW>::T;
     auto k = vals ? bucket_fop_kernel<KW, BS, KW == 32, false, WHOLE>
              : new_out ? bucket_fop_kernel<KW, BS, false, true, WHOLE> : bucket_fop_kernel<KW, BS, false, false, WHOLE>;
-    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, keys, vals, n, d_n, is_new,
-                      static_cast<T*>(new_out), new_count, new_cap);
+    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, keys, vals, n, d_n,
+                      is_new, static_cast<T*>(new_out), new_count, new_cap);
 }
 
 template <int KW, int BS>
@@ -406,9 +402,9 @@ bfs_fused_kernel(const PreparedModel* __restrict__ model, const typename Keys<KW
 cudaError_t bucket_find_or_put(const BucketCfg& c, const DevTable& t, const void* keys,
                                const uint32_t* vals, uint64_t n, const unsigned long long* d_n,
                                uint8_t* is_new, void* new_out, unsigned long long* new_count,
-                               uint64_t new_cap, cudaStream_t s, const L2Window& w) {
+                               uint64_t new_cap, cudaStream_t s, const L2Window& w, bool local) {
     ProfScope ps(kKBucketFop, s);
-    const bool whole = past_l2(t) || n < kSectorKeys;
+    const bool whole = !local && (past_l2(t) || n < kSectorKeys);
 #define L(KW, BS)                                                                                                    \
     return whole ? launch_fop<KW, BS, true>(t, keys, vals, n, d_n, is_new, new_out, new_count, new_cap, s, w)        \
                  : launch_fop<KW, BS, false>(t, keys, vals, n, d_n, is_new, new_out, new_count, new_cap, s, w);

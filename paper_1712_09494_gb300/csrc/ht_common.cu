@@ -210,7 +210,7 @@ Prof& prof() {
 const char* kNames[kKNumKernels] = {
     "bucket_find_or_put", "bucket_lookup", "cuckoo_probe", "cuckoo_insert", "cuckoo_lookup",
     "export", "clear", "compact", "probe_random_read", "successors", "probe_random_rmw",
-    "multi_persistent",
+    "multi_persistent", "partition",
 };
 
 }  // namespace
@@ -260,9 +260,23 @@ int launch_blocks(const void* kernel, int block, size_t smem) {
     return grid;
 }
 
-int launch_grid(const void* kernel, int block, uint64_t items, uint64_t per_block) {
+int launch_grid(const void* kernel, int block, uint64_t items, uint64_t per_block, size_t smem) {
     const uint64_t need = items / per_block + (items % per_block != 0);
-    return int(std::min<uint64_t>(uint64_t(launch_blocks(kernel, block)), std::max<uint64_t>(need, 1)));
+    return int(std::min<uint64_t>(uint64_t(launch_blocks(kernel, block, smem)), std::max<uint64_t>(need, 1)));
+}
+
+cudaError_t allow_smem(const void* kernel, size_t smem) {
+    static std::mutex mu;
+    static std::unordered_map<const void*, size_t> done[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> g(mu);
+    size_t& have = done[dev & 63][kernel];
+    if (have >= smem) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e == cudaSuccess) have = smem;
+    return e;
 }
 
 uint64_t l2_bytes() {

@@ -45,56 +45,18 @@
 // the table during the probe and the dedup set elects one winner.  Every
 // winner is thus truly absent and all winners are distinct -- the
 // precondition of Alcantara's insertion.
-#include "ht_internal.cuh"
+#include "ht_bucket_tile.cuh"
 
 namespace ht {
 namespace {
 
-#ifndef HT_CUCKOO_KEYS_PER_THREAD
-#define HT_CUCKOO_KEYS_PER_THREAD 4
+constexpr int kU = 4;                   // eviction chains in flight per thread (insert)
+constexpr int kStage = 96;              // staged winners per warp
+#ifndef HT_CUCKOO_PROBE_BLOCKS
+#define HT_CUCKOO_PROBE_BLOCKS 4
 #endif
-constexpr int kU = HT_CUCKOO_KEYS_PER_THREAD;   // keys in flight per thread
-// Blocks per SM the probe is compiled for: find-or-put holds the CAS
-// results of its U keys besides their probe words (2 blocks, no spills: the
-// fill is 17% faster than at 3 blocks with spills); lookup keeps 3.
-#ifndef HT_CUCKOO_PROBE_MIN_BLOCKS
-#define HT_CUCKOO_PROBE_MIN_BLOCKS 2
-#endif
-#ifndef HT_CUCKOO_LOOKUP_MIN_BLOCKS
-#define HT_CUCKOO_LOOKUP_MIN_BLOCKS 3
-#endif
-// Tables that fit in L2 get a find-or-put probe of kUL2 keys per thread at
-// 3 blocks per SM: their keys are mostly hits served by L2, where more warps
-// hide more latency (a replay of 10^8 keys of multiplicity 1000: 2.04 ms
-// instead of 2.33).  Larger tables keep kU keys at 2 blocks (the 2^27-key
-// fill: 18.7 ms instead of 19.2).
-#ifndef HT_CUCKOO_KEYS_PER_THREAD_L2
-#define HT_CUCKOO_KEYS_PER_THREAD_L2 3
-#endif
-#ifndef HT_CUCKOO_PROBE_L2_MIN_BLOCKS
-#define HT_CUCKOO_PROBE_L2_MIN_BLOCKS 3
-#endif
-constexpr int kUL2 = HT_CUCKOO_KEYS_PER_THREAD_L2;
-#ifndef HT_CUCKOO_INSERT_MIN_BLOCKS
-#define HT_CUCKOO_INSERT_MIN_BLOCKS 3
-#endif
-
-// Probe (and, for find-or-put, the stores and the dedup).  Each thread
-// holds U keys of a round, strided by the grid so every load of keys stays
-// coalesced; all U first probes are issued together, then the remaining
-// probes of the misses, then the misses' CASes, then the dedup claims of
-// the keys that found every slot full, so U memory latencies overlap.  KH bounds
-// the table's k at compile time (4 for the usual k <= 4, else 8): the probe
-// words in flight are held in registers, and sizing them for k <= 4 keeps
-// enough warps resident per SM.
-#ifndef HT_CUCKOO_PROBE_SPLIT
-#define HT_CUCKOO_PROBE_SPLIT 2
-#endif
-#ifndef HT_CUCKOO_DIRECT
-#define HT_CUCKOO_DIRECT 1                     // absent keys CAS themselves into the EMPTY slot they saw
-#endif
-#ifndef HT_CUCKOO_STAGE
-#define HT_CUCKOO_STAGE 128                    // staged winners per warp
+#ifndef HT_CUCKOO_LOOKUP_BLOCKS
+#define HT_CUCKOO_LOOKUP_BLOCKS 5
 #endif
 
 // Adds the block's per-warp sums (held by each warp's lane 0) to N table
@@ -136,10 +98,24 @@ struct StagedWinner {
     uint32_t start;
 };
 
-template <int KW, bool VALUES, bool LOOKUP, int KH, int U = kU>
-__global__ void __launch_bounds__(kBlock, KH > 4 ? 1 : LOOKUP ? HT_CUCKOO_LOOKUP_MIN_BLOCKS
-                                          : U == kU ? HT_CUCKOO_PROBE_MIN_BLOCKS : HT_CUCKOO_PROBE_L2_MIN_BLOCKS)
-cuckoo_probe_kernel(const DevTable t, const DevScratch sc, uint32_t parity,
+// All k slots (or one past h_1) seen without the key: the stash and overflow
+// set, when in use.  Out of line: rare.
+template <int KW>
+__device__ __noinline__ bool spill_holds(const DevTable& t, uint64_t key, uint32_t stash_used, uint32_t ovf_used,
+                                         uint64_t* w) {
+    return find_spill<KW>(t, key, stash_used, ovf_used, w);
+}
+
+// Probe (and, for find-or-put, the stores and the dedup).  One lane per key; a
+// pass reads one slot, h_(a+1), for each key of a tile of 32 fresh keys or of 32
+// that wait in the warp's queue (bucket::Pending) for their next slot: every
+// lane of a pass has a slot to read, whatever the other keys' paths.  A key is
+// settled by the slot that holds it or by the first EMPTY one (a key never sits
+// past an empty slot of its own), 1.63 slots per key over a fill to load 0.8.
+// AHEAD: tables past L2; the next tile's first slots are touched a tile ahead.
+template <int KW, bool VALUES, bool LOOKUP, bool AHEAD>
+__global__ void __launch_bounds__(kBlock, LOOKUP ? HT_CUCKOO_LOOKUP_BLOCKS : HT_CUCKOO_PROBE_BLOCKS)
+cuckoo_probe_kernel(const __grid_constant__ DevTable t, const __grid_constant__ DevScratch sc, uint32_t parity,
                     const void* __restrict__ keys, const uint32_t* __restrict__ vals, uint64_t n,
                     const unsigned long long* __restrict__ d_n, uint64_t off,
                     uint8_t* __restrict__ out_flag, uint32_t* __restrict__ out_val, bool list_stored) {
@@ -150,18 +126,17 @@ cuckoo_probe_kernel(const DevTable t, const DevScratch sc, uint32_t parity,
     }
     const uint32_t stash_used = __ldcg(&t.ctr->stash_used);
     const uint32_t ovf_used = __ldcg(&t.ctr->ovf_used);
-    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-    const uint64_t tid = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    const uint64_t rounds = (n + stride * U - 1) / (stride * U);     // warp-uniform trip count
+    const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
     const uint64_t dseed = t.aux_seed * 3 + 1;
     const int lane = threadIdx.x & 31;
-    unsigned long long probes = 0;            // slots read (h_1, then h_2..h_k if h_1 is occupied)
+    unsigned long long probes = 0;            // slots read
     unsigned long long misses = 0, miss_reads = 0;   // keys found nowhere, and the slots they read
     unsigned long long direct = 0;            // CASes of absent keys into table slots
     unsigned long long stored = 0;            // keys stored here and not listed
-    constexpr int kStage = LOOKUP ? 1 : HT_CUCKOO_STAGE;
-    __shared__ StagedWinner s_win[kBlock / 32][kStage];
-    StagedWinner* stage = s_win[threadIdx.x >> 5];
+    __shared__ StagedWinner s_win[LOOKUP ? 1 : kBlock / 32][LOOKUP ? 1 : kStage];
+    __shared__ bucket::PendEntry s_pend[kBlock / 32][bucket::kPend];
+    StagedWinner* stage = s_win[LOOKUP ? 0 : (threadIdx.x >> 5)];
+    bucket::Pending queue(s_pend[threadIdx.x >> 5]);
     uint32_t pend = 0;
     // Lists the staged winners: one atomic on the winner count per flush.
     // Entries past the list's capacity (more winners than the table holds)
@@ -195,248 +170,151 @@ cuckoo_probe_kernel(const DevTable t, const DevScratch sc, uint32_t parity,
         __syncwarp();
         pend = 0;
     };
-    // The next round's keys are loaded while this round waits on the table.
-    uint64_t next_key[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const uint64_t i = uint64_t(u) * stride + tid;
-        next_key[u] = i < n ? K::load(keys, i) : 0;
-    }
-    for (uint64_t r = 0; r < rounds; ++r) {
-        uint64_t key[U], w[U];
-        bool act[U], found[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint64_t i = (r * U + u) * stride + tid;
-            act[u] = i < n;
-            key[u] = next_key[u];
-            const uint64_t j = ((r + 1) * U + u) * stride + tid;
-            if (j < n) next_key[u] = K::load(keys, j);
-            if (act[u] && K::reserved(key[u])) {
-                set_flag(t.ctr, kFlagInvalidKey);
-                act[u] = false;
-            }
-        }
-        // Section 4.1: a key is found in at most k probes; h_1 first.
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (act[u]) w[u] = __ldcg(reinterpret_cast<const unsigned long long*>(t.slots + hidx(key[u], t.seed[0], t.nslots)));
-        // An empty h_1 slot ends the table probe: a key stored at h_j has
-        // h_1 .. h_{j-1} all occupied (see the top of this file).  A miss at
-        // table load a then costs 1 + a (k - 1) probes, not k.
-        bool more[U], occ1[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            found[u] = act[u] && K::keyof(w[u]) == key[u];
-            more[u] = act[u] && !found[u] && !K::empty(w[u]);
-            occ1[u] = more[u];
-            probes += act[u] ? 1u : 0u;
-        }
-        // The chain start of a miss: the first of h_2..h_k seen EMPTY (0 =
-        // h_1: empty, or every slot occupied).
-        uint32_t start[U];
-        uint64_t ws[U][KH];
-#pragma unroll
-        for (int u = 0; u < U; ++u) start[u] = 0;
-        // h_2..h_k in groups [a0, a1): the slots of a group are read together,
-        // and a key goes on to the next group only while it is neither found
-        // nor past an EMPTY slot (a key never sits past an empty slot of its
-        // own).  HT_CUCKOO_PROBE_SPLIT: 0 one group; 1 h_2, then the rest;
-        // 2 (default) one slot at a time.  The probe is bound by the random
-        // lines it reads, not by its round trips: one slot at a time reads
-        // 1.63 slots per key over a fill to load 0.8 instead of 2.06, and a
-        // launch takes 0.141 instead of 0.157 ms.
-        auto probe_group = [&](int a0, int a1) {
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-#pragma unroll
-                for (int a = 1; a < KH; ++a)
-                    if (a >= a0 && a < a1 && a < int(t.k) && more[u]) {
-                        ws[u][a] = __ldcg(reinterpret_cast<const unsigned long long*>(t.slots + hidx(key[u], t.seed[a], t.nslots)));
-                        ++probes;
-                    }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (!more[u]) continue;
-#pragma unroll
-                for (int a = KH - 1; a >= 1; --a)
-                    if (a >= a0 && a < a1 && a < int(t.k)) {
-                        if (K::keyof(ws[u][a]) == key[u]) {
-                            found[u] = true;
-                            w[u] = ws[u][a];
-                        }
-                        if (K::empty(ws[u][a])) start[u] = uint32_t(a);
-                    }
-                more[u] = !found[u] && start[u] == 0;
-            }
-        };
-        if (HT_CUCKOO_PROBE_SPLIT == 0) {
-            probe_group(1, KH);
-        } else if (HT_CUCKOO_PROBE_SPLIT == 1) {
-            probe_group(1, 2);
-            bool any = false;
-#pragma unroll
-            for (int u = 0; u < U; ++u) any |= more[u];
-            if (__any_sync(0xFFFFFFFFu, any)) probe_group(2, KH);
+    uint64_t base = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) / 32 * 32;
+    // This tile's key and slot, the next tile's key.
+    uint64_t key0 = 0, key1 = 0;
+    if (base + lane < n) key0 = K::load(keys, base + lane);
+    if (base + step + lane < n) key1 = K::load(keys, base + step + lane);
+    uint64_t slot0 = hidx(key0, t.seed[0], t.nslots);
+    // Bounded: an iteration takes a tile or up to 32 queued keys, and a key is
+    // queued at most k - 1 times.
+    for (;;) {
+        bucket::PendEntry d;
+        d.val = 0;
+        uint64_t at;
+        bool mine, ok;
+        if (queue.n >= 32 || (base >= n && queue.n)) {
+            d.key = d.pos = 0;
+            d.probe = 0;
+            mine = ok = queue.pop(d);
+            at = hidx(d.key, t.seed[d.probe], t.nslots);
+        } else if (base < n) {
+            d.key = key0;
+            d.pos = base + lane;
+            mine = d.pos < n;
+            d.probe = 0;
+            at = slot0;
+            ok = mine && !K::reserved(d.key);
+            if (mine && !ok) set_flag(t.ctr, kFlagInvalidKey);
+            key0 = key1;
+            slot0 = hidx(key0, t.seed[0], t.nslots);
+            if (AHEAD && base + step + lane < n) touch_l2(t.slots + slot0);
+            if (base + 2 * step + lane < n) key1 = K::load(keys, base + 2 * step + lane);
+            base += step;
         } else {
-#pragma unroll
-            for (int a = 1; a < KH; ++a) {
-                bool any = false;
-#pragma unroll
-                for (int u = 0; u < U; ++u) any |= more[u];
-                if (a < int(t.k) && __any_sync(0xFFFFFFFFu, any)) probe_group(a, a + 1);
-            }
+            break;
         }
-        if (stash_used | ovf_used) {
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (act[u] && !found[u]) found[u] = find_spill<KW>(t, key[u], stash_used, ovf_used, &w[u]);
+        uint64_t w = kEmpty;
+        if (ok) w = __ldcg(reinterpret_cast<const unsigned long long*>(t.slots + at));
+        probes += ok;
+        bool found = ok && K::keyof(w) == d.key;
+        bool miss = ok && !found && (K::empty(w) || d.probe + 1 >= t.k);
+        const bool waits = ok && !found && !miss;
+        if (miss && (stash_used | ovf_used) && spill_holds<KW>(t, d.key, stash_used, ovf_used, &w)) {
+            found = true;
+            miss = false;
         }
-        // The slots read by the keys found nowhere (the table counters keep
-        // them apart from the hits' reads; find-or-put only -- counting them
-        // costs a lookup registers it spills).
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (!LOOKUP && act[u] && !found[u]) {
-                ++misses;
-                const uint32_t k = t.k;
-                miss_reads += !occ1[u] ? 1u
-                              : HT_CUCKOO_PROBE_SPLIT == 0 ? k
-                              : HT_CUCKOO_PROBE_SPLIT == 1 ? (start[u] == 1 ? 2u : k)
-                                                           : (start[u] ? 1u + start[u] : k);
-            }
+        if (waits) ++d.probe;
+        queue.push(waits, d);
         if constexpr (LOOKUP) {
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const uint64_t i = (r * U + u) * stride + tid;
-                if (i < n) {
-                    if (out_flag) out_flag[i] = uint8_t(found[u]);
-                    if (out_val) out_val[i] = found[u] ? K::value(w[u]) : 0u;
-                }
+            if (mine && !waits) {
+                if (out_flag) out_flag[d.pos] = uint8_t(found);
+                if (out_val) out_val[d.pos] = found ? K::value(w) : 0u;
             }
         } else {
+            if (miss) {
+                ++misses;
+                miss_reads += d.probe + 1;
+            }
             // A miss that saw an EMPTY slot stores itself there with a CAS
             // from EMPTY, trying its slots in order from that one: a CAS that
             // returns the key means another copy stored it first (not new);
             // one that returns another key moves on to the next slot, which
             // the CAS reads as well.  This is the bucket scheme's claim in
-            // slot order (Section 4.2), over h_a..h_k.  Nothing leaves a slot
+            // a fixed order (Section 4.2), over h_a..h_k.  Nothing leaves a slot
             // during the probe kernel, so a key is stored in at most one slot
             // and every copy probed later finds it; a copy that saw all k
-            // slots full read them after they were full, so no copy stores
+            // slots full read each after it was full, so no copy stores
             // it in the table here.  With t.chain_h1 only an EMPTY h_1 is
             // tried (Section 4.1 starts every insertion at h_1).
-            bool placed[U], claim[U], pend_cas[U];
-            uint32_t at[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const bool miss = act[u] && !found[u];
-                at[u] = occ1[u] ? start[u] : 0u;
-                pend_cas[u] = HT_CUCKOO_DIRECT && miss && (!occ1[u] || (start[u] != 0 && !t.chain_h1));
-                claim[u] = miss && !pend_cas[u];
-                placed[u] = false;
-            }
-#pragma unroll
-            for (int pass = 0; pass < KH; ++pass) {
-                bool any = false;
-#pragma unroll
-                for (int u = 0; u < U; ++u) any |= pend_cas[u];
-                if (!__any_sync(0xFFFFFFFFu, any)) break;
-                uint64_t cw[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (pend_cas[u]) {
-                        const uint64_t i = (r * U + u) * stride + tid;
-                        cw[u] = atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + hidx(key[u], t.seed[at[u]], t.nslots)),
-                                          kEmpty, K::word(key[u], VALUES ? vals[i] : 0u));
-                        ++direct;
-                    }
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    if (!pend_cas[u]) continue;
-                    if (cw[u] == kEmpty) {
-                        placed[u] = true;
-                        pend_cas[u] = false;
-                    } else if (K::keyof(cw[u]) == key[u]) {
-                        pend_cas[u] = false;                   // another copy stored it
-                    } else if (t.chain_h1 || at[u] + 1 >= t.k) {
-                        claim[u] = true;                       // every slot is full now
-                        pend_cas[u] = false;
-                    } else {
-                        ++at[u];
-                    }
+            bool placed = false;
+            bool cas = miss && K::empty(w) && (!t.chain_h1 || d.probe == 0);
+            bool claim = miss && !cas;
+            while (cas) {                          // bounded: on to the next of k slots
+                const uint64_t cw = atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + at), kEmpty,
+                                              K::word(d.key, VALUES ? vals[d.pos] : 0u));
+                ++direct;
+                cas = false;
+                if (cw == kEmpty) {
+                    placed = true;
+                } else if (K::keyof(cw) == d.key) {
+                    // another copy stored it
+                } else if (t.chain_h1 || d.probe + 1 >= t.k) {
+                    claim = true;                  // every slot is full now
+                } else {
+                    ++d.probe;
+                    at = hidx(d.key, t.seed[d.probe], t.nslots);
+                    cas = true;
                 }
             }
+            __syncwarp();
             // The misses that found all k slots full go through the claim
             // set: the one claimant of each such key wins and runs an
             // eviction chain from h_1 in the insert kernel.  Each CASes its
             // key into its slot of the claim set (kept in L2); a slot holding
             // another key sends it on by linear probing.
-            uint32_t spos[U];
-            uint64_t sw[U];
-            bool winner[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                spos[u] = uint32_t(mix64(key[u] ^ dseed) & sc.mask);
-                sw[u] = kEmpty;
-                if (claim[u]) sw[u] = atomicCAS(reinterpret_cast<unsigned long long*>(sc.set + spos[u]), kEmpty, key[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                winner[u] = placed[u];
-                if (!claim[u]) continue;
-                if (sw[u] == kEmpty) {
-                    winner[u] = true;                          // our CAS filled the empty slot
-                } else if (K::keyof(sw[u]) != key[u]) {        // another key sits there: probe on
-                    uint32_t sat = 0;
-                    const uint32_t next = spos[u] + 1 == uint32_t(sc.mask + 1) ? 0u : spos[u] + 1;
-                    const int rc = lp_insert<KW>(sc.set, uint32_t(sc.mask + 1), next, key[u], key[u], &sat);
-                    winner[u] = rc == 1;
-                    spos[u] = sat;
-                    if (rc < 0) {                              // more distinct misses than the table holds
-                        set_flag(t.ctr, kFlagDropped);
-                        atomicAdd(&t.ctr->dropped, 1ull);
-                    }
+            bool winner = placed;
+            uint32_t spos = 0;
+            if (claim) {
+                const int rc = lp_insert<KW>(sc.set, uint32_t(sc.mask + 1), mix64(d.key ^ dseed) & sc.mask, d.key, d.key,
+                                             &spos);
+                winner = rc == 1;
+                if (rc < 0) {                      // more distinct misses than the table holds
+                    set_flag(t.ctr, kFlagDropped);
+                    atomicAdd(&t.ctr->dropped, 1ull);
                 }
             }
-            // The round's winners go to the warp's stage in shared memory,
-            // listed with one atomic per flush rather than one per round, so
-            // the next round does not wait on a shared counter.  Keys this
-            // kernel stored are listed only for a caller that appends the new
-            // keys (list_stored); otherwise they are just counted.
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const uint64_t i = (r * U + u) * stride + tid;
-                const bool listed = winner[u] && (list_stored || !placed[u]);
-                stored += (placed[u] && !list_stored) ? 1u : 0u;
-                const unsigned wm = __ballot_sync(0xFFFFFFFFu, listed);
-                if (wm) {
-                    if (pend + __popc(wm) > uint32_t(kStage)) flush();
-                    if (listed) {
-                        StagedWinner& e = stage[pend + __popc(wm & ((1u << lane) - 1))];
-                        e.word = K::word(key[u], VALUES ? vals[i] : 0u);
-                        e.i = i;
-                        e.spos = spos[u];
-                        e.start = placed[u] ? kStartPlaced : (HT_CUCKOO_DIRECT || t.chain_h1) ? 0u : start[u];
-                    }
-                    pend += __popc(wm);
+            if (mine && !waits && out_flag) out_flag[d.pos] = uint8_t(winner);
+            // Winners go to the warp's stage in shared memory, listed with one
+            // atomic per flush, so that no pass waits on a shared counter.
+            // Keys this kernel stored are listed only for a caller that appends
+            // the new keys (list_stored); otherwise they are just counted.
+            const bool listed = winner && (list_stored || !placed);
+            stored += placed && !list_stored;
+            const unsigned wm = __ballot_sync(0xFFFFFFFFu, listed);
+            if (wm) {
+                if (pend + __popc(wm) > uint32_t(kStage)) flush();
+                if (listed) {
+                    StagedWinner& e = stage[pend + __popc(wm & ((1u << lane) - 1))];
+                    e.word = K::word(d.key, VALUES ? vals[d.pos] : 0u);
+                    e.i = d.pos;
+                    e.spos = spos;
+                    e.start = placed ? kStartPlaced : 0u;
                 }
-                if (i < n && out_flag) out_flag[i] = uint8_t(winner[u]);
+                pend += __popc(wm);
             }
         }
     }
     if constexpr (!LOOKUP) flush();
     for (int o = 16; o; o >>= 1) {
         probes += __shfl_down_sync(0xFFFFFFFFu, probes, o);
-        misses += __shfl_down_sync(0xFFFFFFFFu, misses, o);
-        miss_reads += __shfl_down_sync(0xFFFFFFFFu, miss_reads, o);
-        direct += __shfl_down_sync(0xFFFFFFFFu, direct, o);
-        stored += __shfl_down_sync(0xFFFFFFFFu, stored, o);
+        if (!LOOKUP) {
+            misses += __shfl_down_sync(0xFFFFFFFFu, misses, o);
+            miss_reads += __shfl_down_sync(0xFFFFFFFFu, miss_reads, o);
+            direct += __shfl_down_sync(0xFFFFFFFFu, direct, o);
+            stored += __shfl_down_sync(0xFFFFFFFFu, stored, o);
+        }
     }
-    unsigned long long* const dst[5] = {&t.ctr->size, &t.ctr->probes, &t.ctr->probe_cas, &t.ctr->probe_misses,
-                                        &t.ctr->probe_miss_reads};
-    const unsigned long long sums[5] = {stored, probes, direct, misses, miss_reads};
-    block_add_counters<5>(dst, sums);
+    if constexpr (LOOKUP) {
+        unsigned long long* const dst[1] = {&t.ctr->probes};
+        const unsigned long long sums[1] = {probes};
+        block_add_counters<1>(dst, sums);
+    } else {
+        unsigned long long* const dst[5] = {&t.ctr->size, &t.ctr->probes, &t.ctr->probe_cas, &t.ctr->probe_misses,
+                                            &t.ctr->probe_miss_reads};
+        const unsigned long long sums[5] = {stored, probes, direct, misses, miss_reads};
+        block_add_counters<5>(dst, sums);
+    }
 }
 
 // Eviction-chain insert of the winners.  Each thread keeps U chains in
@@ -448,7 +326,7 @@ cuckoo_probe_kernel(const DevTable t, const DevScratch sc, uint32_t parity,
 // live chains' exchanges.  A record of a key the probe stored (listed only
 // for a caller that collects the new keys) holds no claim and is counted.
 template <int KW, bool APPEND>
-__global__ void __launch_bounds__(kBlock, HT_CUCKOO_INSERT_MIN_BLOCKS)
+__global__ void __launch_bounds__(kBlock, 3)
 cuckoo_insert_kernel(const DevTable t, const DevScratch sc, uint32_t parity, uint64_t max_winners,
                      typename Keys<KW>::T* __restrict__ new_out, unsigned long long* __restrict__ new_count,
                      uint64_t new_cap) {
@@ -568,15 +446,14 @@ cuckoo_insert_kernel(const DevTable t, const DevScratch sc, uint32_t parity, uin
 cudaError_t cuckoo_probe(int kw, const DevTable& t, const DevScratch& sc, uint32_t parity,
                          const void* keys, const uint32_t* vals, uint64_t n,
                          const unsigned long long* d_n, uint64_t off, uint8_t* is_new, cudaStream_t s,
-                         const L2Window& w, bool list_stored) {
+                         const L2Window& w, bool list_stored, bool local) {
     ProfScope ps(kKCuckooProbe, s);
-    const bool in_l2 = t.nslots * 8 <= l2_bytes();
+    const bool past_l2 = !local && t.nslots * 8 > l2_bytes();
 #define L(KW, V)                                                                                        \
     {                                                                                                   \
-        auto k = t.k > 4 ? cuckoo_probe_kernel<KW, V, false, kMaxCuckooHashes>                          \
-                 : in_l2 ? cuckoo_probe_kernel<KW, V, false, 4, kUL2> : cuckoo_probe_kernel<KW, V, false, 4>; \
-        return launch_win(k, launch_blocks((const void*)k, kBlock), kBlock, s, w, t, sc, parity, keys, vals, n, \
-                          d_n, off, is_new, (uint32_t*)nullptr, list_stored);                           \
+        auto k = past_l2 ? cuckoo_probe_kernel<KW, V, false, true> : cuckoo_probe_kernel<KW, V, false, false>; \
+        return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, sc, parity, keys, vals, \
+                          n, d_n, off, is_new, (uint32_t*)nullptr, list_stored);                        \
     }
     if (kw == 32) {
         if (vals) L(32, true) else L(32, false)
@@ -607,16 +484,18 @@ cudaError_t cuckoo_lookup(int kw, const DevTable& t, const void* keys, uint64_t 
                           uint8_t* found, cudaStream_t s, const L2Window& w) {
     ProfScope ps(kKCuckooLookup, s);
     DevScratch none{};
-    if (kw == 32) {
-        auto k = t.k <= 4 ? cuckoo_probe_kernel<32, false, true, 4> : cuckoo_probe_kernel<32, false, true, kMaxCuckooHashes>;
-        return launch_win(k, launch_blocks((const void*)k, kBlock), kBlock, s, w, t, none, 0u, keys,
-                          (const uint32_t*)nullptr, n, (const unsigned long long*)nullptr, uint64_t(0), found, vals,
-                          false);
+    const bool past_l2 = t.nslots * 8 > l2_bytes();
+#define L(KW)                                                                                           \
+    {                                                                                                   \
+        auto k = past_l2 ? cuckoo_probe_kernel<KW, false, true, true> : cuckoo_probe_kernel<KW, false, true, false>; \
+        return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, none, 0u, keys, \
+                          (const uint32_t*)nullptr, n, (const unsigned long long*)nullptr,              \
+                          uint64_t(0), found, vals,                                                     \
+                          false);                                                                       \
     }
-    auto k = t.k <= 4 ? cuckoo_probe_kernel<64, false, true, 4> : cuckoo_probe_kernel<64, false, true, kMaxCuckooHashes>;
-    return launch_win(k, launch_blocks((const void*)k, kBlock), kBlock, s, w, t, none, 0u, keys,
-                      (const uint32_t*)nullptr, n, (const unsigned long long*)nullptr, uint64_t(0), found, vals,
-                      false);
+    if (kw == 32) L(32)
+    L(64)
+#undef L
 }
 
 }  // namespace ht

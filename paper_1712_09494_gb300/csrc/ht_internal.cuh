@@ -321,6 +321,7 @@ enum KernelId : uint32_t {
     kKSuccessors,
     kKProbeRmw,
     kKMultiPersistent,
+    kKPartition,
     kKNumKernels
 };
 
@@ -336,7 +337,9 @@ int launch_blocks(const void* kernel, int block, size_t smem = 0);
 // The grid of a kernel whose blocks take `per_block` work items at a time: the
 // resident blocks, or fewer where `items` needs fewer (blocks without work
 // cost a small call its launch and end).
-int launch_grid(const void* kernel, int block, uint64_t items, uint64_t per_block);
+int launch_grid(const void* kernel, int block, uint64_t items, uint64_t per_block, size_t smem = 0);
+// Lets a kernel use `smem` bytes of dynamic shared memory (set once per device).
+cudaError_t allow_smem(const void* kernel, size_t smem);
 // The current device's L2 size in bytes (0 if unknown).
 uint64_t l2_bytes();
 
@@ -389,10 +392,12 @@ struct BucketCfg {
 };
 
 // d_n (nullable): the batch size lives on the device; n is then an upper bound.
+// local: the keys come in the order of the table's regions (partition_keys).
 cudaError_t bucket_find_or_put(const BucketCfg& c, const DevTable& t, const void* keys,
                                const uint32_t* vals, uint64_t n, const unsigned long long* d_n,
                                uint8_t* is_new, void* new_out, unsigned long long* new_count,
-                               uint64_t new_cap, cudaStream_t s, const L2Window& w = L2Window());
+                               uint64_t new_cap, cudaStream_t s, const L2Window& w = L2Window(),
+                               bool local = false);
 cudaError_t bucket_lookup(const BucketCfg& c, const DevTable& t, const void* keys, uint64_t n,
                           uint32_t* vals, uint8_t* found, cudaStream_t s, const L2Window& w = L2Window());
 
@@ -402,12 +407,24 @@ cudaError_t bucket_lookup(const BucketCfg& c, const DevTable& t, const void* key
 cudaError_t cuckoo_probe(int kw, const DevTable& t, const DevScratch& sc, uint32_t parity,
                          const void* keys, const uint32_t* vals, uint64_t n,
                          const unsigned long long* d_n, uint64_t off, uint8_t* is_new,
-                         cudaStream_t s, const L2Window& w = L2Window(), bool list_stored = true);
+                         cudaStream_t s, const L2Window& w = L2Window(), bool list_stored = true,
+                         bool local = false);
 cudaError_t cuckoo_insert(int kw, const DevTable& t, const DevScratch& sc, uint32_t parity,
                           void* new_out, unsigned long long* new_count, uint64_t new_cap,
                           uint64_t max_winners, cudaStream_t s, const L2Window& w = L2Window());
 cudaError_t cuckoo_lookup(int kw, const DevTable& t, const void* keys, uint64_t n,
                           uint32_t* vals, uint8_t* found, cudaStream_t s, const L2Window& w = L2Window());
+
+// Reorders n (or *d_n) 32- or 64-bit keys by the top `bits` of their first hash
+// (mix64 of key xor seed) into out.  ctl: 2 * kMaxRegions words of scratch.  loc
+// (nullable; n places) and runs (8 << bits bytes per kPartTile keys) keep what
+// partition_back needs to bring one byte per key back to the batch's order.
+constexpr int kMaxRegions = 256;
+constexpr uint64_t kPartTile = 4096;
+cudaError_t partition_keys(int kw, const void* keys, uint64_t n, const unsigned long long* d_n, uint64_t seed, int bits,
+                           unsigned int* ctl, void* out, uint16_t* loc, void* runs, cudaStream_t s);
+cudaError_t partition_back(const uint8_t* from, const uint16_t* loc, const void* runs, int bits, uint64_t n, uint8_t* to,
+                           cudaStream_t s);
 
 cudaError_t table_export(int kw, const DevTable& t, void* keys_out, uint32_t* vals_out,
                          unsigned long long* count, uint64_t cap, cudaStream_t s);

@@ -152,3 +152,53 @@ def test_nearly_full_table_of_long_keys(w, digest_bits):
     assert t.sync() == 0 and t.size() == n
     got, _ = t.export()
     assert set(map(tuple, to_np(got, np.uint64).tolist())) == set(map(tuple, keys[:n].tolist()))
+
+
+@pytest.mark.parametrize("scheme", ["bucket", "cuckoo"])
+@pytest.mark.parametrize("kw", [32, 64])
+def test_large_batches_are_reordered_by_table_region(scheme, kw):
+    """Batches with more keys than the table (past L2) has lines, taken region by region: whole pieces of 2^24 keys
+    with a ragged one after them, batches with and without flags, appended keys, repeats in other batches, and an
+    odd flag address."""
+    from workloads import device_keys as dk
+    slots = 24_000_000                                  # 192 MB: 1.5 M lines
+    n = int(slots * 0.85)
+    idx = torch.arange(2 * n, dtype=torch.int64, device="cuda")
+    if kw == 64:
+        keys = dk.mix63_perm_dev(idx, 3)
+    else:
+        k = dk.mix32_perm_dev(idx, 3)
+        keys = (k - ((k >> 31) << 32)).to(torch.int32)
+    t = ht.HashTable(slots, scheme, kw)
+    order = torch.randperm(n, device="cuda")
+    first = keys[:n][order][:2_000_001]                 # a ragged tile
+    flags = torch.full((len(first) + 8,), 7, dtype=torch.uint8, device="cuda")
+    ht.ht_find_or_put(t.handle, first, flags[3:3 + len(first)])
+    assert bool((flags[3:3 + len(first)] == 1).all()) and flags[:3].tolist() == [7] * 3
+    assert flags[3 + len(first):].tolist() == [7] * 5
+    t.insert(keys[:n][order][1_000_000:5_000_000])      # no flags
+    every = torch.randperm(n, device="cuda")            # n > 2^24: a whole piece and the rest
+    new = torch.empty(n, dtype=torch.uint8, device="cuda")
+    out = torch.empty(n, dtype=keys.dtype, device="cuda")
+    count = torch.zeros(1, dtype=torch.int64, device="cuda")
+    ht.ht_find_or_put_append(t.handle, keys[:n][every], out, count, new)
+    stored = torch.zeros(n, dtype=torch.bool, device="cuda")
+    stored[order[:5_000_000]] = True
+    assert torch.equal(new, (~stored[every]).to(torch.uint8))
+    assert int(count) == n - 5_000_000
+    assert torch.equal(torch.sort(out[:int(count)])[0], torch.sort(keys[:n][~stored])[0])
+    found, _ = t.lookup(keys)
+    assert torch.equal(found, (idx < n).to(torch.uint8))
+    assert t.sync() == 0 and t.size() == n
+
+
+def test_reordered_batch_of_one_key_and_reserved_keys():
+    """Every key in one region, and reserved keys among them: skipped and reported."""
+    t = ht.HashTable(24_000_000, "bucket", 64)
+    keys = torch.full((3_000_000,), 12345, dtype=torch.int64, device="cuda")
+    keys[1_000_000:] = torch.arange(2_000_000, device="cuda") + (1 << 40)
+    keys[::1000] = -1
+    flags = t.find_or_put(keys)
+    assert int(flags[:1_000_000].sum()) == 1 and int(flags.sum()) == 1 + 2_000_000 - 2000
+    assert int(flags[::1000].sum()) == 0
+    assert t.sync() == 1 and t.size() == 1 + 2_000_000 - 2000
