@@ -349,12 +349,14 @@ typedef struct ht_bfs_result {
  * order: level d occupies [sum of sizes of levels < d, + size of level d).
  * h_level_sizes (nullable, max_levels entries) receives the level sizes.
  * Stops when a level is empty (complete = 1), or when max_levels or
- * states_cap would be exceeded (complete = 0).  Synchronises once per level.
+ * states_cap would be exceeded (complete = 0).  Synchronises once per level,
+ * or once per four small ones.
  * With a 128-bit table (models wider than 63 bits) states are 16-byte
  * pairs (low word first) and s0 is the initial state's low word (its high
  * word is 0).
- * Allocates its work buffers with cudaMalloc and frees them before
- * returning. */
+ * Allocates its work buffers in the order of `stream` (cudaMallocAsync) and
+ * frees them there before returning; a table keeps up to 16 MB of them, or as
+ * much as its slots take, until it is destroyed, for its next exploration. */
 ht_status ht_bfs(ht_table* t, const ht_model* h_model, uint64_t s0, uint32_t max_levels,
                  uint64_t* h_level_sizes, void* d_states, uint64_t states_cap,
                  ht_bfs_result* result, void* stream);

@@ -23,8 +23,10 @@ struct ht_table {
     ht_status sticky;            // HT_ERR_FULL once a key was dropped
     uint64_t seed_base;
     L2Window win;                // l2_persist: the slots (or the Cuckoo claim set)
-    void* part;                  // scratch of a reordered batch (keys, positions, counters), made on first use
+    void* part;                  // scratch of a reordered batch (PartScratch), made on first use
     size_t part_bytes;
+    void* bfs_mem;               // work memory of a small exploration, kept for the next
+    size_t bfs_bytes;
 };
 
 namespace {
@@ -415,7 +417,7 @@ void free_table(ht_table* t, cudaStream_t s) {
     if (!t) return;
     if (t->win.base) window_release(t->device);
     void* ptrs[] = {t->dt.slots, t->dt.stash, t->dt.ovf, t->dt.ctr, t->sc.set, t->sc.win, t->dt.kstore,
-                    t->part};
+                    t->part, t->bfs_mem};
     for (void* p : ptrs)
         if (p) cudaFreeAsync(p, s);
     delete t;
@@ -938,6 +940,22 @@ struct DevBuf {
     ~DevBuf() { cudaFree(p); }
 };
 
+// Stream-ordered device memory, freed in the stream's order unless it is kept.
+struct BfsMem {
+    explicit BfsMem(cudaStream_t st) : s(st) {}
+    void* p = nullptr;
+    bool keep = false;
+    cudaStream_t s;
+    cudaError_t alloc(size_t bytes) { return cudaMallocAsync(&p, bytes, s); }
+    void take(void* q) {
+        p = q;
+        keep = true;
+    }
+    ~BfsMem() {
+        if (p && !keep) cudaFreeAsync(p, s);
+    }
+};
+
 }  // namespace
 
 extern "C" {
@@ -953,8 +971,8 @@ ht_status ht_successors(const ht_model* h_model, uint32_t key_width, const void*
     const PreparedModel pm = prepare_model(*h_model);
     HT_TRY(cudaMalloc(&dm.p, sizeof(PreparedModel)));
     HT_TRY(cudaMemcpyAsync(dm.p, &pm, sizeof(pm), cudaMemcpyHostToDevice, s));
-    HT_TRY(successors(int(key_width), static_cast<const PreparedModel*>(dm.p), d_states, n, nullptr, 0, d_succ, cap,
-                      d_count, nullptr, s));
+    HT_TRY(successors(int(key_width), static_cast<const PreparedModel*>(dm.p), d_states, n, nullptr, d_succ, cap, d_count,
+                      nullptr, s));
     HT_TRY(cudaStreamSynchronize(s));        // the model copy is freed on return
     return HT_OK;
 }
@@ -976,25 +994,45 @@ static ht_status bfs_common(ht_table* t, const ht_model* h_model, uint64_t s0, u
     } else if (!states_cap) {
         return HT_ERR_INVALID;
     }
-    // Successor buffer (split form): up to 2^26 vectors per find-or-put
-    // launch sequence; the fused form has none.
-    const uint64_t succ_cap =
-        fused ? 1 : std::min<uint64_t>(1ull << 26, std::max<uint64_t>(msucc, (t->dt.nslots + 1) * msucc));
+    // Successor buffer (split form): up to 2^26 vectors per find-or-put launch
+    // sequence, no more than four per slot; the fused form has none.
+    const uint64_t slots = t->dt.nslots;
+    const uint64_t succ_cap = fused ? 1 : std::min<uint64_t>({1ull << 26, (slots + 1) * msucc, std::max(msucc, 4 * slots)});
     const uint64_t chunk_states = std::max<uint64_t>(1, succ_cap / msucc);
-    DevBuf dm, states_own, succ, ctr;
+    // States of a level that may run without the host: one Cuckoo launch pair.
+    const uint64_t ahead_states = t->scheme == HT_CUCKOO ? std::min(chunk_states, t->chunk / msucc) : chunk_states;
+    // One block of work memory, stream-ordered: the model, the counters, the
+    // successors.  A table keeps a block of up to 16 MB, or its slots' size, for its
+    // next exploration: mapping and unmapping one took 100 us of a small one's
+    // 1800 and, with the reordering scratch, 2 ms of a large one's 50.
+    const size_t model_bytes = (sizeof(PreparedModel) + 255) / 256 * 256;
+    const size_t need = model_bytes + 256 + 256 + succ_cap * ksz;
+    BfsMem work(s), states_own(s);
+    if (t->bfs_bytes >= need) {
+        work.take(t->bfs_mem);
+    } else {
+        HT_TRY(work.alloc(need));
+        if (need <= std::max<uint64_t>(16u << 20, slots * 8)) {
+            if (t->bfs_mem) cudaFreeAsync(t->bfs_mem, s);
+            t->bfs_mem = work.p;
+            t->bfs_bytes = need;
+            work.keep = true;
+        }
+    }
+    PreparedModel* model = static_cast<PreparedModel*>(work.p);
+    BfsCursor* cursor = reinterpret_cast<BfsCursor*>(static_cast<char*>(work.p) + model_bytes);
+    unsigned long long* c = reinterpret_cast<unsigned long long*>(static_cast<char*>(work.p) + model_bytes + 256);
+    void* succ = static_cast<char*>(work.p) + model_bytes + 512;
+    static_assert(sizeof(BfsCursor) <= 256, "work block layout");
     const PreparedModel pm = prepare_model(*h_model);
-    HT_TRY(cudaMalloc(&dm.p, sizeof(PreparedModel)));
-    HT_TRY(cudaMemcpyAsync(dm.p, &pm, sizeof(pm), cudaMemcpyHostToDevice, s));
+    HT_TRY(cudaMemcpyAsync(model, &pm, sizeof(pm), cudaMemcpyHostToDevice, s));
     if (!d_states) {
-        HT_TRY(cudaMalloc(&states_own.p, states_cap * ksz));
+        HT_TRY(states_own.alloc(states_cap * ksz));
         d_states = states_own.p;
     }
-    HT_TRY(cudaMalloc(&succ.p, succ_cap * ksz));
-    // ctr[0]: states stored so far; ctr[1]: successors of the current chunk;
-    // ctr[2]: successors generated in total; ctr[4..5]: the initial state
+    // c[0]: states stored so far; c[1]: successors of the current chunk;
+    // c[2]: successors generated in total; c[4..5]: the initial state
     // (16-byte aligned; for 128-bit tables s0 is its low word, the high word 0).
-    HT_TRY(cudaMalloc(&ctr.p, 6 * sizeof(unsigned long long)));
-    unsigned long long* c = static_cast<unsigned long long*>(ctr.p);
     unsigned long long init[6] = {0, 0, 0, 0, s0, 0};
     HT_TRY(cudaMemcpyAsync(c, init, sizeof(init), cudaMemcpyHostToDevice, s));
     // Level 0: the initial state (the open set starts with it).
@@ -1005,10 +1043,10 @@ static ht_status bfs_common(ht_table* t, const ht_model* h_model, uint64_t s0, u
     char* states = static_cast<char*>(d_states);
     uint64_t lo = 0;
     uint32_t level = 0;
+    unsigned long long hi = 0;
+    HT_TRY(cudaMemcpyAsync(&hi, c, sizeof(hi), cudaMemcpyDeviceToHost, s));
+    HT_TRY(cudaStreamSynchronize(s));
     for (;;) {
-        unsigned long long hi = 0;
-        HT_TRY(cudaMemcpyAsync(&hi, c, sizeof(hi), cudaMemcpyDeviceToHost, s));
-        HT_TRY(cudaStreamSynchronize(s));
         if (hi > states_cap) {               // the states buffer overflowed: stop
             result->states = states_cap;
             result->levels = level;
@@ -1027,29 +1065,58 @@ static ht_status bfs_common(ht_table* t, const ht_model* h_model, uint64_t s0, u
             break;
         }
         if (h_level_sizes) h_level_sizes[level] = nd;
-        if (fused) {
-            HT_TRY(bfs_fused_level(bucket_cfg(t), static_cast<const PreparedModel*>(dm.p), states + lo * ksz, nd,
-                                   t->dt, d_states, c, states_cap, c + 2, s));
-            lo = hi;
-            ++level;
+        if (!fused && nd <= ahead_states / 4) {
+            // A small level: it and the next few run without the host, each
+            // advance opening the next one on the device.  Waiting for the host
+            // after every level took 10 of a small exploration's 75 us a level.
+            BfsCursor cur = {lo, hi, level, 0, 0, 0, {}};
+            HT_TRY(cudaMemcpyAsync(cursor, &cur, sizeof(cur), cudaMemcpyHostToDevice, s));
+            HT_TRY(cudaMemsetAsync(c + 1, 0, sizeof(unsigned long long), s));
+            for (int i = 0; i < kBfsAhead; ++i) {
+                const uint64_t most = i ? ahead_states : nd;
+                HT_TRY(successors(int(t->kw), model, states, most, cursor, succ, succ_cap, c + 1, c + 2, s));
+                st = run_put(t, succ, nullptr, std::min<uint64_t>(succ_cap, most * msucc), nullptr, d_states, c, s, c + 1,
+                             states_cap);
+                if (st != HT_OK) return st;
+                HT_TRY(bfs_advance(cursor, c, c + 1, states_cap, max_levels, ahead_states, s));
+            }
+            HT_TRY(cudaMemcpyAsync(&cur, cursor, sizeof(cur), cudaMemcpyDeviceToHost, s));
+            HT_TRY(cudaMemcpyAsync(&hi, c, sizeof(hi), cudaMemcpyDeviceToHost, s));
+            HT_TRY(cudaStreamSynchronize(s));
+            // The levels opened but for the last are expanded; the loop's head
+            // records the last one again, or ends as the cursor stopped.
+            const bool open = !cur.stop || cur.stop == BfsCursor::kLarge;
+            for (unsigned long long i = 0; i < cur.opened; ++i)
+                if (h_level_sizes) h_level_sizes[level + 1 + i] = cur.sizes[i];
+            level = uint32_t(cur.level) + (open ? 0u : 1u);
+            lo = cur.stop == BfsCursor::kLarge ? cur.next_lo : cur.lo;
             continue;
         }
-        for (uint64_t c0 = lo; c0 < hi; c0 += chunk_states) {
+        if (fused) {
+            HT_TRY(bfs_fused_level(bucket_cfg(t), model, states + lo * ksz, nd, t->dt, d_states, c, states_cap, c + 2, s));
+        }
+        for (uint64_t c0 = lo; !fused && c0 < hi; c0 += chunk_states) {
             const uint64_t m = std::min<uint64_t>(chunk_states, hi - c0);
             HT_TRY(cudaMemsetAsync(c + 1, 0, sizeof(unsigned long long), s));
-            HT_TRY(successors(int(t->kw), static_cast<const PreparedModel*>(dm.p), states + c0 * ksz, m, nullptr, 0, succ.p,
-                              succ_cap, c + 1, c + 2, s));
-            st = run_put(t, succ.p, nullptr, std::min<uint64_t>(succ_cap, m * msucc), nullptr, d_states, c, s, c + 1,
+            HT_TRY(successors(int(t->kw), model, states + c0 * ksz, m, nullptr, succ, succ_cap, c + 1, c + 2, s));
+            st = run_put(t, succ, nullptr, std::min<uint64_t>(succ_cap, m * msucc), nullptr, d_states, c, s, c + 1,
                          states_cap, succ_cap);
             if (st != HT_OK) return st;
         }
         lo = hi;
         ++level;
+        HT_TRY(cudaMemcpyAsync(&hi, c, sizeof(hi), cudaMemcpyDeviceToHost, s));
+        HT_TRY(cudaStreamSynchronize(s));
     }
     unsigned long long gen = 0;
     HT_TRY(cudaMemcpyAsync(&gen, c + 2, sizeof(gen), cudaMemcpyDeviceToHost, s));
     HT_TRY(cudaStreamSynchronize(s));
     result->successors = gen;
+    if (t->part_bytes > std::max<uint64_t>(256u << 20, slots * 8)) {     // nor reordering scratch past that size
+        cudaFreeAsync(t->part, s);
+        t->part = nullptr;
+        t->part_bytes = 0;
+    }
     const ht_status ts = sync_and_status(t, s);
     return ts;
 }

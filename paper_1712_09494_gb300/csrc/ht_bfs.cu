@@ -23,9 +23,8 @@ constexpr int kSuccStage = 1024;
 template <typename T>
 __global__ void __launch_bounds__(kSuccBlock)
 successors_kernel(const PreparedModel* __restrict__ model, const T* __restrict__ states, uint64_t n,
-                  const unsigned long long* __restrict__ d_n, uint64_t off, T* __restrict__ succ,
-                  uint64_t cap, unsigned long long* __restrict__ count,
-                  unsigned long long* __restrict__ total) {
+                  const BfsCursor* __restrict__ cur, T* __restrict__ succ, uint64_t cap,
+                  unsigned long long* __restrict__ count, unsigned long long* __restrict__ total) {
     // 16-byte states (models wider than 63 bits) use a half-size stage.
     constexpr int kStage = sizeof(T) > 8 ? kSuccStage / 2 : kSuccStage;
     using S = typename std::conditional<(sizeof(T) > 8), unsigned __int128, uint64_t>::type;
@@ -37,9 +36,10 @@ successors_kernel(const PreparedModel* __restrict__ model, const T* __restrict__
         for (int i = threadIdx.x; i < int(sizeof(PreparedModel) / 4); i += blockDim.x) dst[i] = src[i];
     }
     __syncthreads();
-    if (d_n) {
-        const uint64_t all = __ldcg(d_n);
-        n = all > off ? min(n, all - off) : 0;
+    if (cur) {                                   // the level that a BfsCursor holds
+        const uint64_t lo = __ldcg(&cur->lo), hi = __ldcg(&cur->hi);
+        states += lo;
+        n = min(n, hi - lo);
     }
     const int lane = threadIdx.x & 31;
     T* buf = s_out[threadIdx.x >> 5];
@@ -84,6 +84,30 @@ successors_kernel(const PreparedModel* __restrict__ model, const T* __restrict__
         for (int o = 16; o; o >>= 1) made += __shfl_down_sync(0xFFFFFFFFu, made, o);
         if (lane == 0 && made) atomicAdd(total, made);
     }
+}
+
+// Opens the next level of an exploration whose levels run without the host
+// (ht_bfs), or stops it.
+__global__ void bfs_advance_kernel(BfsCursor* __restrict__ c, unsigned long long* __restrict__ count,
+                                   unsigned long long* __restrict__ succ_count, uint64_t states_cap, uint32_t max_levels,
+                                   uint64_t most) {
+    *succ_count = 0;
+    if (c->stop) return;
+    const unsigned long long nh = *count, nd = nh - c->hi;
+    c->lo = c->hi;
+    if (nh > states_cap) {
+        c->stop = BfsCursor::kOverflow;
+    } else if (nd == 0) {
+        c->stop = BfsCursor::kDone;
+    } else if (c->level + 1 >= max_levels) {
+        c->stop = BfsCursor::kLimit;
+    } else {
+        if (nd > most) c->stop = BfsCursor::kLarge;
+        c->sizes[c->opened++] = nd;
+        ++c->level;
+    }
+    if (!c->stop || c->stop == BfsCursor::kLarge) c->hi = nh;
+    if (c->stop == BfsCursor::kLarge) c->next_lo = c->lo, c->lo = c->hi;      // nothing to expand here
 }
 
 // Multi-table successors: the expanded states of every exploration form one
@@ -136,23 +160,29 @@ cudaError_t multi_successors(int, const MultiDev& m, uint64_t max_work, cudaStre
     return cudaGetLastError();
 }
 
+cudaError_t bfs_advance(BfsCursor* c, unsigned long long* count, unsigned long long* succ_count, uint64_t states_cap,
+                        uint32_t max_levels, uint64_t most, cudaStream_t s) {
+    bfs_advance_kernel<<<1, 1, 0, s>>>(c, count, succ_count, states_cap, max_levels, most);
+    return cudaGetLastError();
+}
+
 cudaError_t successors(int kw, const PreparedModel* model, const void* states, uint64_t n,
-                       const unsigned long long* d_n, uint64_t off, void* succ, uint64_t cap,
+                       const BfsCursor* cur, void* succ, uint64_t cap,
                        unsigned long long* count, unsigned long long* total, cudaStream_t s) {
     ProfScope ps(kKSuccessors, s);
     if (kw == 32) {
         auto k = successors_kernel<uint32_t>;
-        k<<<launch_blocks((const void*)k, kSuccBlock), kSuccBlock, 0, s>>>(
-            model, static_cast<const uint32_t*>(states), n, d_n, off, static_cast<uint32_t*>(succ), cap, count, total);
+        k<<<launch_grid((const void*)k, kSuccBlock, n, kSuccBlock), kSuccBlock, 0, s>>>(
+            model, static_cast<const uint32_t*>(states), n, cur, static_cast<uint32_t*>(succ), cap, count, total);
     } else if (kw == 128) {
         using U = unsigned __int128;
         auto k = successors_kernel<U>;
-        k<<<launch_blocks((const void*)k, kSuccBlock), kSuccBlock, 0, s>>>(
-            model, static_cast<const U*>(states), n, d_n, off, static_cast<U*>(succ), cap, count, total);
+        k<<<launch_grid((const void*)k, kSuccBlock, n, kSuccBlock), kSuccBlock, 0, s>>>(
+            model, static_cast<const U*>(states), n, cur, static_cast<U*>(succ), cap, count, total);
     } else {
         auto k = successors_kernel<uint64_t>;
-        k<<<launch_blocks((const void*)k, kSuccBlock), kSuccBlock, 0, s>>>(
-            model, static_cast<const uint64_t*>(states), n, d_n, off, static_cast<uint64_t*>(succ), cap, count, total);
+        k<<<launch_grid((const void*)k, kSuccBlock, n, kSuccBlock), kSuccBlock, 0, s>>>(
+            model, static_cast<const uint64_t*>(states), n, cur, static_cast<uint64_t*>(succ), cap, count, total);
     }
     return cudaGetLastError();
 }

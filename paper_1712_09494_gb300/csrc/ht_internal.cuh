@@ -569,12 +569,29 @@ void table_forget(ht_table* t);
 // synchronisation (the caller guarantees no work on the table is pending).
 void table_release(ht_table* t, cudaStream_t s);
 
-// State-space successors (ht_bfs.cu).  `model` is a device copy of ht_model.
+// State-space successors (ht_bfs.cu) of states[0..n), or (cur given) of the level
+// it holds, at most n.  `model` is a device copy of ht_model.
 // count: reservation counter for succ[]; total (nullable): running count of
 // successors generated.
 cudaError_t successors(int kw, const PreparedModel* model, const void* states, uint64_t n,
-                       const unsigned long long* d_n, uint64_t off, void* succ, uint64_t cap,
+                       const struct BfsCursor* cur, void* succ, uint64_t cap,
                        unsigned long long* count, unsigned long long* total, cudaStream_t s);
+
+// Where an exploration stands whose levels run one after another on the device,
+// kBfsAhead of them before the host looks: the level to expand is states
+// [lo, hi); stop ends it, and lo = hi then leaves later launches nothing to do.
+constexpr int kBfsAhead = 4;
+struct BfsCursor {
+    enum : unsigned long long { kDone = 1, kOverflow = 2, kLimit = 3, kLarge = 4 };
+    unsigned long long lo, hi, level, stop;
+    unsigned long long next_lo;               // kLarge: the level's start (a level too large for one buffer)
+    unsigned long long opened;                // levels opened since the host looked, and their sizes
+    unsigned long long sizes[kBfsAhead];
+};
+// Opens the next level: count is the number of states stored, *succ_count is
+// zeroed, a level of more than `most` states is left to the host.
+cudaError_t bfs_advance(BfsCursor* c, unsigned long long* count, unsigned long long* succ_count, uint64_t states_cap,
+                        uint32_t max_levels, uint64_t most, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Batched exploration of many models at once (ht_multi.cu).  One step
