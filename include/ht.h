@@ -67,10 +67,10 @@ typedef enum {
  *   stash_slots    default 101 (both schemes).
  *   bucket_slots   8, 16 or 32 slots of 8 bytes; default 16 (128 bytes).
  *   lanes_per_key  lanes that read one bucket (2..32, with 1 to 8 slots per
- *                  lane); default 2.  Checked, and used by 128-bit tables;
- *                  32- and 64-bit buckets are read by one lane a sector at a
- *                  time, or whole by bucket_slots / 8 lanes in tables larger
- *                  than L2, whatever it says (the fastest on GB300).
+ *                  lane); default 2.  Checked, but the kernels choose by the
+ *                  table's and the batch's size: one lane reads a part of the
+ *                  bucket at a time, or one lane per 64 bytes reads it whole
+ *                  (whichever measured faster on GB300).
  *   max_rebuilds   rebuild attempts with fresh hash constants, default 8.
  *   max_batch      cuckoo keys per probe/insert launch pair (sizes the
  *                  in-batch dedup scratch), default 2^22.

@@ -99,7 +99,7 @@ cudaError_t export_any(ht_table* t, void* keys, uint32_t* vals, unsigned long lo
 // batch 400 instead of 730, and 120 to reorder).  Regions of at most 24 MB: all
 // blocks work on two or three of them at a time.
 int region_bits(const ht_table* t, uint64_t n) {
-    const uint64_t bytes = t->dt.nslots * 8, l2 = l2_bytes();
+    const uint64_t bytes = t->dt.nslots * (t->kw == 128 ? 16 : 8), l2 = l2_bytes();
     if (!l2 || bytes <= l2 || t->win.bytes || n / 5 * 4 < bytes / 128) return 0;
     int bits = 1;
     while (bits < 8 && (bytes >> bits) > (24u << 20)) ++bits;
@@ -160,6 +160,32 @@ void* part_scratch(ht_table* t, size_t need, cudaStream_t s) {
 // with flags) stays a fraction of a table that wants it.
 constexpr uint64_t kPartPiece = 1ull << 24;
 
+// Runs op(keys, count, flags, local) over a batch: in pieces in region order
+// where that pays (local), with the flags brought back to the batch's order,
+// else as it is.
+template <class Op>
+ht_status in_region_order(ht_table* t, const void* keys, uint64_t n, const unsigned long long* d_n, uint8_t* flags,
+                          cudaStream_t s, Op&& op) {
+    const size_t ksz = t->kw / 8;
+    const uint64_t piece = d_n ? n : std::min(n, kPartPiece);
+    const int bits = region_bits(t, d_n ? piece / 2 : piece);        // d_n: about half of the bound
+    void* p = bits ? part_scratch(t, PartScratch(nullptr, piece, ksz, flags != nullptr, bits).bytes, s) : nullptr;
+    if (!p) return op(keys, n, flags, false);
+    const PartScratch ps(p, piece, ksz, flags != nullptr, bits);
+    uint64_t off = 0;
+    for (; off < n && (d_n || region_bits(t, std::min(piece, n - off))); off += piece) {
+        const uint64_t m = std::min(piece, n - off);
+        HT_TRY(partition_keys(int(t->kw), static_cast<const char*>(keys) + off * ksz, m, d_n, t->dt.seed[0], bits, ps.ctl,
+                              ps.keys, ps.loc, ps.runs, s));
+        const ht_status st = op(ps.keys, m, ps.flags, true);
+        if (st != HT_OK) return st;
+        if (flags) HT_TRY(partition_back(ps.flags, ps.loc, ps.runs, bits, m, flags + off, s));
+    }
+    if (off >= n) return HT_OK;
+    // A last piece too small to be worth it.
+    return op(static_cast<const char*>(keys) + off * ksz, n - off, flags ? flags + off : nullptr, false);
+}
+
 // Runs find-or-put / insert over a batch without touching rebuild state.
 ht_status run_put(ht_table* t, const void* keys, const uint32_t* vals, uint64_t n, uint8_t* is_new,
                   void* new_out, unsigned long long* new_count, cudaStream_t s,
@@ -180,9 +206,12 @@ ht_status run_put(ht_table* t, const void* keys, const uint32_t* vals, uint64_t 
     }
     if (t->kw == 128) {
         if (vals) return HT_ERR_INVALID;
-        if (t->scheme == HT_BUCKET)
-            return cuda_status(wide_find_or_put(int(t->p.lanes_per_key), t->dt, keys, n, d_n, is_new, new_out,
-                                                new_count, new_cap, s));
+        if (t->scheme == HT_BUCKET) {
+            auto put = [&](const void* k, uint64_t m, uint8_t* flags, bool local) {
+                return cuda_status(wide_find_or_put(t->dt, k, m, d_n, flags, new_out, new_count, new_cap, s, local));
+            };
+            return d_n && n > part_cap ? put(keys, n, is_new, false) : in_region_order(t, keys, n, d_n, is_new, s, put);
+        }
         for (uint64_t off = 0; off < n; off += t->chunk) {
             const uint64_t m = std::min(t->chunk, n - off);
             HT_TRY(wide_cuckoo_probe(t->dt, t->sc, t->parity, static_cast<const char*>(keys) + off * 16, m, d_n, off,
@@ -211,26 +240,10 @@ ht_status run_put(ht_table* t, const void* keys, const uint32_t* vals, uint64_t 
         }
         return HT_OK;
     };
-    if (!vals && (!d_n || n <= part_cap)) {
-        const uint64_t piece = d_n ? n : std::min(n, kPartPiece);
-        const int bits = region_bits(t, d_n ? piece / 2 : piece);   // d_n: about half of the bound
-        void* p = bits ? part_scratch(t, PartScratch(nullptr, piece, ksz, is_new != nullptr, bits).bytes, s) : nullptr;
-        if (p) {
-            const PartScratch ps(p, piece, ksz, is_new != nullptr, bits);
-            uint64_t off = 0;
-            for (; off < n && (d_n || region_bits(t, std::min(piece, n - off))); off += piece) {
-                const uint64_t m = std::min(piece, n - off);
-                HT_TRY(partition_keys(int(t->kw), static_cast<const char*>(keys) + off * ksz, m, d_n, t->dt.seed[0], bits,
-                                      ps.ctl, ps.keys, ps.loc, ps.runs, s));
-                const ht_status st = put(ps.keys, m, d_n, ps.flags, nullptr, true);
-                if (st != HT_OK) return st;
-                if (is_new) HT_TRY(partition_back(ps.flags, ps.loc, ps.runs, bits, m, is_new + off, s));
-            }
-            if (off >= n) return HT_OK;
-            return put(static_cast<const char*>(keys) + off * ksz, n - off, nullptr, is_new ? is_new + off : nullptr,
-                       nullptr, false);              // a last piece too small to be worth it
-        }
-    }
+    if (!vals && (!d_n || n <= part_cap))
+        return in_region_order(t, keys, n, d_n, is_new, s, [&](const void* k, uint64_t m, uint8_t* flags, bool local) {
+            return put(k, m, d_n, flags, nullptr, local);
+        });
     return put(keys, n, d_n, is_new, vals, false);
 }
 
@@ -702,7 +715,7 @@ ht_status ht_lookup(ht_table* t, const void* d_keys, uint64_t n, uint32_t* d_val
     if (t->kw == 128) {
         if (d_values) return HT_ERR_INVALID;
         if (t->scheme == HT_CUCKOO) return cuda_status(wide_cuckoo_lookup(t->dt, d_keys, n, d_found, s));
-        return cuda_status(wide_lookup(int(t->p.lanes_per_key), t->dt, d_keys, n, d_found, s));
+        return cuda_status(wide_lookup(t->dt, d_keys, n, d_found, s));
     }
     if (t->scheme == HT_BUCKET)
         return cuda_status(bucket_lookup(bucket_cfg(t), t->dt, d_keys, n, d_values, d_found, s, t->win));

@@ -134,6 +134,12 @@ template <> struct Keys<64> {
     }
 };
 
+// The bucket hash of a 128-bit key: the 64-bit family applied to a fold of
+// both words (mix64 of the high word, xored into the low word).
+__device__ __forceinline__ uint64_t wide_fold(uint64_t lo, uint64_t hi) {
+    return lo ^ mix64(hi ^ 0xD1B54A32D192ED03ull);
+}
+
 // 16-byte atomics on a 16-byte-aligned pair of words (sm_90 and later):
 // compare-and-swap from EMPTY (all ones in both words), and exchange.
 __device__ __forceinline__ void cas128(uint64_t* addr, uint64_t new_lo, uint64_t new_hi, uint64_t& old_lo,
@@ -415,8 +421,8 @@ cudaError_t cuckoo_insert(int kw, const DevTable& t, const DevScratch& sc, uint3
 cudaError_t cuckoo_lookup(int kw, const DevTable& t, const void* keys, uint64_t n,
                           uint32_t* vals, uint8_t* found, cudaStream_t s, const L2Window& w = L2Window());
 
-// Reorders n (or *d_n) 32- or 64-bit keys by the top `bits` of their first hash
-// (mix64 of key xor seed) into out.  ctl: 2 * kMaxRegions words of scratch.  loc
+// Reorders n (or *d_n) 32-, 64- or 128-bit keys by the top `bits` of their first
+// hash (mix64 of key xor seed) into out.  ctl: 2 * kMaxRegions words of scratch.  loc
 // (nullable; n places) and runs (8 << bits bytes per kPartTile keys) keep what
 // partition_back needs to bring one byte per key back to the batch's order.
 constexpr int kMaxRegions = 256;
@@ -517,11 +523,10 @@ cudaError_t bfs_fused_level(const BucketCfg& c, const PreparedModel* model, cons
 
 // Bucket-scheme tables of 128-bit keys (ht_wide.cu): keys are 16-byte pairs
 // (low word, high word), 16-byte aligned; slots are 16 bytes, buckets 8 slots.
-cudaError_t wide_find_or_put(int lanes, const DevTable& t, const void* keys, uint64_t n,
-                             const unsigned long long* d_n, uint8_t* is_new, void* new_out,
-                             unsigned long long* new_count, uint64_t new_cap, cudaStream_t s);
-cudaError_t wide_lookup(int lanes, const DevTable& t, const void* keys, uint64_t n, uint8_t* found,
-                        cudaStream_t s);
+cudaError_t wide_find_or_put(const DevTable& t, const void* keys, uint64_t n, const unsigned long long* d_n,
+                             uint8_t* is_new, void* new_out, unsigned long long* new_count, uint64_t new_cap,
+                             cudaStream_t s, bool local = false);
+cudaError_t wide_lookup(const DevTable& t, const void* keys, uint64_t n, uint8_t* found, cudaStream_t s);
 cudaError_t wide_export(const DevTable& t, void* keys, unsigned long long* count, uint64_t cap, cudaStream_t s);
 // Cuckoo tables of 128-bit keys: probe (stores into the first empty slot,
 // dedup of the keys with every slot full, winners of `parity`; list_stored:

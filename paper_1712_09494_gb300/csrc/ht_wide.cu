@@ -27,12 +27,6 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 
 __device__ __forceinline__ bool wide_reserved(uint64_t hi) { return (hi >> 63) != 0; }
 
-// The bucket hash of a 128-bit key: the 64-bit family applied to a fold of
-// both words (mix64 of the high word, xored into the low word).
-__device__ __forceinline__ uint64_t wide_fold(uint64_t lo, uint64_t hi) {
-    return lo ^ mix64(hi ^ 0xD1B54A32D192ED03ull);
-}
-
 // Slot classes of a read: 2 = a complete key, 1 = a claim candidate.
 __device__ __forceinline__ int slot_class(uint64_t lo, uint64_t hi) {
     return (lo != kOnes && hi != kOnes) ? 2 : 1;
@@ -78,7 +72,7 @@ struct WideEntry {
     ulonglong2 key;
     uint64_t pos;      // where its answer goes
     uint32_t f;        // the hash function to try next
-    uint32_t pad_;
+    uint32_t half;     // halves of that bucket tried
 };
 
 // All k buckets full: the overflow set.  Out of line: rare.  Returns 1 when
@@ -97,20 +91,23 @@ __device__ __noinline__ uint32_t wide_spill_find(const DevTable& t, uint64_t lo,
     return wide_ovf_find(t, lo, hi);
 }
 
+// Where a key's claims start in its bucket: the half, then the slot in each half.
+__device__ __forceinline__ uint32_t wide_rot(ulonglong2 key) { return bucket::claim_rot(key.x ^ key.y) % kWideBS; }
+
 // One pass of a tile of 32 keys over one bucket each (lane l holds key l and
 // its bucket's index; ok false without one): 0 found (lookup: absent), 1 stored
-// (lookup: found), 2 its bucket is full of other keys.  Group g (G lanes)
+// (lookup: found), 2 its bucket is full of other keys.  Group g (two lanes)
 // serves key q*(32/G)+g in round q; all rounds' buckets are read up front with
 // 256-bit loads and the first claims go out together.  A claim that another
 // key's won is followed by the next candidate slot's at once: a stored key
 // whose low word is all ones always reads as a candidate, so reading the bucket
 // again would not get past it.
-template <int G, bool LOOKUP>
+template <bool LOOKUP>
 __device__ __forceinline__ uint32_t wide_pass(uint64_t* slots, ulonglong2 mykey, uint64_t mybkt, bool myok) {
-    constexpr int SPL = kWideBS / G;
+    constexpr int G = 2, SPL = kWideBS / G;
     constexpr int GPW = 32 / G;
     constexpr uint32_t kGMask = (1u << G) - 1u;
-    constexpr int PF = G < 4 ? G : 2;               // 16 words of buckets in flight per lane
+    constexpr int PF = G;                           // 16 words of buckets in flight per lane
     const int lane = threadIdx.x & 31;
     const int grp = lane / G, sub = lane % G, gbase = grp * G;
     const int mysh = (lane % GPW) * G, myround = lane / GPW;
@@ -158,7 +155,7 @@ __device__ __forceinline__ uint32_t wide_pass(uint64_t* slots, ulonglong2 mykey,
                 done[q] |= ge != 0;                 // a key moves on only from a full bucket
                 if (myround == r0 + q && ((M >> mysh) & kGMask)) status = 1;
             } else {
-                rot[q] = (bucket::claim_rot(lo[q] ^ hi[q]) % kWideBS);
+                rot[q] = wide_rot(make_ulonglong2(lo[q], hi[q]));
                 const uint32_t ge = (__ballot_sync(kFull, cand[q] != 0) >> gbase) & kGMask;
                 if (cand[q] && uint32_t(sub) == bucket::first_from<G>(ge, rot[q] / SPL)) {
                     claim[q] = int(bucket::first_from<SPL>(cand[q], rot[q] % SPL));
@@ -208,18 +205,51 @@ __device__ __forceinline__ uint32_t wide_pass(uint64_t* slots, ulonglong2 mykey,
     return status;
 }
 
+// The same for one key by one lane over half of its bucket (find-or-put only):
+// 64 bytes, searched from the half that the key's claims start in; a free slot
+// in a half ends the search, as a sector does in the 64-bit kernels.
+__device__ __forceinline__ uint32_t half_pass(uint64_t* slots, ulonglong2 key, uint64_t half, bool ok) {
+    constexpr int S = kWideBS / 2;
+    if (!ok) return 0;
+    uint64_t* p = slots + half * (2 * S);
+    uint64_t w[2 * S];
+    bucket::load_sectors<2 * S>(p, true, w);
+    uint32_t e = 0;
+    bool hit = false;
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+        const uint64_t x = w[2 * j], y = w[2 * j + 1];
+        const bool part = (y >> 63) != 0 || x == kOnes;
+        hit |= x == key.x && y == key.y && !part;
+        e |= uint32_t(part) << j;
+    }
+    if (hit) return 0;
+    const uint32_t rot = wide_rot(key);
+    while (e) {                                     // bounded: each turn spends a candidate slot
+        const uint32_t j = bucket::first_from<S>(e, rot % S);
+        e &= ~(1u << j);
+        uint64_t ol, oh;
+        cas128(p + 2 * j, key.x, key.y, ol, oh);
+        if (ol == kOnes && oh == kOnes) return 1;
+        if (ol == key.x && oh == key.y) return 0;
+    }
+    return 2;
+}
+
 // find-or-put or lookup: a warp takes a fresh tile of 32 keys, or 32 queued
 // ones, for one pass over one bucket each, as the 64-bit kernel does
-// (bucket_tiles in ht_bucket.cu).  Bound by random 128-byte lines.
+// (bucket_tiles in ht_bucket.cu).  Bound by random 128-byte lines.  HALF: one
+// lane per key and half a bucket a pass, where the table's lines are in L2.
 // APPEND: the keys new to the table also go to new_out at *new_count
 // (staged per warp in shared memory; entries past new_cap not written).
 // d_n (nullable): the batch size produced on the device, at most n.
 // ahead: a lookup in a table larger than L2 touches the next tile's buckets.
-#ifndef HT_WIDE_MIN_BLOCKS
-#define HT_WIDE_MIN_BLOCKS 3
-#endif
-template <int G, bool LOOKUP, bool APPEND>
-__global__ void __launch_bounds__(kBlock, HT_WIDE_MIN_BLOCKS)
+// Fill of 2^26 keys to load 0.8 in batches of 2^24: 3.97 ms (whole buckets, not
+// reordered: 4.15; before, a round of the tile at a time: 5.40); of 2^22 keys in
+// L2 198 us (313).  Blocks per SM: whole 3 (2: 4.90, 4: 5.27 ms), halves 4 (3:
+// 3.99, 5: 4.30).
+template <bool LOOKUP, bool APPEND, bool HALF>
+__global__ void __launch_bounds__(kBlock, HALF ? 4 : 3)
 wide_kernel(const __grid_constant__ DevTable t, const ulonglong2* __restrict__ keys, uint64_t n,
             const unsigned long long* __restrict__ d_n, uint8_t* __restrict__ out,
             ulonglong2* __restrict__ new_out, unsigned long long* __restrict__ new_count, uint64_t new_cap, bool ahead) {
@@ -242,7 +272,7 @@ wide_kernel(const __grid_constant__ DevTable t, const ulonglong2* __restrict__ k
     for (;;) {
         ulonglong2 key = make_ulonglong2(0, 0);
         uint64_t pos = 0;
-        uint32_t f = 0;
+        uint32_t f = 0, half = 0;
         bool mine, ok;
         if (waiting >= 32 || (base >= n && waiting)) {
             const uint32_t m = min(waiting, 32u);
@@ -252,6 +282,7 @@ wide_kernel(const __grid_constant__ DevTable t, const ulonglong2* __restrict__ k
                 key = e.key;
                 pos = e.pos;
                 f = e.f;
+                half = e.half;
             }
             waiting -= m;
             __syncwarp();
@@ -270,9 +301,13 @@ wide_kernel(const __grid_constant__ DevTable t, const ulonglong2* __restrict__ k
             break;
         }
         const uint64_t fold = wide_fold(key.x, key.y);
-        uint32_t st = wide_pass<G, LOOKUP>(t.slots, key, hidx(fold, t.seed[f], t.nbuckets), ok);
+        const uint64_t bkt = hidx(fold, t.seed[f], t.nbuckets);
+        uint32_t st;
+        if constexpr (HALF) st = half_pass(t.slots, key, bkt * 2 + ((wide_rot(key) / (kWideBS / 2) + half) & 1u), ok);
+        else st = wide_pass<LOOKUP>(t.slots, key, bkt, ok);
         bool waits = st == 2;
-        if (waits && ++f >= t.k) {
+        if (HALF && waits) half ^= 1u;
+        if (waits && !half && ++f >= t.k) {
             st = LOOKUP ? wide_spill_find(t, key.x, key.y) : wide_spill_put(t, key.x, key.y);
             waits = false;
         }
@@ -283,6 +318,7 @@ wide_kernel(const __grid_constant__ DevTable t, const ulonglong2* __restrict__ k
                 e.key = key;
                 e.pos = pos;
                 e.f = f;
+                e.half = half;
                 if (LOOKUP && ahead) touch_l2(t.slots + 2 * kWideBS * hidx(fold, t.seed[f], t.nbuckets));
             }
             waiting += __popc(wm);
@@ -682,40 +718,39 @@ wide_cuckoo_insert_kernel(const DevTable t, const DevScratch sc, uint32_t parity
     if (lane == 0 && exchanges) atomicAdd(&t.ctr->exchanges, exchanges);
 }
 
-template <int G, bool LOOKUP, bool APPEND>
+template <bool LOOKUP, bool APPEND, bool HALF>
 cudaError_t launch_wide(const DevTable& t, const void* keys, uint64_t n, const unsigned long long* d_n,
                         uint8_t* out, void* new_out, unsigned long long* new_count, uint64_t new_cap,
                         cudaStream_t s) {
-    auto k = wide_kernel<G, LOOKUP, APPEND>;
+    auto k = wide_kernel<LOOKUP, APPEND, HALF>;
     k<<<launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s>>>(
         t, static_cast<const ulonglong2*>(keys), n, d_n, out, static_cast<ulonglong2*>(new_out), new_count, new_cap,
         t.nslots * 16 > l2_bytes());
     return cudaGetLastError();
 }
 
+// As for 64-bit buckets: smaller batches are read a bucket at a time.
+constexpr uint64_t kHalfKeys = 1ull << 19;
+
 }  // namespace
 
-cudaError_t wide_find_or_put(int lanes, const DevTable& t, const void* keys, uint64_t n,
-                             const unsigned long long* d_n, uint8_t* is_new, void* new_out,
-                             unsigned long long* new_count, uint64_t new_cap, cudaStream_t s) {
+cudaError_t wide_find_or_put(const DevTable& t, const void* keys, uint64_t n, const unsigned long long* d_n,
+                             uint8_t* is_new, void* new_out, unsigned long long* new_count, uint64_t new_cap,
+                             cudaStream_t s, bool local) {
     if (!n) return cudaSuccess;
     ProfScope ps(kKBucketFop, s);
-#define L(G)                                                                                                 \
-    return new_out ? launch_wide<G, false, true>(t, keys, n, d_n, is_new, new_out, new_count, new_cap, s)     \
-                   : launch_wide<G, false, false>(t, keys, n, d_n, is_new, nullptr, nullptr, 0, s);
-    if (lanes == 2) L(2)
-    if (lanes == 4) L(4)
-#undef L
-    return cudaErrorInvalidValue;
+    const bool half = local || (n >= kHalfKeys && t.nslots * 16 <= l2_bytes());
+    if (new_out)
+        return half ? launch_wide<false, true, true>(t, keys, n, d_n, is_new, new_out, new_count, new_cap, s)
+                    : launch_wide<false, true, false>(t, keys, n, d_n, is_new, new_out, new_count, new_cap, s);
+    return half ? launch_wide<false, false, true>(t, keys, n, d_n, is_new, nullptr, nullptr, 0, s)
+                : launch_wide<false, false, false>(t, keys, n, d_n, is_new, nullptr, nullptr, 0, s);
 }
 
-cudaError_t wide_lookup(int lanes, const DevTable& t, const void* keys, uint64_t n, uint8_t* found,
-                        cudaStream_t s) {
+cudaError_t wide_lookup(const DevTable& t, const void* keys, uint64_t n, uint8_t* found, cudaStream_t s) {
     if (!n) return cudaSuccess;
     ProfScope ps(kKBucketLookup, s);
-    if (lanes == 2) return launch_wide<2, true, false>(t, keys, n, nullptr, found, nullptr, nullptr, 0, s);
-    if (lanes == 4) return launch_wide<4, true, false>(t, keys, n, nullptr, found, nullptr, nullptr, 0, s);
-    return cudaErrorInvalidValue;
+    return launch_wide<true, false, false>(t, keys, n, nullptr, found, nullptr, nullptr, 0, s);
 }
 
 cudaError_t wide_cuckoo_probe(const DevTable& t, const DevScratch& sc, uint32_t parity, const void* keys, uint64_t n,

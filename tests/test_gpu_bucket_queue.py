@@ -154,8 +154,7 @@ def test_nearly_full_table_of_long_keys(w, digest_bits):
     assert set(map(tuple, to_np(got, np.uint64).tolist())) == set(map(tuple, keys[:n].tolist()))
 
 
-@pytest.mark.parametrize("scheme", ["bucket", "cuckoo"])
-@pytest.mark.parametrize("kw", [32, 64])
+@pytest.mark.parametrize("scheme,kw", [("bucket", 32), ("bucket", 64), ("bucket", 128), ("cuckoo", 32), ("cuckoo", 64)])
 def test_large_batches_are_reordered_by_table_region(scheme, kw):
     """Batches with more keys than the table (past L2) has lines, taken region by region: whole pieces of 2^24 keys
     with a ragged one after them, batches with and without flags, appended keys, repeats in other batches, and an
@@ -164,11 +163,13 @@ def test_large_batches_are_reordered_by_table_region(scheme, kw):
     slots = 24_000_000                                  # 192 MB: 1.5 M lines
     n = int(slots * 0.85)
     idx = torch.arange(2 * n, dtype=torch.int64, device="cuda")
-    if kw == 64:
+    if kw >= 64:
         keys = dk.mix63_perm_dev(idx, 3)
     else:
         k = dk.mix32_perm_dev(idx, 3)
         keys = (k - ((k >> 31) << 32)).to(torch.int32)
+    if kw == 128:                                       # low words of all ones among them
+        keys = torch.stack([torch.where(idx % 5 == 0, torch.full_like(keys, -1), keys), keys], dim=1).contiguous()
     t = ht.HashTable(slots, scheme, kw)
     order = torch.randperm(n, device="cuda")
     first = keys[:n][order][:2_000_001]                 # a ragged tile
@@ -179,14 +180,15 @@ def test_large_batches_are_reordered_by_table_region(scheme, kw):
     t.insert(keys[:n][order][1_000_000:5_000_000])      # no flags
     every = torch.randperm(n, device="cuda")            # n > 2^24: a whole piece and the rest
     new = torch.empty(n, dtype=torch.uint8, device="cuda")
-    out = torch.empty(n, dtype=keys.dtype, device="cuda")
+    out = torch.empty_like(keys[:n])
     count = torch.zeros(1, dtype=torch.int64, device="cuda")
     ht.ht_find_or_put_append(t.handle, keys[:n][every], out, count, new)
     stored = torch.zeros(n, dtype=torch.bool, device="cuda")
     stored[order[:5_000_000]] = True
     assert torch.equal(new, (~stored[every]).to(torch.uint8))
     assert int(count) == n - 5_000_000
-    assert torch.equal(torch.sort(out[:int(count)])[0], torch.sort(keys[:n][~stored])[0])
+    own = (lambda x: x[:, 1]) if kw == 128 else (lambda x: x)       # the word that tells keys apart
+    assert torch.equal(torch.sort(own(out[:int(count)]))[0], torch.sort(own(keys[:n][~stored]))[0])
     found, _ = t.lookup(keys)
     assert torch.equal(found, (idx < n).to(torch.uint8))
     assert t.sync() == 0 and t.size() == n
