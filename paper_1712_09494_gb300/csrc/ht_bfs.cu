@@ -114,8 +114,9 @@ __global__ void bfs_advance_kernel(BfsCursor* __restrict__ c, unsigned long long
 // index space; each thread finds its exploration by binary search and
 // appends to that exploration's segment of the successor buffer.
 __global__ void __launch_bounds__(kBlock) multi_successors_kernel(const MultiDev m, uint64_t max_work) {
-    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-    multi::successors(m, max_work, uint64_t(blockIdx.x) * blockDim.x + threadIdx.x, stride);
+    __shared__ unsigned int s_off[multi::kExactTileExpl];
+    __shared__ PreparedModel s_model;
+    multi::successors<kBlock>(m, max_work, s_off, &s_model);
 }
 
 }  // namespace

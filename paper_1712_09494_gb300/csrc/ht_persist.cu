@@ -116,19 +116,22 @@ __device__ void place_initial_states(const MultiDev& m, uint64_t gtid, uint64_t 
 }
 
 // Cuckoo probe of one step over warps [gw] of [nwarps]: each warp takes a
-// contiguous range of the step's 32-key tiles (the TileMap numbering), one
-// key per lane, against the tile's exploration e.  A key is looked up at h_1, then (h_1 occupied by another
-// key) at h_2..h_k, then in the stash / overflow set when those are in use;
-// a key stored at h_j has h_1..h_(j-1) occupied, so an empty h_1 proves it
-// absent.  An absent key that saw an EMPTY slot stores itself there (a CAS
-// in slot order); one whose k slots are all full claims its key in e's
-// claim set, and the one claimant per distinct key joins the group's
-// winner list with its exploration, for a chain from h_1.  Every new key is
-// appended to e's states.
-constexpr int kWinStage = 64;            // staged winner records per warp
+// contiguous range of the step's 32-key tiles (the TileMap numbering), one key
+// per lane, against the tile's exploration e, a slot of each key a pass; keys
+// that meet another key's slot wait in the warp's queue for their next one, 32 a
+// pass, and the queue empties before the warp moves on to another exploration
+// (one tile at a time through all its slots: 25.4 ms of 256 explorations' 28;
+// now 19.8).  A key is settled by the slot that holds it or by the first
+// EMPTY one, else by the stash / overflow set when those are in use; a key
+// stored at h_j has h_1..h_(j-1) occupied, so an EMPTY slot proves it absent.
+// An absent key that saw an EMPTY slot stores itself there (a CAS in slot
+// order); one whose k slots are all full claims its key in e's claim set, and
+// the one claimant per distinct key joins the group's winner list with its
+// exploration, for a chain from h_1.  Every new key is appended to e's states.
+constexpr int kWinStage = 48;            // staged winner records per warp
 
 __device__ void cuckoo_probe_tiles(const MultiDev& m, const multi::TileMap& tm, uint64_t gw, uint64_t nwarps,
-                                   uint64_t* stage_buf, MultiWinner* wstage) {
+                                   uint64_t* stage_buf, MultiWinner* wstage, bucket::PendEntry* pend_buf) {
     constexpr int KW = 64;
     using K = Keys<KW>;
     uint32_t wpend = 0;
@@ -162,122 +165,104 @@ __device__ void cuckoo_probe_tiles(const MultiDev& m, const multi::TileMap& tm, 
     const uint64_t per = (tiles + nwarps - 1) / nwarps;
     const uint64_t t_begin = min(tiles, gw * per), t_end = min(tiles, t_begin + per);
     if (t_begin >= t_end) return;
-    multi::StateStage<kStageCap> stage(stage_buf);
+    multi::StateStage<bucket::kMultiStage> stage(stage_buf);
+    bucket::Pending queue(pend_buf);
     multi::TileCursor cur;
     cur.start(m, tm, t_begin);
     uint32_t e = cur.e;
     uint64_t cnt = 0;
     uint32_t stash_used = 0, ovf_used = 0;
+    unsigned long long stored = 0;             // keys stored by this warp's CASes in e's table
     auto load_desc = [&]() {
         cnt = multi::step_count(m, e);
         stash_used = __ldcg(&m.tables[e].ctr->stash_used);
         ovf_used = __ldcg(&m.tables[e].ctr->ovf_used);
     };
     load_desc();
-    uint32_t run_e = e;                        // keys stored by this warp's CASes, per run of e
-    unsigned long long run_n = 0;
     uint64_t next_key = __ldcg(reinterpret_cast<const unsigned long long*>(m.succ + cur.key_index(m, t_begin, lane)));
-    for (uint64_t tile = t_begin; tile < t_end; ++tile) {
-        const uint64_t cur_key = next_key;
-        if (tile >= cur.b1) {                          // into a later exploration's tiles
-            stage.flush(m, e);
-            cur.seek(m, tm, tile);
-            e = cur.e;
-            load_desc();
+    // Bounded: an iteration takes a tile or up to 32 queued keys, and a key is
+    // queued at most k - 1 times.
+    for (uint64_t tile = t_begin;;) {
+        const bool moves = tile >= t_end || tile >= cur.b1;    // done with exploration e's tiles
+        bucket::PendEntry d;
+        d.key = d.pos = d.sec = 0;
+        d.val = d.probe = 0;
+        bool ok;
+        if (queue.n >= 32 || (moves && queue.n)) {
+            ok = queue.pop(d);
+        } else {
+            if (moves) {
+                stage.flush(m, e);
+                if (lane == 0 && stored) atomicAdd(&m.tables[e].ctr->size, stored);
+                stored = 0;
+                if (tile >= t_end) break;
+                cur.seek(m, tm, tile);
+                e = cur.e;
+                load_desc();
+            }
+            d.key = K::keyof(next_key);
+            const bool mine = 32 * (tile - cur.b0) + lane < cnt;
+            ok = mine && !K::reserved(d.key);
+            if (mine && !ok) set_flag(m.tables[e].ctr, kFlagInvalidKey);
+            if (++tile < t_end) {
+                multi::TileCursor nx = cur;
+                nx.seek(m, tm, tile);
+                next_key = __ldcg(reinterpret_cast<const unsigned long long*>(m.succ + nx.key_index(m, tile, lane)));
+            }
+            if (!__any_sync(0xFFFFFFFFu, ok)) continue;
         }
-        const uint64_t i = 32 * (tile - cur.b0) + lane;
-        if (tile + 1 < t_end) {
-            multi::TileCursor nx = cur;
-            nx.seek(m, tm, tile + 1);
-            next_key = __ldcg(reinterpret_cast<const unsigned long long*>(m.succ + nx.key_index(m, tile + 1, lane)));
-        }
-        const bool mine = i < cnt;
-        if (!__any_sync(0xFFFFFFFFu, mine)) continue;
         const DevTable& t = m.tables[e];
-        const uint64_t key = mine ? K::keyof(cur_key) : 0;
-        const bool ok = mine && !K::reserved(key);
-        if (mine && !ok) set_flag(t.ctr, kFlagInvalidKey);
+        uint64_t at = hidx(d.key, t.seed[d.probe], t.nslots);
         uint64_t w = kEmpty;
-        if (ok) w = __ldcg(reinterpret_cast<const unsigned long long*>(t.slots + hidx(key, t.seed[0], t.nslots)));
-        bool found = ok && K::keyof(w) == key;
-        const bool more = ok && !found && !K::empty(w);
-        uint32_t start = 0;
-        // h_2..h_k one slot at a time, stopping at the key or at the first
-        // EMPTY slot (the key is not past it; a new key's chain starts
-        // there): the probe is bound by the random lines it reads.
-        bool go = more;
-        for (uint32_t a = 1; a < t.k && __any_sync(0xFFFFFFFFu, go); ++a) {
-            if (go) {
-                const uint64_t v = __ldcg(reinterpret_cast<const unsigned long long*>(t.slots + hidx(key, t.seed[a], t.nslots)));
-                if (K::keyof(v) == key) found = true;
-                else if (K::empty(v)) start = a;
-                go = !found && start == 0;
-            }
-        }
-        if ((stash_used | ovf_used) && ok && !found) {
+        if (ok) w = __ldcg(reinterpret_cast<const unsigned long long*>(t.slots + at));
+        const bool found = ok && K::keyof(w) == d.key;
+        bool miss = ok && !found && (K::empty(w) || d.probe + 1 >= t.k);
+        const bool waits = ok && !found && !miss;
+        if (miss && (stash_used | ovf_used)) {
             uint64_t sw;
-            found = find_spill<KW>(t, key, stash_used, ovf_used, &sw);
+            miss = !find_spill<KW>(t, d.key, stash_used, ovf_used, &sw);
         }
-        // An absent key that saw an EMPTY slot (h_1, or the first of
-        // h_2..h_k; with t.chain_h1 only h_1) stores itself there with a CAS
-        // from EMPTY, going on in slot order while the CAS returns another
-        // key; a CAS that returns the key means another copy stored it.  Only
-        // keys whose k slots are all full claim and run a chain.  (The
-        // argument is the single-table kernel's: nothing moves a key during
-        // the probe phase, the grid barrier ends it before any chain runs.)
+        if (waits) ++d.probe;
+        queue.push(waits, d);
+        // An absent key that saw an EMPTY slot (with t.chain_h1 only h_1)
+        // stores itself there with a CAS from EMPTY, going on in slot order
+        // while the CAS returns another key; a CAS that returns the key means
+        // another copy stored it.  Only keys whose k slots are all full claim
+        // and run a chain.  (The argument is the single-table kernel's: nothing
+        // moves a key during the probe phase, the grid barrier ends it before
+        // any chain runs.)
         bool placed = false;
-        bool pend = ok && !found && (!more || (start != 0 && !t.chain_h1));
-        bool claim = ok && !found && !pend;
-        uint32_t at = more ? start : 0u;
-        for (uint32_t pass = 0; pass < t.k && __any_sync(0xFFFFFFFFu, pend); ++pass) {
-            if (pend) {
-                const uint64_t cw = atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + hidx(key, t.seed[at], t.nslots)),
-                                              kEmpty, K::word(key, 0u));
-                if (cw == kEmpty) {
-                    placed = true;
-                    pend = false;
-                } else if (K::keyof(cw) == key) {
-                    found = true;                      // another copy stored it
-                    pend = false;
-                } else if (t.chain_h1 || at + 1 >= t.k) {
-                    claim = true;                      // every slot holds another key now
-                    pend = false;
-                } else {
-                    ++at;
-                }
+        bool cas = miss && K::empty(w) && (!t.chain_h1 || d.probe == 0);
+        bool claim = miss && !cas;
+        while (cas) {                          // bounded: on to the next of k slots
+            const uint64_t cw = atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + at), kEmpty, K::word(d.key, 0u));
+            cas = false;
+            if (cw == kEmpty) {
+                placed = true;
+            } else if (K::keyof(cw) == d.key) {
+                // another copy stored it
+            } else if (t.chain_h1 || d.probe + 1 >= t.k) {
+                claim = true;                  // every slot holds another key now
+            } else {
+                ++d.probe;
+                at = hidx(d.key, t.seed[d.probe], t.nslots);
+                cas = true;
             }
         }
-        // The stored keys count toward e's size, per run of tiles of e.
-        {
-            const unsigned pm = __ballot_sync(0xFFFFFFFFu, placed);
-            if (e != run_e) {
-                if (lane == 0 && run_n) atomicAdd(&m.tables[run_e].ctr->size, run_n);
-                run_e = e;
-                run_n = 0;
-            }
-            run_n += __popc(pm);
-        }
+        __syncwarp();
+        stored += __popc(__ballot_sync(0xFFFFFFFFu, placed));
         // In-batch dedup in e's claim set of the keys with every slot full:
         // the one claimant of each such key wins.
-        const bool need = claim;
         bool winner = placed;
         uint32_t spos = 0;
-        if (need) {
+        if (claim) {
             const DevScratch& sc = m.scratch[e];
-            spos = uint32_t(mix64(key ^ (t.aux_seed * 3 + 1)) & sc.mask);
-            const uint64_t sw = atomicCAS(reinterpret_cast<unsigned long long*>(sc.set + spos), kEmpty, key);
-            if (sw == kEmpty) {
-                winner = true;
-            } else if (K::keyof(sw) != key) {
-                uint32_t at = 0;
-                const uint32_t n = uint32_t(sc.mask + 1);
-                const int rc = lp_insert<KW>(sc.set, n, spos + 1 == n ? 0u : spos + 1, key, key, &at);
-                winner = rc == 1;
-                spos = at;
-                if (rc < 0) {                          // more distinct misses than the claim set holds
-                    set_flag(t.ctr, kFlagDropped);
-                    atomicAdd(&t.ctr->dropped, 1ull);
-                }
+            const int rc = lp_insert<KW>(sc.set, uint32_t(sc.mask + 1), mix64(d.key ^ (t.aux_seed * 3 + 1)) & sc.mask, d.key,
+                                         d.key, &spos);
+            winner = rc == 1;
+            if (rc < 0) {                      // more distinct misses than the claim set holds
+                set_flag(t.ctr, kFlagDropped);
+                atomicAdd(&t.ctr->dropped, 1ull);
             }
         }
         // Claim winners to the warp's stage of winner records (listed with
@@ -289,16 +274,14 @@ __device__ void cuckoo_probe_tiles(const MultiDev& m, const multi::TileMap& tm, 
             if (wpend + __popc(wm) > uint32_t(kWinStage)) flush_winners();
             if (listed) {
                 MultiWinner& wn = wstage[wpend + __popc(wm & ((1u << lane) - 1))];
-                wn.word = K::word(key, 0u);
+                wn.word = K::word(d.key, 0u);
                 wn.spos = spos;
                 wn.tag = e << 8;
             }
             wpend += __popc(wm);
         }
-        stage.push(winner, key, m, e);
+        stage.push(winner, d.key, m, e);
     }
-    if (lane == 0 && run_n) atomicAdd(&m.tables[run_e].ctr->size, run_n);
-    stage.flush(m, e);
     flush_winners();
 }
 
@@ -389,24 +372,26 @@ __device__ void cuckoo_insert_winners(const MultiDev& m, uint64_t gtid, uint64_t
 }
 
 // Resident blocks per SM the kernel is compiled for (registers): measured on
-// 256 explorations of 38 M states, the bucket kernel is fastest at 4 (20.0 ms;
-// 22.5 at 3, 28.7 at 2), the Cuckoo kernel at 3.
+// 256 explorations of 38 M states, both are fastest at 4 (bucket 20.0 ms, 22.5
+// at 3, 28.7 at 2; Cuckoo 28.2, 30.4 at 3, 32.1 at 5).
 #ifndef HT_PERSIST_MIN_BLOCKS_BUCKET
 #define HT_PERSIST_MIN_BLOCKS_BUCKET 4
 #endif
 #ifndef HT_PERSIST_MIN_BLOCKS_CUCKOO
-#define HT_PERSIST_MIN_BLOCKS_CUCKOO 3
+#define HT_PERSIST_MIN_BLOCKS_CUCKOO 4
 #endif
+
+static_assert(sizeof(PreparedModel) <= kBlock / 32 * bucket::kMultiStage * 8, "a model fits the stage");
 
 template <bool CUCKOO, int BS>
 __global__ void __launch_bounds__(kBlock, CUCKOO ? HT_PERSIST_MIN_BLOCKS_CUCKOO : HT_PERSIST_MIN_BLOCKS_BUCKET)
 multi_persistent_kernel(const __grid_constant__ MultiDev m, uint64_t budget, uint64_t max_steps, uint64_t max_work,
                         uint64_t max_tiles) {
-    __shared__ uint64_t s_new[kBlock / 32][CUCKOO ? kStageCap : bucket::kMultiStage];
+    __shared__ uint64_t s_new[kBlock / 32][bucket::kMultiStage];
     __shared__ unsigned long long sh[multi::kAdvShared];
     __shared__ unsigned int s_first[multi::kExactTileExpl + 1];
     __shared__ MultiWinner s_win[kBlock / 32][CUCKOO ? kWinStage : 1];
-    __shared__ bucket::PendEntry s_pend[CUCKOO ? 1 : kBlock / 32][CUCKOO ? 1 : bucket::kPend];
+    __shared__ bucket::PendEntry s_pend[kBlock / 32][bucket::kPend];
     __shared__ int s_ok;
     const uint64_t gtid = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const uint64_t nthreads = uint64_t(gridDim.x) * blockDim.x;
@@ -420,12 +405,13 @@ multi_persistent_kernel(const __grid_constant__ MultiDev m, uint64_t budget, uin
         if (blockIdx.x == 0) multi::advance<kBlock>(m, budget, sh);
         if (!grid_sync(m, &s_ok)) return;
         if (__ldcg(m.active) == 0) break;
-        multi::successors(m, max_work, gtid, nthreads);
+        // In memory that the find-or-put phase uses: the tile prefix, the new states' stage.
+        multi::successors<kBlock>(m, max_work, s_first, reinterpret_cast<PreparedModel*>(&s_new[0][0]));
         if (!grid_sync(m, &s_ok)) return;
         // Every block numbers the step's tiles over the successors made.
         const multi::TileMap tm = multi::tile_map<kBlock>(m, s_first, sh);
         if constexpr (CUCKOO) {
-            cuckoo_probe_tiles(m, tm, gw, nwarps, stage, s_win[threadIdx.x >> 5]);
+            cuckoo_probe_tiles(m, tm, gw, nwarps, stage, s_win[threadIdx.x >> 5], s_pend[threadIdx.x >> 5]);
             if (!grid_sync(m, &s_ok)) return;
             cuckoo_insert_winners(m, gtid, nthreads);
         } else {
