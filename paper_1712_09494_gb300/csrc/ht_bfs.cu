@@ -28,6 +28,7 @@ successors_kernel(const PreparedModel* __restrict__ model, const T* __restrict__
     // 16-byte states (models wider than 63 bits) use a half-size stage.
     constexpr int kStage = sizeof(T) > 8 ? kSuccStage / 2 : kSuccStage;
     using S = typename std::conditional<(sizeof(T) > 8), unsigned __int128, uint64_t>::type;
+    pdl_wait();
     __shared__ PreparedModel sm;
     __shared__ T s_out[kSuccBlock / 32][kStage];
     {
@@ -91,6 +92,7 @@ successors_kernel(const PreparedModel* __restrict__ model, const T* __restrict__
 __global__ void bfs_advance_kernel(BfsCursor* __restrict__ c, unsigned long long* __restrict__ count,
                                    unsigned long long* __restrict__ succ_count, uint64_t states_cap, uint32_t max_levels,
                                    uint64_t most) {
+    pdl_wait();
     *succ_count = 0;
     if (c->stop) return;
     const unsigned long long nh = *count, nd = nh - c->hi;
@@ -163,8 +165,7 @@ cudaError_t multi_successors(int, const MultiDev& m, uint64_t max_work, cudaStre
 
 cudaError_t bfs_advance(BfsCursor* c, unsigned long long* count, unsigned long long* succ_count, uint64_t states_cap,
                         uint32_t max_levels, uint64_t most, cudaStream_t s) {
-    bfs_advance_kernel<<<1, 1, 0, s>>>(c, count, succ_count, states_cap, max_levels, most);
-    return cudaGetLastError();
+    return launch_after(bfs_advance_kernel, 1, 1, 0, s, c, count, succ_count, states_cap, max_levels, most);
 }
 
 cudaError_t successors(int kw, const PreparedModel* model, const void* states, uint64_t n,
@@ -173,19 +174,18 @@ cudaError_t successors(int kw, const PreparedModel* model, const void* states, u
     ProfScope ps(kKSuccessors, s);
     if (kw == 32) {
         auto k = successors_kernel<uint32_t>;
-        k<<<launch_grid((const void*)k, kSuccBlock, n, kSuccBlock), kSuccBlock, 0, s>>>(
-            model, static_cast<const uint32_t*>(states), n, cur, static_cast<uint32_t*>(succ), cap, count, total);
-    } else if (kw == 128) {
+        return launch_after(k, launch_grid((const void*)k, kSuccBlock, n, kSuccBlock), kSuccBlock, 0, s, model,
+                            static_cast<const uint32_t*>(states), n, cur, static_cast<uint32_t*>(succ), cap, count, total);
+    }
+    if (kw == 128) {
         using U = unsigned __int128;
         auto k = successors_kernel<U>;
-        k<<<launch_grid((const void*)k, kSuccBlock, n, kSuccBlock), kSuccBlock, 0, s>>>(
-            model, static_cast<const U*>(states), n, cur, static_cast<U*>(succ), cap, count, total);
-    } else {
-        auto k = successors_kernel<uint64_t>;
-        k<<<launch_grid((const void*)k, kSuccBlock, n, kSuccBlock), kSuccBlock, 0, s>>>(
-            model, static_cast<const uint64_t*>(states), n, cur, static_cast<uint64_t*>(succ), cap, count, total);
+        return launch_after(k, launch_grid((const void*)k, kSuccBlock, n, kSuccBlock), kSuccBlock, 0, s, model,
+                            static_cast<const U*>(states), n, cur, static_cast<U*>(succ), cap, count, total);
     }
-    return cudaGetLastError();
+    auto k = successors_kernel<uint64_t>;
+    return launch_after(k, launch_grid((const void*)k, kSuccBlock, n, kSuccBlock), kSuccBlock, 0, s, model,
+                            static_cast<const uint64_t*>(states), n, cur, static_cast<uint64_t*>(succ), cap, count, total);
 }
 
 }  // namespace ht

@@ -121,6 +121,7 @@ bucket_fop_kernel(const __grid_constant__ DevTable t, const void* __restrict__ k
                   uint64_t n, const unsigned long long* __restrict__ d_n, uint8_t* __restrict__ is_new,
                   typename Keys<KW>::T* __restrict__ new_out, unsigned long long* __restrict__ new_count,
                   uint64_t new_cap) {
+    pdl_wait();
     if (d_n) n = min(n, uint64_t(__ldcg(d_n)));        // batch size produced on the device
     bucket_tiles<KW, BS, VALUES, APPEND, false, WHOLE, false>(t, keys, vals, n, is_new, nullptr, new_out, new_count, new_cap);
 }
@@ -133,6 +134,7 @@ template <int KW, int BS, bool VALUES, bool AHEAD>
 __global__ void __launch_bounds__(kBlock, kWholeBlocks)
 bucket_lookup_kernel(const __grid_constant__ DevTable t, const void* __restrict__ keys, uint64_t n,
                      uint32_t* __restrict__ vals, uint8_t* __restrict__ found) {
+    pdl_wait();
     bucket_tiles<KW, BS, VALUES, false, true, true, AHEAD>(t, keys, nullptr, n, found, vals, nullptr, nullptr, 0);
 }
 
@@ -154,7 +156,7 @@ cudaError_t launch_fop(const DevTable& t, const void* keys, const uint32_t* vals
     using T = typename Keys<KW>::T;
     auto k = vals ? bucket_fop_kernel<KW, BS, KW == 32, false, WHOLE>
              : new_out ? bucket_fop_kernel<KW, BS, false, true, WHOLE> : bucket_fop_kernel<KW, BS, false, false, WHOLE>;
-    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, keys, vals, n, d_n,
+    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, w, t, keys, vals, n, d_n,
                       is_new, static_cast<T*>(new_out), new_count, new_cap);
 }
 
@@ -163,7 +165,7 @@ cudaError_t launch_lookup(const DevTable& t, const void* keys, uint64_t n, uint3
                           uint8_t* found, cudaStream_t s, const L2Window& w) {
     auto k = past_l2(t) ? (vals ? bucket_lookup_kernel<KW, BS, true, true> : bucket_lookup_kernel<KW, BS, false, true>)
                         : (vals ? bucket_lookup_kernel<KW, BS, true, false> : bucket_lookup_kernel<KW, BS, false, false>);
-    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, keys, n, vals, found);
+    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, w, t, keys, n, vals, found);
 }
 
 // Multi-table find-or-put of one step (the body is shared with the

@@ -80,6 +80,7 @@ __device__ __forceinline__ void empty_table(const DevTable& t, uint32_t slot_wor
 // MB, then by the stores.
 __global__ void __launch_bounds__(kBlock)
 clear_kernel(const __grid_constant__ DevTable t, uint32_t slot_words, uint32_t ovf_words) {
+    pdl_wait();
     empty_table(t, slot_words, ovf_words, uint64_t(blockIdx.x) * blockDim.x + threadIdx.x,
                 uint64_t(gridDim.x) * blockDim.x);
 }
@@ -338,9 +339,9 @@ cudaError_t fill_words(uint64_t* p, uint64_t n, uint64_t v, cudaStream_t s) {
 cudaError_t clear_words(const DevTable& t, uint32_t slot_words, uint32_t ovf_words, cudaStream_t s) {
     ProfScope ps(kKClear, s);
     auto k = clear_kernel;
-    // At least four 32-byte stores a thread: a 512 KB table takes 16 blocks.
-    k<<<launch_grid((const void*)k, kBlock, t.nslots * slot_words, 16 * kBlock), kBlock, 0, s>>>(t, slot_words, ovf_words);
-    return cudaGetLastError();
+    // At least one 32-byte store a thread: a 512 KB table takes 64 blocks.
+    return launch_after(k, launch_grid((const void*)k, kBlock, t.nslots * slot_words, 4 * kBlock), kBlock, 0, s, t,
+                        slot_words, ovf_words);
 }
 
 cudaError_t clear_many(const DevTable* tables, uint32_t n, cudaStream_t s) {

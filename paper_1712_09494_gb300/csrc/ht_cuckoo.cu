@@ -120,6 +120,7 @@ cuckoo_probe_kernel(const __grid_constant__ DevTable t, const __grid_constant__ 
                     const unsigned long long* __restrict__ d_n, uint64_t off,
                     uint8_t* __restrict__ out_flag, uint32_t* __restrict__ out_val, bool list_stored) {
     using K = Keys<KW>;
+    pdl_wait();
     if (d_n) {                                   // batch size produced on the device
         const uint64_t total = __ldcg(d_n);
         n = total > off ? min(n, total - off) : 0;
@@ -327,6 +328,7 @@ __global__ void __launch_bounds__(kBlock, 3)
 cuckoo_lookup_kernel(const __grid_constant__ DevTable t, const void* __restrict__ keys, uint64_t n,
                      uint8_t* __restrict__ found_out, uint32_t* __restrict__ val_out) {
     using K = Keys<KW>;
+    pdl_wait();
     const uint32_t stash_used = __ldcg(&t.ctr->stash_used);
     const uint32_t ovf_used = __ldcg(&t.ctr->ovf_used);
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
@@ -409,6 +411,7 @@ cuckoo_insert_kernel(const DevTable t, const DevScratch sc, uint32_t parity, uin
                      typename Keys<KW>::T* __restrict__ new_out, unsigned long long* __restrict__ new_count,
                      uint64_t new_cap) {
     using K = Keys<KW>;
+    pdl_wait();
     const uint64_t count = min(uint64_t(__ldcg(&t.ctr->winners[parity])), max_winners);
     // The other parity's list was consumed by the previous insert kernel on
     // this stream; reset its counter for the next probe kernel.
@@ -530,7 +533,7 @@ cudaError_t cuckoo_probe(int kw, const DevTable& t, const DevScratch& sc, uint32
 #define L(KW, V)                                                                                        \
     {                                                                                                   \
         auto k = past_l2 ? cuckoo_probe_kernel<KW, V, false, true> : cuckoo_probe_kernel<KW, V, false, false>; \
-        return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, sc, parity, keys, vals, \
+        return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, w, t, sc, parity, keys, vals, \
                           n, d_n, off, is_new, (uint32_t*)nullptr, list_stored);                        \
     }
     if (kw == 32) {
@@ -547,7 +550,7 @@ cudaError_t cuckoo_insert(int kw, const DevTable& t, const DevScratch& sc, uint3
 #define L(KW, A)                                                                                        \
     {                                                                                                   \
         auto k = cuckoo_insert_kernel<KW, A>;                                                           \
-        return launch_win(k, launch_blocks((const void*)k, kBlock), kBlock, s, w, t, sc, parity, max_winners, \
+        return launch_win(k, launch_grid((const void*)k, kBlock, max_winners, kBlock), kBlock, 0, s, w, t, sc, parity, max_winners, \
                           static_cast<typename Keys<KW>::T*>(new_out), new_count, new_cap);             \
     }
     if (kw == 32) {
@@ -563,11 +566,11 @@ cudaError_t cuckoo_lookup(int kw, const DevTable& t, const void* keys, uint64_t 
     ProfScope ps(kKCuckooLookup, s);
     if (t.nslots * 8 <= l2_bytes()) {
         auto k = kw == 32 ? cuckoo_lookup_kernel<32> : cuckoo_lookup_kernel<64>;
-        return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, keys, n, found, vals);
+        return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, w, t, keys, n, found, vals);
     }
     DevScratch none{};
     auto k = kw == 32 ? cuckoo_probe_kernel<32, false, true, true> : cuckoo_probe_kernel<64, false, true, true>;
-    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, s, w, t, none, 0u, keys,
+    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, w, t, none, 0u, keys,
                       (const uint32_t*)nullptr, n, (const unsigned long long*)nullptr, uint64_t(0), found, vals, false);
 }
 

@@ -363,28 +363,43 @@ struct L2Window {
 // device maximum; hit < 1 when the range is larger than that.
 L2Window l2_window(const void* base, size_t bytes);
 
+// Starts a kernel early: programmatic stream serialisation lets its blocks be
+// placed as those of the kernel before it in the stream end, and pdl_wait(), the
+// kernel's first statement, holds them until that kernel has ended and its
+// writes are visible.  Back to back, a small clear takes 1.9 us instead of 4.2, a
+// find-or-put of 2^14 stored keys 2.8 instead of 4.2, a small exploration 1.31
+// ms instead of 1.45.  (Triggering the next kernel at the start of each instead
+// of by its end gains nothing more: its blocks then hold what this one's need.)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 template <typename... KArgs, typename... Args>
-cudaError_t launch_win(void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, const L2Window& w,
+cudaError_t launch_win(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, const L2Window& w,
                        Args&&... args) {
-    if (!w.bytes) {
-        kernel<<<grid, block, 0, s>>>(std::forward<Args>(args)...);
-        return cudaGetLastError();
-    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeAccessPolicyWindow;
-    at[0].val.accessPolicyWindow.base_ptr = const_cast<void*>(w.base);
-    at[0].val.accessPolicyWindow.num_bytes = w.bytes;
-    at[0].val.accessPolicyWindow.hitRatio = w.hit;
-    at[0].val.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
-    at[0].val.accessPolicyWindow.missProp = cudaAccessPropertyStreaming;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    if (w.bytes) {
+        at[1].id = cudaLaunchAttributeAccessPolicyWindow;
+        at[1].val.accessPolicyWindow.base_ptr = const_cast<void*>(w.base);
+        at[1].val.accessPolicyWindow.num_bytes = w.bytes;
+        at[1].val.accessPolicyWindow.hitRatio = w.hit;
+        at[1].val.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
+        at[1].val.accessPolicyWindow.missProp = cudaAccessPropertyStreaming;
+    }
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = w.bytes ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+// The same without a window.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_after(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, Args&&... args) {
+    return launch_win(kernel, grid, block, smem, s, L2Window(), std::forward<Args>(args)...);
 }
 
 // ---------------------------------------------------------------------------

@@ -217,6 +217,7 @@ template <bool LOOKUP>
 __global__ void __launch_bounds__(kBlock, 3)
 long_bucket_kernel(const __grid_constant__ DevTable t, const uint64_t* __restrict__ keys, uint64_t n,
                    uint8_t* __restrict__ out, bool ahead) {
+    pdl_wait();
     const uint32_t W = t.words, RW = t.row_words;
     const int lane = threadIdx.x & 31;
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
@@ -369,6 +370,7 @@ template <bool LOOKUP>
 __global__ void __launch_bounds__(kBlock)
 long_cuckoo_probe_kernel(const DevTable t, const DevScratch sc, uint32_t parity, const uint64_t* __restrict__ keys,
                          uint64_t n, uint8_t* __restrict__ out) {
+    pdl_wait();
     const uint32_t W = t.words, RW = t.row_words;
     const uint32_t ovf_used = __ldcg(&t.ctr->ovf_used);
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
@@ -498,6 +500,7 @@ long_cuckoo_probe_kernel(const DevTable t, const DevScratch sc, uint32_t parity,
 __global__ void __launch_bounds__(kBlock)
 long_cuckoo_insert_kernel(const DevTable t, const DevScratch sc, uint32_t parity, uint64_t max_winners) {
     constexpr int U = 4;
+    pdl_wait();
     const uint64_t count = min(uint64_t(__ldcg(&t.ctr->winners[parity])), max_winners);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         t.ctr->winners[parity ^ 1u] = 0;
@@ -637,35 +640,31 @@ cudaError_t long_find_or_put(const DevTable& t, const void* keys, uint64_t n, ui
     if (!n) return cudaSuccess;
     ProfScope ps(kKBucketFop, s);
     auto k = long_bucket_kernel<false>;
-    k<<<launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s>>>(t, static_cast<const uint64_t*>(keys), n, is_new,
-                                                                       false);
-    return cudaGetLastError();
+    return launch_after(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, t, static_cast<const uint64_t*>(keys),
+                        n, is_new, false);
 }
 
 cudaError_t long_lookup(const DevTable& t, const void* keys, uint64_t n, uint8_t* found, cudaStream_t s) {
     if (!n) return cudaSuccess;
     ProfScope ps(kKBucketLookup, s);
     auto k = long_bucket_kernel<true>;
-    k<<<launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s>>>(t, static_cast<const uint64_t*>(keys), n, found,
-                                                                       t.nslots * 8 > l2_bytes());
-    return cudaGetLastError();
+    return launch_after(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, t, static_cast<const uint64_t*>(keys),
+                        n, found, t.nslots * 8 > l2_bytes());
 }
 
 cudaError_t long_cuckoo_probe(const DevTable& t, const DevScratch& sc, uint32_t parity, const void* keys, uint64_t n,
                               uint8_t* is_new, cudaStream_t s) {
     ProfScope ps(kKCuckooProbe, s);
     auto k = long_cuckoo_probe_kernel<false>;
-    k<<<launch_blocks((const void*)k, kBlock), kBlock, 0, s>>>(t, sc, parity, static_cast<const uint64_t*>(keys), n,
-                                                              is_new);
-    return cudaGetLastError();
+    return launch_after(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, t, sc, parity,
+                        static_cast<const uint64_t*>(keys), n, is_new);
 }
 
 cudaError_t long_cuckoo_insert(const DevTable& t, const DevScratch& sc, uint32_t parity, uint64_t max_winners,
                                cudaStream_t s) {
     ProfScope ps(kKCuckooInsert, s);
     auto k = long_cuckoo_insert_kernel;
-    k<<<launch_blocks((const void*)k, kBlock), kBlock, 0, s>>>(t, sc, parity, max_winners);
-    return cudaGetLastError();
+    return launch_after(k, launch_grid((const void*)k, kBlock, max_winners, kBlock), kBlock, 0, s, t, sc, parity, max_winners);
 }
 
 cudaError_t long_cuckoo_lookup(const DevTable& t, const void* keys, uint64_t n, uint8_t* found, cudaStream_t s) {
@@ -673,9 +672,8 @@ cudaError_t long_cuckoo_lookup(const DevTable& t, const void* keys, uint64_t n, 
     ProfScope ps(kKCuckooLookup, s);
     DevScratch none{};
     auto k = long_cuckoo_probe_kernel<true>;
-    k<<<launch_blocks((const void*)k, kBlock), kBlock, 0, s>>>(t, none, 0u, static_cast<const uint64_t*>(keys), n,
-                                                              found);
-    return cudaGetLastError();
+    return launch_after(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, t, none, 0u,
+                        static_cast<const uint64_t*>(keys), n, found);
 }
 
 cudaError_t long_export(const DevTable& t, bool cuckoo, void* keys, unsigned long long* count, uint64_t cap,

@@ -34,6 +34,7 @@ __global__ void __launch_bounds__(kPartThreads)
 part_count_kernel(const T* __restrict__ keys, uint64_t n, const unsigned long long* __restrict__ d_n, uint64_t seed,
                   int shift, unsigned int* __restrict__ hist) {
     __shared__ unsigned int s_cnt[kMaxRegions];
+    pdl_wait();
     if (d_n) n = min(n, uint64_t(__ldcg(d_n)));
     for (int i = threadIdx.x; i < kMaxRegions; i += kPartThreads) s_cnt[i] = 0;
     __syncthreads();
@@ -71,6 +72,7 @@ part_move_kernel(const T* __restrict__ keys, uint64_t n, const unsigned long lon
     __shared__ unsigned int s_first[kMaxRegions];         // the region's start in out
     __shared__ unsigned int s_at[kMaxRegions];            // this tile's run in out
     __shared__ unsigned int s_warp[kMaxRegions / 32];
+    pdl_wait();
     if (d_n) n = min(n, uint64_t(__ldcg(d_n)));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // Exclusive scan of one value per region (threads < kMaxRegions).
@@ -147,6 +149,7 @@ part_back_kernel(const uint8_t* __restrict__ from, const uint16_t* __restrict__ 
                  uint32_t regions, uint64_t n, uint8_t* __restrict__ to) {
     __shared__ __align__(16) uint8_t s_out[kPartTile];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pdl_wait();
     for (uint64_t base = uint64_t(blockIdx.x) * kPartTile; base < n; base += uint64_t(gridDim.x) * kPartTile) {
         for (uint32_t r = warp; r < regions; r += kPartThreads / 32) {
             const uint2 run = runs[base / kPartTile * regions + r];
@@ -172,14 +175,15 @@ cudaError_t part_run(const T* keys, uint64_t n, const unsigned long long* d_n, u
     cudaError_t e = cudaMemsetAsync(ctl, 0, 2 * kMaxRegions * sizeof(unsigned int), s);
     if (e != cudaSuccess) return e;
     auto c = part_count_kernel<T>;
-    c<<<launch_grid((const void*)c, kPartThreads, n, kPartTile), kPartThreads, 0, s>>>(keys, n, d_n, seed, shift, ctl);
+    e = launch_after(c, launch_grid((const void*)c, kPartThreads, n, kPartTile), kPartThreads, 0, s, keys, n, d_n, seed,
+                     shift, ctl);
+    if (e != cudaSuccess) return e;
     auto k = loc ? part_move_kernel<T, true> : part_move_kernel<T, false>;
     const size_t smem = kPartTile * (sizeof(T) + 1 + (loc ? 2 : 0));
     e = allow_smem((const void*)k, smem);
     if (e != cudaSuccess) return e;
-    k<<<launch_grid((const void*)k, kPartThreads, n, kPartTile, smem), kPartThreads, smem, s>>>(
-        keys, n, d_n, seed, shift, ctl, ctl + kMaxRegions, out, loc, runs);
-    return cudaGetLastError();
+    return launch_after(k, launch_grid((const void*)k, kPartThreads, n, kPartTile, smem), kPartThreads, smem, s, keys, n,
+                        d_n, seed, shift, ctl, ctl + kMaxRegions, out, loc, runs);
 }
 
 }  // namespace
@@ -200,9 +204,8 @@ cudaError_t partition_back(const uint8_t* from, const uint16_t* loc, const void*
                            cudaStream_t s) {
     ProfScope ps(kKPartition, s);
     auto k = part_back_kernel;
-    k<<<launch_grid((const void*)k, kPartThreads, n, kPartTile), kPartThreads, 0, s>>>(
-        from, loc, static_cast<const uint2*>(runs), 1u << bits, n, to);
-    return cudaGetLastError();
+    return launch_after(k, launch_grid((const void*)k, kPartThreads, n, kPartTile), kPartThreads, 0, s, from, loc,
+                        static_cast<const uint2*>(runs), 1u << bits, n, to);
 }
 
 }  // namespace ht

@@ -253,6 +253,7 @@ __global__ void __launch_bounds__(kBlock, HALF ? 4 : 3)
 wide_kernel(const __grid_constant__ DevTable t, const ulonglong2* __restrict__ keys, uint64_t n,
             const unsigned long long* __restrict__ d_n, uint8_t* __restrict__ out,
             ulonglong2* __restrict__ new_out, unsigned long long* __restrict__ new_count, uint64_t new_cap, bool ahead) {
+    pdl_wait();
     if (d_n) n = min(n, uint64_t(__ldcg(d_n)));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
@@ -399,6 +400,7 @@ __global__ void __launch_bounds__(kBlock, HT_WIDE_PROBE_MIN_BLOCKS)
 wide_cuckoo_probe_kernel(const DevTable t, const DevScratch sc, uint32_t parity, const ulonglong2* __restrict__ keys,
                          uint64_t n, const unsigned long long* __restrict__ d_n, uint64_t off,
                          uint8_t* __restrict__ out, bool list_stored) {
+    pdl_wait();
     if (d_n) {
         const uint64_t total = __ldcg(d_n);
         n = total > off ? min(n, total - off) : 0;
@@ -615,6 +617,7 @@ __global__ void __launch_bounds__(kBlock)
 wide_cuckoo_insert_kernel(const DevTable t, const DevScratch sc, uint32_t parity, uint64_t max_winners,
                           ulonglong2* __restrict__ new_out, unsigned long long* __restrict__ new_count,
                           uint64_t new_cap) {
+    pdl_wait();
     const uint64_t count = min(uint64_t(__ldcg(&t.ctr->winners[parity])), max_winners);
     if (blockIdx.x == 0 && threadIdx.x == 0) t.ctr->winners[parity ^ 1u] = 0;
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
@@ -723,10 +726,9 @@ cudaError_t launch_wide(const DevTable& t, const void* keys, uint64_t n, const u
                         uint8_t* out, void* new_out, unsigned long long* new_count, uint64_t new_cap,
                         cudaStream_t s) {
     auto k = wide_kernel<LOOKUP, APPEND, HALF>;
-    k<<<launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s>>>(
-        t, static_cast<const ulonglong2*>(keys), n, d_n, out, static_cast<ulonglong2*>(new_out), new_count, new_cap,
-        t.nslots * 16 > l2_bytes());
-    return cudaGetLastError();
+    return launch_after(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, t,
+                        static_cast<const ulonglong2*>(keys), n, d_n, out, static_cast<ulonglong2*>(new_out), new_count,
+                        new_cap, t.nslots * 16 > l2_bytes());
 }
 
 // As for 64-bit buckets: smaller batches are read a bucket at a time.
@@ -758,24 +760,17 @@ cudaError_t wide_cuckoo_probe(const DevTable& t, const DevScratch& sc, uint32_t 
                               bool list_stored) {
     ProfScope ps(kKCuckooProbe, s);
     auto k = wide_cuckoo_probe_kernel<false>;
-    k<<<launch_blocks((const void*)k, kBlock), kBlock, 0, s>>>(t, sc, parity, static_cast<const ulonglong2*>(keys),
-                                                              n, d_n, off, is_new, list_stored);
-    return cudaGetLastError();
+    return launch_after(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, t, sc, parity,
+                        static_cast<const ulonglong2*>(keys), n, d_n, off, is_new, list_stored);
 }
 
 cudaError_t wide_cuckoo_insert(const DevTable& t, const DevScratch& sc, uint32_t parity, void* new_out,
                                unsigned long long* new_count, uint64_t new_cap, uint64_t max_winners,
                                cudaStream_t s) {
     ProfScope ps(kKCuckooInsert, s);
-    if (new_out) {
-        auto k = wide_cuckoo_insert_kernel<true>;
-        k<<<launch_blocks((const void*)k, kBlock), kBlock, 0, s>>>(t, sc, parity, max_winners,
-                                                                  static_cast<ulonglong2*>(new_out), new_count, new_cap);
-    } else {
-        auto k = wide_cuckoo_insert_kernel<false>;
-        k<<<launch_blocks((const void*)k, kBlock), kBlock, 0, s>>>(t, sc, parity, max_winners, nullptr, nullptr, 0);
-    }
-    return cudaGetLastError();
+    auto k = new_out ? wide_cuckoo_insert_kernel<true> : wide_cuckoo_insert_kernel<false>;
+    return launch_after(k, launch_grid((const void*)k, kBlock, max_winners, kBlock), kBlock, 0, s, t, sc, parity,
+                        max_winners, static_cast<ulonglong2*>(new_out), new_count, new_cap);
 }
 
 cudaError_t wide_cuckoo_lookup(const DevTable& t, const void* keys, uint64_t n, uint8_t* found, cudaStream_t s) {
@@ -783,9 +778,9 @@ cudaError_t wide_cuckoo_lookup(const DevTable& t, const void* keys, uint64_t n, 
     ProfScope ps(kKCuckooLookup, s);
     DevScratch none{};
     auto k = wide_cuckoo_probe_kernel<true>;
-    k<<<launch_blocks((const void*)k, kBlock), kBlock, 0, s>>>(t, none, 0u, static_cast<const ulonglong2*>(keys), n,
-                                                              nullptr, 0, found, false);
-    return cudaGetLastError();
+    return launch_after(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, t, none, 0u,
+                        static_cast<const ulonglong2*>(keys), n, (const unsigned long long*)nullptr, uint64_t(0), found,
+                        false);
 }
 
 cudaError_t wide_export(const DevTable& t, void* keys, unsigned long long* count, uint64_t cap, cudaStream_t s) {
