@@ -47,3 +47,26 @@ def test_levels_ahead_of_the_host(scheme, params, max_levels):
         short, got = ht.ht_bfs(t.handle, hm, 0, max_levels, states[:cap])
         assert short.complete == 0 and short.states == cap and got == want[:short.levels]
         assert bool((states[cap:] == -1).all())
+
+
+@pytest.mark.parametrize("width", [32, 64])
+def test_large_levels_are_reordered_by_region(width):
+    """A table past L2 with levels large enough for their successors to be reordered by table region (their number
+    known on the device only), every state with the most successors a state can have; against smaller tables."""
+    m = ss.random_model(5, C=8, L=8, R=6, deg_lo=3, deg_hi=3)
+    hm = ht.make_model(m.C, m.bits, m.deg, m.tgt, m.lab, m.pairs)
+    dt = torch.int32 if width == 32 else torch.int64
+    total = 6 ** 8
+    runs = []
+    for scheme, slots in (("bucket", 24_000_000), ("cuckoo", int(total / 0.8)), ("bucket", int(total / 0.8))):
+        t = ht.HashTable(slots, scheme, width)
+        states = torch.empty(total + 10, dtype=dt, device="cuda")
+        res, sizes = ht.ht_bfs(t.handle, hm, 0, 4096, states)
+        assert res.complete == 1 and res.states == total and t.size() == total
+        at, levels = 0, []
+        for n in sizes:
+            levels.append(torch.sort(states[at:at + n])[0])
+            at += n
+        runs.append((res.successors, sizes, torch.cat(levels)))
+    for r in runs[1:]:
+        assert r[0] == runs[0][0] and r[1] == runs[0][1] and torch.equal(r[2], runs[0][2])
