@@ -571,7 +571,9 @@ ht_status ht_probe_random_read(const void* d_buf, uint64_t bytes, uint32_t gran,
  * (the words the scheme's kernels read and claim; 8 or 16 bytes per slot,
  * laid out as ht_create describes).  For tests and tools that inspect the
  * words or prepare a slot state on purpose; a caller that writes them must
- * keep the table's invariants.  Host only; HT_ERR_INVALID for NULL. */
+ * keep the table's invariants (for buckets of 32- and 64-bit keys: a key is in
+ * the first 32-byte sector of its bucket, from the one its search starts in,
+ * that had a free slot when it was stored).  Host only; HT_ERR_INVALID for NULL. */
 ht_status ht_table_words(const ht_table* t, void** d_slots, uint64_t* bytes);
 
 /* Random read-modify-write probe (not part of the hash table): n_access

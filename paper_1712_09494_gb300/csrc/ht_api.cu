@@ -47,7 +47,7 @@ void derive_seeds(ht_table* t) {
 bool is_long(uint32_t kw) { return kw > 128; }
 
 BucketCfg bucket_cfg(const ht_table* t) {
-    return BucketCfg{int(t->kw), int(t->p.bucket_slots), int(t->p.lanes_per_key)};
+    return BucketCfg{int(t->kw), int(t->p.bucket_slots)};
 }
 
 cudaStream_t as_stream(void* s) { return static_cast<cudaStream_t>(s); }
@@ -138,12 +138,16 @@ struct PartScratch {
 };
 
 // The table keeps one block of that scratch, freed with it, that grows to the
-// largest piece seen.  Null when it cannot be had (no memory, or a stream
-// capture, which must not allocate): the batch then goes in its own order.
+// largest piece seen.  Null when it cannot be had: the batch then goes in its own
+// order.  So it does during a stream capture: a graph must not hold the address
+// of a block that a later, larger batch replaces.
 void* part_scratch(ht_table* t, size_t need, cudaStream_t s) {
-    if (t->part_bytes >= need) return t->part;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return nullptr;
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();                          // not an error of this call
+        return nullptr;
+    }
+    if (t->part_bytes >= need) return t->part;
     if (t->part) cudaFreeAsync(t->part, s);
     t->part = nullptr;
     t->part_bytes = 0;
@@ -366,7 +370,7 @@ bool valid_params(ht_scheme scheme, const ht_params& p) {
         if (p.num_hashes < 1 || p.num_hashes > uint32_t(kMaxHashes)) return false;
         if (p.bucket_slots != 8 && p.bucket_slots != 16 && p.bucket_slots != 32) return false;
         const uint32_t g = p.lanes_per_key;
-        // (bucket_slots, lanes) pairs the bucket kernels are instantiated for.
+        // The (bucket_slots, lanes) pairs that are accepted.
         static const uint32_t kShapes[][2] = {{8, 2}, {8, 4}, {8, 8}, {16, 2}, {16, 4}, {16, 8},
                                               {16, 16}, {32, 4}, {32, 8}, {32, 16}, {32, 32}};
         bool shape_ok = false;
@@ -744,7 +748,7 @@ ht_status ht_multi_find_or_put(ht_table* const* tables, uint32_t ntables, const 
         const BucketCfg c = bucket_cfg(t);
         PackGroup* gp = nullptr;
         for (auto& gr : groups)
-            if (gr.cfg.kw == c.kw && gr.cfg.bucket_slots == c.bucket_slots && gr.cfg.lanes == c.lanes) gp = &gr;
+            if (gr.cfg.kw == c.kw && gr.cfg.bucket_slots == c.bucket_slots) gp = &gr;
         if (!gp) {
             groups.emplace_back();
             gp = &groups.back();

@@ -52,12 +52,10 @@ namespace {
 
 constexpr int kU = 4;                   // eviction chains in flight per thread (insert)
 constexpr int kStage = 96;              // staged winners per warp
-#ifndef HT_CUCKOO_PROBE_BLOCKS
-#define HT_CUCKOO_PROBE_BLOCKS 4
-#endif
-#ifndef HT_CUCKOO_LOOKUP_BLOCKS
-#define HT_CUCKOO_LOOKUP_BLOCKS 5
-#endif
+// Resident blocks per SM that the probe is compiled for: find-or-put 4 (fill of
+// 2^27 keys, not reordered, 14.4 ms; 14.5 at 3, 14.7 at 5), lookup 5.
+constexpr int kProbeBlocks = 4;
+constexpr int kLookupBlocks = 5;
 
 // Adds the block's per-warp sums (held by each warp's lane 0) to N table
 // counters with one atomic per counter and block, not per warp: the last
@@ -112,9 +110,13 @@ __device__ __noinline__ bool spill_holds(const DevTable& t, uint64_t key, uint32
 // lane of a pass has a slot to read, whatever the other keys' paths.  A key is
 // settled by the slot that holds it or by the first EMPTY one (a key never sits
 // past an empty slot of its own), 1.63 slots per key over a fill to load 0.8.
+// Past L2 bound by random lines (27 G slot reads and 11 G CASes a second; the
+// same time with four keys per thread in lock step, at twice the registers);
+// in region order 7.8 instead of 10.8 ms of the 2^27-key fill; in L2 a replay
+// of 10^8 keys of 100 occurrences takes 1.87 ms (2.16 in lock step).
 // AHEAD: tables past L2; the next tile's first slots are touched a tile ahead.
 template <int KW, bool VALUES, bool LOOKUP, bool AHEAD>
-__global__ void __launch_bounds__(kBlock, LOOKUP ? HT_CUCKOO_LOOKUP_BLOCKS : HT_CUCKOO_PROBE_BLOCKS)
+__global__ void __launch_bounds__(kBlock, LOOKUP ? kLookupBlocks : kProbeBlocks)
 cuckoo_probe_kernel(const __grid_constant__ DevTable t, const __grid_constant__ DevScratch sc, uint32_t parity,
                     const void* __restrict__ keys, const uint32_t* __restrict__ vals, uint64_t n,
                     const unsigned long long* __restrict__ d_n, uint64_t off,

@@ -409,7 +409,6 @@ cudaError_t launch_after(void (*kernel)(KArgs...), int grid, int block, size_t s
 struct BucketCfg {
     int kw;
     int bucket_slots;
-    int lanes;
 };
 
 // d_n (nullable): the batch size lives on the device; n is then an upper bound.

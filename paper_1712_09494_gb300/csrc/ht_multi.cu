@@ -295,11 +295,10 @@ ht_status ht_multi_create_ex(uint32_t count, const ht_model* h_models, const uin
         const ht_scheme sch = table_scheme(m->tables[e]);
         BucketCfg c = table_bucket_cfg(m->tables[e]);
         c.kw = 64;
-        if (sch == HT_CUCKOO) c.bucket_slots = c.lanes = 0;    // no bucket shape
+        if (sch == HT_CUCKOO) c.bucket_slots = 0;    // no bucket shape
         Group* g = nullptr;
         for (auto& x : m->groups)
-            if (x.scheme == sch && x.cfg.kw == c.kw && x.cfg.bucket_slots == c.bucket_slots && x.cfg.lanes == c.lanes)
-                g = &x;
+            if (x.scheme == sch && x.cfg.kw == c.kw && x.cfg.bucket_slots == c.bucket_slots) g = &x;
         if (!g) {
             m->groups.emplace_back();
             g = &m->groups.back();
