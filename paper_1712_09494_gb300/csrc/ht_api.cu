@@ -54,7 +54,10 @@ cudaStream_t as_stream(void* s) { return static_cast<cudaStream_t>(s); }
 
 ht_status cuda_status(cudaError_t e) {
     if (e == cudaSuccess) return HT_OK;
-    if (e == cudaErrorMemoryAllocation) return HT_ERR_OOM;
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();           // reported here: not the next launch's error too
+        return HT_ERR_OOM;
+    }
     return HT_ERR_CUDA;
 }
 
@@ -272,12 +275,12 @@ ht_status rebuild(ht_table* t, cudaStream_t s) {
     HT_TRY(cudaMalloc(&keys, std::max<uint64_t>(n, 1) * (t->kw / 8)));
     if (t->kw == 32 && cudaMalloc(&vals, std::max<uint64_t>(n, 1) * 4) != cudaSuccess) {
         cudaFree(keys);
-        return HT_ERR_OOM;
+        return cuda_status(cudaErrorMemoryAllocation);
     }
     if (cudaMalloc(&cnt, sizeof(unsigned long long)) != cudaSuccess) {
         cudaFree(keys);
         cudaFree(vals);
-        return HT_ERR_OOM;
+        return cuda_status(cudaErrorMemoryAllocation);
     }
     st = HT_OK;
     do {

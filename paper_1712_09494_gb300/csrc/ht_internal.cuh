@@ -393,7 +393,9 @@ cudaError_t launch_win(void (*kernel)(KArgs...), int grid, int block, size_t sme
     }
     cfg.attrs = at;
     cfg.numAttrs = w.bytes ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();     // returned here: not the next launch's error too
+    return e;
 }
 
 // The same without a window.

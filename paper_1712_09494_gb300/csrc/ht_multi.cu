@@ -119,6 +119,7 @@ void destroy_multi(ht_multi* m) {
     for (void* p : m->states) cudaFree(p);
     for (ht_table* t : m->tables) ht_destroy(t);
     if (m->stream) cudaStreamDestroy(m->stream);
+    cudaGetLastError();               // of a creation that failed: its status says so
     delete m;
 }
 

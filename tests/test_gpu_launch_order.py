@@ -77,3 +77,20 @@ def test_captured_and_replayed(scheme, slots, n):
     g2.replay()
     torch.cuda.synchronize()
     assert bool(flags.all()) and t.size() == n
+
+
+def test_a_failed_allocation_is_no_later_calls_error():
+    keys = _keys(1000, 64, 1)
+    small = ht.HashTable(4000, "bucket", 64)
+    flags = torch.empty(1000, dtype=torch.uint8, device="cuda")
+    out = torch.empty(1000, dtype=torch.int64, device="cuda")
+    for r in range(2):
+        for scheme in ("bucket", "cuckoo"):
+            with pytest.raises(ht.HtError) as err:
+                ht.HashTable(1 << 39, scheme, 64)            # 4 TB
+            assert err.value.status == 2
+            small.clear()
+            ht.ht_multi_find_or_put([small.handle], [(0, keys, flags)])
+            count = torch.zeros(1, dtype=torch.int64, device="cuda")
+            ht.ht_compact(keys, flags, out, count)
+            assert int(count) == 1000 and small.size() == 1000
