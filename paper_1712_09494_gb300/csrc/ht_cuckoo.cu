@@ -50,12 +50,12 @@
 namespace ht {
 namespace {
 
-constexpr int kU = 4;                   // eviction chains in flight per thread (insert)
+constexpr int kU = 4;                   // keys or eviction chains in flight per thread
 constexpr int kStage = 96;              // staged winners per warp
-// Resident blocks per SM that the probe is compiled for: find-or-put 4 (fill of
-// 2^27 keys, not reordered, 14.4 ms; 14.5 at 3, 14.7 at 5), lookup 5.
+// Resident blocks per SM that the probe with a queue is compiled for (fill of 2^27
+// keys in region order 12.7 ms; 13.3 at 3, 13.5 at 5).
 constexpr int kProbeBlocks = 4;
-constexpr int kLookupBlocks = 5;
+constexpr int kFarBlocks = 3;           // fill of 2^26 keys to load 0.5 4.91 ms; 4.96 at 2
 
 // Adds the block's per-warp sums (held by each warp's lane 0) to N table
 // counters with one atomic per counter and block, not per warp: the last
@@ -104,48 +104,23 @@ __device__ __noinline__ bool spill_holds(const DevTable& t, uint64_t key, uint32
     return find_spill<KW>(t, key, stash_used, ovf_used, w);
 }
 
-// Probe (and, for find-or-put, the stores and the dedup).  One lane per key; a
-// pass reads one slot, h_(a+1), for each key of a tile of 32 fresh keys or of 32
-// that wait in the warp's queue (bucket::Pending) for their next slot: every
-// lane of a pass has a slot to read, whatever the other keys' paths.  A key is
-// settled by the slot that holds it or by the first EMPTY one (a key never sits
-// past an empty slot of its own), 1.63 slots per key over a fill to load 0.8.
-// Past L2 bound by random lines (27 G slot reads and 11 G CASes a second; the
-// same time with four keys per thread in lock step, at twice the registers);
-// in region order 7.8 instead of 10.8 ms of the 2^27-key fill; in L2 a replay
-// of 10^8 keys of 100 occurrences takes 1.87 ms (2.16 in lock step).
-// AHEAD: tables past L2; the next tile's first slots are touched a tile ahead.
-template <int KW, bool VALUES, bool LOOKUP, bool AHEAD>
-__global__ void __launch_bounds__(kBlock, LOOKUP ? kLookupBlocks : kProbeBlocks)
-cuckoo_probe_kernel(const __grid_constant__ DevTable t, const __grid_constant__ DevScratch sc, uint32_t parity,
-                    const void* __restrict__ keys, const uint32_t* __restrict__ vals, uint64_t n,
-                    const unsigned long long* __restrict__ d_n, uint64_t off,
-                    uint8_t* __restrict__ out_flag, uint32_t* __restrict__ out_val, bool list_stored) {
-    using K = Keys<KW>;
-    pdl_wait();
-    if (d_n) {                                   // batch size produced on the device
-        const uint64_t total = __ldcg(d_n);
-        n = total > off ? min(n, total - off) : 0;
-    }
-    const uint32_t stash_used = __ldcg(&t.ctr->stash_used);
-    const uint32_t ovf_used = __ldcg(&t.ctr->ovf_used);
-    const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
-    const uint64_t dseed = t.aux_seed * 3 + 1;
-    const int lane = threadIdx.x & 31;
-    unsigned long long probes = 0;            // slots read
-    unsigned long long misses = 0, miss_reads = 0;   // keys found nowhere, and the slots they read
-    unsigned long long direct = 0;            // CASes of absent keys into table slots
-    unsigned long long stored = 0;            // keys stored here and not listed
-    __shared__ StagedWinner s_win[LOOKUP ? 1 : kBlock / 32][LOOKUP ? 1 : kStage];
-    __shared__ bucket::PendEntry s_pend[kBlock / 32][bucket::kPend];
-    StagedWinner* stage = s_win[LOOKUP ? 0 : (threadIdx.x >> 5)];
-    bucket::Pending queue(s_pend[threadIdx.x >> 5]);
+// A warp's stage of winners in shared memory, listed with one atomic on the
+// winner count per flush, so that no pass waits on a shared counter.
+template <int KW>
+struct WinnerStage {
+    const DevTable& t;
+    const DevScratch& sc;
+    uint32_t parity;
+    uint8_t* out_flag;
+    StagedWinner* stage;
     uint32_t pend = 0;
-    // Lists the staged winners: one atomic on the winner count per flush.
+    __device__ WinnerStage(const DevTable& t, const DevScratch& sc, uint32_t parity, uint8_t* out_flag, StagedWinner* stage)
+        : t(t), sc(sc), parity(parity), out_flag(out_flag), stage(stage) {}
     // Entries past the list's capacity (more winners than the table holds)
     // give their claim back, are reported dropped and lose their flag --
     // unless the probe stored them already.
-    auto flush = [&]() {
+    __device__ void flush() {
+        const int lane = threadIdx.x & 31;
         __syncwarp();
         if (pend) {
             unsigned int b = 0;
@@ -172,7 +147,89 @@ cuckoo_probe_kernel(const __grid_constant__ DevTable t, const __grid_constant__ 
         }
         __syncwarp();
         pend = 0;
-    };
+    }
+    // Called by all lanes of the warp.
+    __device__ __forceinline__ void add(bool listed, uint64_t word, uint64_t i, uint32_t spos, bool placed) {
+        const unsigned wm = __ballot_sync(0xFFFFFFFFu, listed);
+        if (!wm) return;
+        if (pend + __popc(wm) > uint32_t(kStage)) flush();
+        if (listed) {
+            StagedWinner& e = stage[pend + __popc(wm & ((1u << (threadIdx.x & 31)) - 1))];
+            e.word = word;
+            e.i = i;
+            e.spos = spos;
+            e.start = placed ? kStartPlaced : 0u;
+        }
+        pend += __popc(wm);
+    }
+};
+
+// A miss that found all k slots full goes through the claim set: the one
+// claimant of each such key wins and runs an eviction chain from h_1 in the
+// insert kernel.  Each CASes its key into its slot of the claim set (kept in
+// L2); a slot holding another key sends it on by linear probing.
+template <int KW>
+__device__ __forceinline__ bool claim_key(const DevTable& t, const DevScratch& sc, uint64_t dseed, uint64_t key,
+                                          uint32_t* spos) {
+    const int rc = lp_insert<KW>(sc.set, uint32_t(sc.mask + 1), mix64(key ^ dseed) & sc.mask, key, key, spos);
+    if (rc < 0) {                                  // more distinct misses than the table holds
+        set_flag(t.ctr, kFlagDropped);
+        atomicAdd(&t.ctr->dropped, 1ull);
+    }
+    return rc == 1;
+}
+
+// The probe's sums over the block, to the table: the last step of a kernel.
+__device__ __forceinline__ void add_probe_counters(const DevTable& t, unsigned long long probes, unsigned long long misses,
+                                                   unsigned long long miss_reads, unsigned long long direct,
+                                                   unsigned long long stored) {
+    for (int o = 16; o; o >>= 1) {
+        probes += __shfl_down_sync(0xFFFFFFFFu, probes, o);
+        misses += __shfl_down_sync(0xFFFFFFFFu, misses, o);
+        miss_reads += __shfl_down_sync(0xFFFFFFFFu, miss_reads, o);
+        direct += __shfl_down_sync(0xFFFFFFFFu, direct, o);
+        stored += __shfl_down_sync(0xFFFFFFFFu, stored, o);
+    }
+    unsigned long long* const dst[5] = {&t.ctr->size, &t.ctr->probes, &t.ctr->probe_cas, &t.ctr->probe_misses,
+                                        &t.ctr->probe_miss_reads};
+    const unsigned long long sums[5] = {stored, probes, direct, misses, miss_reads};
+    block_add_counters<5>(dst, sums);
+}
+
+// Probe, with the stores and the dedup.  One lane per key; a
+// pass reads one slot, h_(a+1), for each key of a tile of 32 fresh keys or of 32
+// that wait in the warp's queue (bucket::Pending) for their next slot: every
+// lane of a pass has a slot to read, whatever the other keys' paths.  A key is
+// settled by the slot that holds it or by the first EMPTY one (a key never sits
+// past an empty slot of its own), 1.63 slots per key over a fill to load 0.8.
+// For tables in L2 and batches in region order, where round trips are short: the
+// 2^27-key fill in region order takes 7.8 instead of 10.8 ms; in L2 a replay
+// of 10^8 keys of 100 occurrences takes 1.87 ms (2.16 with the kernel below).
+template <int KW, bool VALUES>
+__global__ void __launch_bounds__(kBlock, kProbeBlocks)
+cuckoo_probe_kernel(const __grid_constant__ DevTable t, const __grid_constant__ DevScratch sc, uint32_t parity,
+                    const void* __restrict__ keys, const uint32_t* __restrict__ vals, uint64_t n,
+                    const unsigned long long* __restrict__ d_n, uint64_t off,
+                    uint8_t* __restrict__ out_flag, bool list_stored) {
+    using K = Keys<KW>;
+    pdl_wait();
+    if (d_n) {                                   // batch size produced on the device
+        const uint64_t total = __ldcg(d_n);
+        n = total > off ? min(n, total - off) : 0;
+    }
+    const uint32_t stash_used = __ldcg(&t.ctr->stash_used);
+    const uint32_t ovf_used = __ldcg(&t.ctr->ovf_used);
+    const uint64_t step = uint64_t(gridDim.x) * blockDim.x;
+    const uint64_t dseed = t.aux_seed * 3 + 1;
+    const int lane = threadIdx.x & 31;
+    unsigned long long probes = 0;            // slots read
+    unsigned long long misses = 0, miss_reads = 0;   // keys found nowhere, and the slots they read
+    unsigned long long direct = 0;            // CASes of absent keys into table slots
+    unsigned long long stored = 0;            // keys stored here and not listed
+    __shared__ StagedWinner s_win[kBlock / 32][kStage];
+    __shared__ bucket::PendEntry s_pend[kBlock / 32][bucket::kPend];
+    bucket::Pending queue(s_pend[threadIdx.x >> 5]);
+    WinnerStage<KW> winners(t, sc, parity, out_flag, s_win[threadIdx.x >> 5]);
     uint64_t base = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) / 32 * 32;
     // This tile's key and slot, the next tile's key.
     uint64_t key0 = 0, key1 = 0;
@@ -201,7 +258,6 @@ cuckoo_probe_kernel(const __grid_constant__ DevTable t, const __grid_constant__ 
             if (mine && !ok) set_flag(t.ctr, kFlagInvalidKey);
             key0 = key1;
             slot0 = hidx(key0, t.seed[0], t.nslots);
-            if (AHEAD && base + step + lane < n) touch_l2(t.slots + slot0);
             if (base + 2 * step + lane < n) key1 = K::load(keys, base + 2 * step + lane);
             base += step;
         } else {
@@ -219,112 +275,196 @@ cuckoo_probe_kernel(const __grid_constant__ DevTable t, const __grid_constant__ 
         }
         if (waits) ++d.probe;
         queue.push(waits, d);
-        if constexpr (LOOKUP) {
-            if (mine && !waits) {
-                if (out_flag) out_flag[d.pos] = uint8_t(found);
-                if (out_val) out_val[d.pos] = found ? K::value(w) : 0u;
-            }
-        } else {
-            if (miss) {
-                ++misses;
-                miss_reads += d.probe + 1;
-            }
-            // A miss that saw an EMPTY slot stores itself there with a CAS
-            // from EMPTY, trying its slots in order from that one: a CAS that
-            // returns the key means another copy stored it first (not new);
-            // one that returns another key moves on to the next slot, which
-            // the CAS reads as well.  This is the bucket scheme's claim in
-            // a fixed order (Section 4.2), over h_a..h_k.  Nothing leaves a slot
-            // during the probe kernel, so a key is stored in at most one slot
-            // and every copy probed later finds it; a copy that saw all k
-            // slots full read each after it was full, so no copy stores
-            // it in the table here.  With t.chain_h1 only an EMPTY h_1 is
-            // tried (Section 4.1 starts every insertion at h_1).
-            bool placed = false;
-            bool cas = miss && K::empty(w) && (!t.chain_h1 || d.probe == 0);
-            bool claim = miss && !cas;
-            while (cas) {                          // bounded: on to the next of k slots
-                const uint64_t cw = atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + at), kEmpty,
-                                              K::word(d.key, VALUES ? vals[d.pos] : 0u));
-                ++direct;
-                cas = false;
-                if (cw == kEmpty) {
-                    placed = true;
-                } else if (K::keyof(cw) == d.key) {
-                    // another copy stored it
-                } else if (t.chain_h1 || d.probe + 1 >= t.k) {
-                    claim = true;                  // every slot is full now
-                } else {
-                    ++d.probe;
-                    at = hidx(d.key, t.seed[d.probe], t.nslots);
-                    cas = true;
-                }
-            }
-            __syncwarp();
-            // The misses that found all k slots full go through the claim
-            // set: the one claimant of each such key wins and runs an
-            // eviction chain from h_1 in the insert kernel.  Each CASes its
-            // key into its slot of the claim set (kept in L2); a slot holding
-            // another key sends it on by linear probing.
-            bool winner = placed;
-            uint32_t spos = 0;
-            if (claim) {
-                const int rc = lp_insert<KW>(sc.set, uint32_t(sc.mask + 1), mix64(d.key ^ dseed) & sc.mask, d.key, d.key,
-                                             &spos);
-                winner = rc == 1;
-                if (rc < 0) {                      // more distinct misses than the table holds
-                    set_flag(t.ctr, kFlagDropped);
-                    atomicAdd(&t.ctr->dropped, 1ull);
-                }
-            }
-            if (mine && !waits && out_flag) out_flag[d.pos] = uint8_t(winner);
-            // Winners go to the warp's stage in shared memory, listed with one
-            // atomic per flush, so that no pass waits on a shared counter.
-            // Keys this kernel stored are listed only for a caller that appends
-            // the new keys (list_stored); otherwise they are just counted.
-            const bool listed = winner && (list_stored || !placed);
-            stored += placed && !list_stored;
-            const unsigned wm = __ballot_sync(0xFFFFFFFFu, listed);
-            if (wm) {
-                if (pend + __popc(wm) > uint32_t(kStage)) flush();
-                if (listed) {
-                    StagedWinner& e = stage[pend + __popc(wm & ((1u << lane) - 1))];
-                    e.word = K::word(d.key, VALUES ? vals[d.pos] : 0u);
-                    e.i = d.pos;
-                    e.spos = spos;
-                    e.start = placed ? kStartPlaced : 0u;
-                }
-                pend += __popc(wm);
+        if (miss) {
+            ++misses;
+            miss_reads += d.probe + 1;
+        }
+        // A miss that saw an EMPTY slot stores itself there with a CAS
+        // from EMPTY, trying its slots in order from that one: a CAS that
+        // returns the key means another copy stored it first (not new);
+        // one that returns another key moves on to the next slot, which
+        // the CAS reads as well.  This is the bucket scheme's claim in
+        // a fixed order (Section 4.2), over h_a..h_k.  Nothing leaves a slot
+        // during the probe kernel, so a key is stored in at most one slot
+        // and every copy probed later finds it; a copy that saw all k
+        // slots full read each after it was full, so no copy stores
+        // it in the table here.  With t.chain_h1 only an EMPTY h_1 is
+        // tried (Section 4.1 starts every insertion at h_1).
+        bool placed = false;
+        bool cas = miss && K::empty(w) && (!t.chain_h1 || d.probe == 0);
+        bool claim = miss && !cas;
+        while (cas) {                          // bounded: on to the next of k slots
+            const uint64_t cw = atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + at), kEmpty,
+                                          K::word(d.key, VALUES ? vals[d.pos] : 0u));
+            ++direct;
+            cas = false;
+            if (cw == kEmpty) {
+                placed = true;
+            } else if (K::keyof(cw) == d.key) {
+                // another copy stored it
+            } else if (t.chain_h1 || d.probe + 1 >= t.k) {
+                claim = true;                  // every slot is full now
+            } else {
+                ++d.probe;
+                at = hidx(d.key, t.seed[d.probe], t.nslots);
+                cas = true;
             }
         }
+        __syncwarp();
+        bool winner = placed;
+        uint32_t spos = 0;
+        if (claim) winner = claim_key<KW>(t, sc, dseed, d.key, &spos);
+        if (mine && !waits && out_flag) out_flag[d.pos] = uint8_t(winner);
+        // Keys this kernel stored are listed only for a caller that appends
+        // the new keys (list_stored); otherwise they are just counted.
+        stored += placed && !list_stored;
+        const bool listed = winner && (list_stored || !placed);
+        winners.add(listed, listed ? K::word(d.key, VALUES ? vals[d.pos] : 0u) : 0, d.pos, spos, placed);
     }
-    if constexpr (!LOOKUP) flush();
-    for (int o = 16; o; o >>= 1) {
-        probes += __shfl_down_sync(0xFFFFFFFFu, probes, o);
-        if (!LOOKUP) {
-            misses += __shfl_down_sync(0xFFFFFFFFu, misses, o);
-            miss_reads += __shfl_down_sync(0xFFFFFFFFu, miss_reads, o);
-            direct += __shfl_down_sync(0xFFFFFFFFu, direct, o);
-            stored += __shfl_down_sync(0xFFFFFFFFu, stored, o);
-        }
-    }
-    if constexpr (LOOKUP) {
-        unsigned long long* const dst[1] = {&t.ctr->probes};
-        const unsigned long long sums[1] = {probes};
-        block_add_counters<1>(dst, sums);
-    } else {
-        unsigned long long* const dst[5] = {&t.ctr->size, &t.ctr->probes, &t.ctr->probe_cas, &t.ctr->probe_misses,
-                                            &t.ctr->probe_miss_reads};
-        const unsigned long long sums[5] = {stored, probes, direct, misses, miss_reads};
-        block_add_counters<5>(dst, sums);
-    }
+    winners.flush();
+    add_probe_counters(t, probes, misses, miss_reads, direct, stored);
 }
 
-// Lookup in a table that fits in L2: four keys per thread, one slot of each at
-// a time until it is found or meets an EMPTY slot.  With L2's short latency the
-// probe kernel's queue costs more than the lanes it keeps busy (20 M lookups,
-// half absent, in 8 MB: 276 us there, 246 here; 32-bit keys with values 380, 265;
-// in 500 MB 928 us there, 994 here).
+// The same with four keys per thread in lock step, one slot of each at a time
+// until all are settled, then their CASes.  For tables past L2 whose batch is not
+// in region order: bound by random lines, read and then claimed, of which it keeps
+// 96 warps' worth in flight per SM (the queue 32).  Fills to load 0.5: 2^26 keys in
+// batches of 2^22 4.91 ms (5.12 with the queue), 2^27 in 2^24 10.4 (10.8); 2^25 to
+// load 0.85 in batches of 2^21 3.47 (3.76 with one more array of words per key
+// in registers and 2 blocks per SM).
+template <int KW, bool VALUES>
+__global__ void __launch_bounds__(kBlock, kFarBlocks)
+cuckoo_probe_far_kernel(const __grid_constant__ DevTable t, const __grid_constant__ DevScratch sc, uint32_t parity,
+                        const void* __restrict__ keys, const uint32_t* __restrict__ vals, uint64_t n,
+                        const unsigned long long* __restrict__ d_n, uint64_t off, uint8_t* __restrict__ out_flag,
+                        bool list_stored) {
+    using K = Keys<KW>;
+    pdl_wait();
+    if (d_n) {                                   // batch size produced on the device
+        const uint64_t total = __ldcg(d_n);
+        n = total > off ? min(n, total - off) : 0;
+    }
+    const uint32_t stash_used = __ldcg(&t.ctr->stash_used);
+    const uint32_t ovf_used = __ldcg(&t.ctr->ovf_used);
+    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
+    const uint64_t tid = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    const uint64_t rounds = (n + stride * kU - 1) / (stride * kU);     // warp-uniform trip count
+    const uint64_t dseed = t.aux_seed * 3 + 1;
+    unsigned long long probes = 0, misses = 0, miss_reads = 0, direct = 0, stored = 0;
+    __shared__ StagedWinner s_win[kBlock / 32][kStage];
+    WinnerStage<KW> winners(t, sc, parity, out_flag, s_win[threadIdx.x >> 5]);
+    // The next round's keys are loaded while this round waits on the table.
+    uint64_t next_key[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+        const uint64_t i = uint64_t(u) * stride + tid;
+        next_key[u] = i < n ? K::load(keys, i) : 0;
+    }
+    for (uint64_t r = 0; r < rounds; ++r) {
+        uint64_t key[kU], w[kU];
+        uint32_t at[kU];                         // the function whose slot was read last
+        bool act[kU], found[kU], more[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            act[u] = (r * kU + u) * stride + tid < n;
+            key[u] = next_key[u];
+            const uint64_t j = ((r + 1) * kU + u) * stride + tid;
+            if (j < n) next_key[u] = K::load(keys, j);
+            if (act[u] && K::reserved(key[u])) {
+                set_flag(t.ctr, kFlagInvalidKey);
+                act[u] = false;
+            }
+            more[u] = act[u];
+            found[u] = false;
+            w[u] = kEmpty;
+            at[u] = 0;
+        }
+        for (uint32_t a = 0; a < t.k; ++a) {
+            bool any = false;
+#pragma unroll
+            for (int u = 0; u < kU; ++u) any |= more[u];
+            if (!__any_sync(0xFFFFFFFFu, any)) break;
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+                if (more[u])
+                    w[u] = __ldcg(reinterpret_cast<const unsigned long long*>(t.slots + hidx(key[u], t.seed[a], t.nslots)));
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                if (!more[u]) continue;
+                ++probes;
+                at[u] = a;
+                found[u] = K::keyof(w[u]) == key[u];
+                more[u] = !found[u] && !K::empty(w[u]);
+            }
+        }
+        // The CASes of the misses that saw an EMPTY slot, in slot order from it,
+        // by the rules of the kernel above.
+        bool placed[kU], claim[kU], cas[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const bool empty = K::empty(w[u]);
+            uint64_t kept;
+            if (act[u] && !found[u] && (stash_used | ovf_used))
+                found[u] = spill_holds<KW>(t, key[u], stash_used, ovf_used, &kept);
+            const bool miss = act[u] && !found[u];
+            misses += miss;
+            miss_reads += miss ? at[u] + 1 : 0;
+            cas[u] = miss && empty && (!t.chain_h1 || at[u] == 0);
+            claim[u] = miss && !cas[u];
+            placed[u] = false;
+        }
+        for (uint32_t pass = 0; pass < t.k; ++pass) {
+            bool any = false;
+#pragma unroll
+            for (int u = 0; u < kU; ++u) any |= cas[u];
+            if (!__any_sync(0xFFFFFFFFu, any)) break;
+            uint64_t cw[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+                if (cas[u]) {
+                    cw[u] = atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + hidx(key[u], t.seed[at[u]], t.nslots)),
+                                      kEmpty, K::word(key[u], VALUES ? vals[(r * kU + u) * stride + tid] : 0u));
+                    ++direct;
+                }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                if (!cas[u]) continue;
+                if (cw[u] == kEmpty) {
+                    placed[u] = true;
+                    cas[u] = false;
+                } else if (K::keyof(cw[u]) == key[u]) {
+                    cas[u] = false;                        // another copy stored it
+                } else if (t.chain_h1 || at[u] + 1 >= t.k) {
+                    claim[u] = true;                       // every slot is full now
+                    cas[u] = false;
+                } else {
+                    ++at[u];
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const uint64_t i = (r * kU + u) * stride + tid;
+            bool winner = placed[u];
+            uint32_t spos = 0;
+            if (claim[u]) winner = claim_key<KW>(t, sc, dseed, key[u], &spos);
+            if (i < n && out_flag) out_flag[i] = uint8_t(winner);
+            stored += placed[u] && !list_stored;
+            const bool listed = winner && (list_stored || !placed[u]);
+            winners.add(listed, listed ? K::word(key[u], VALUES ? vals[i] : 0u) : 0, i, spos, placed[u]);
+        }
+    }
+    winners.flush();
+    add_probe_counters(t, probes, misses, miss_reads, direct, stored);
+}
+
+// Lookup: four keys per thread, one slot of each at a time until it is found or
+// meets an EMPTY slot.  Without claims to wait for, a queue costs more than the
+// lanes it keeps busy: 20 M lookups, half absent, in 8 MB 276 us with the probe
+// kernel's queue, 246 here, 32-bit keys with values 380, 265; past L2 at load 0.5
+// (2^24 lookups) 662 us, 605 here in 1 GB, 32-bit keys with values 502, 385 in 270
+// MB.  Touching the next round's first slots ahead gives nothing (605, 411 us).
+// Past L2 bound by random lines.
 template <int KW>
 __global__ void __launch_bounds__(kBlock, 3)
 cuckoo_lookup_kernel(const __grid_constant__ DevTable t, const void* __restrict__ keys, uint64_t n,
@@ -531,12 +671,12 @@ cudaError_t cuckoo_probe(int kw, const DevTable& t, const DevScratch& sc, uint32
                          const unsigned long long* d_n, uint64_t off, uint8_t* is_new, cudaStream_t s,
                          const L2Window& w, bool list_stored, bool local) {
     ProfScope ps(kKCuckooProbe, s);
-    const bool past_l2 = !local && t.nslots * 8 > l2_bytes();
+    const bool far = !local && t.nslots * 8 > l2_bytes();
 #define L(KW, V)                                                                                        \
     {                                                                                                   \
-        auto k = past_l2 ? cuckoo_probe_kernel<KW, V, false, true> : cuckoo_probe_kernel<KW, V, false, false>; \
+        auto k = far ? cuckoo_probe_far_kernel<KW, V> : cuckoo_probe_kernel<KW, V>;                     \
         return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, w, t, sc, parity, keys, vals, \
-                          n, d_n, off, is_new, (uint32_t*)nullptr, list_stored);                        \
+                          n, d_n, off, is_new, list_stored);                                            \
     }
     if (kw == 32) {
         if (vals) L(32, true) else L(32, false)
@@ -566,14 +706,8 @@ cudaError_t cuckoo_insert(int kw, const DevTable& t, const DevScratch& sc, uint3
 cudaError_t cuckoo_lookup(int kw, const DevTable& t, const void* keys, uint64_t n, uint32_t* vals,
                           uint8_t* found, cudaStream_t s, const L2Window& w) {
     ProfScope ps(kKCuckooLookup, s);
-    if (t.nslots * 8 <= l2_bytes()) {
-        auto k = kw == 32 ? cuckoo_lookup_kernel<32> : cuckoo_lookup_kernel<64>;
-        return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, w, t, keys, n, found, vals);
-    }
-    DevScratch none{};
-    auto k = kw == 32 ? cuckoo_probe_kernel<32, false, true, true> : cuckoo_probe_kernel<64, false, true, true>;
-    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, w, t, none, 0u, keys,
-                      (const uint32_t*)nullptr, n, (const unsigned long long*)nullptr, uint64_t(0), found, vals, false);
+    auto k = kw == 32 ? cuckoo_lookup_kernel<32> : cuckoo_lookup_kernel<64>;
+    return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, w, t, keys, n, found, vals);
 }
 
 }  // namespace ht

@@ -244,8 +244,9 @@ __device__ __forceinline__ uint32_t half_pass(uint64_t* slots, ulonglong2 key, u
 // (staged per warp in shared memory; entries past new_cap not written).
 // d_n (nullable): the batch size produced on the device, at most n.
 // ahead: a lookup in a table larger than L2 touches the next tile's buckets.
-// Fill of 2^26 keys to load 0.8 in batches of 2^24: 3.97 ms (whole buckets, not
-// reordered: 4.15; before, a round of the tile at a time: 5.40); of 2^22 keys in
+// Fill of 2^26 keys to load 0.8 in batches of 2^24: 3.7 ms (side by side with
+// plain launches 3.97; whole buckets, not reordered: 4.15; before, a round of the
+// tile at a time: 5.40); of 2^22 keys in
 // L2 198 us (313).  Blocks per SM: whole 3 (2: 4.90, 4: 5.27 ms), halves 4 (3:
 // 3.99, 5: 4.30).
 template <bool LOOKUP, bool APPEND, bool HALF>

@@ -204,3 +204,42 @@ def test_reordered_batch_of_one_key_and_reserved_keys():
     assert int(flags[:1_000_000].sum()) == 1 and int(flags.sum()) == 1 + 2_000_000 - 2000
     assert int(flags[::1000].sum()) == 0
     assert t.sync() == 1 and t.size() == 1 + 2_000_000 - 2000
+
+
+@pytest.mark.parametrize("k,h1,load", [(2, 0, 0.4), (4, 0, 0.85), (4, 1, 0.85), (8, 0, 0.9)])
+@pytest.mark.parametrize("kw", [32, 64])
+def test_cuckoo_table_past_l2_in_the_batchs_order(kw, k, h1, load):
+    """Cuckoo tables larger than L2 with batches too small to be reordered: each key of a batch is new in exactly one
+    of its two places, stored keys are not, and lookups return the stored values."""
+    from workloads import device_keys as dk
+    slots = 24_000_000                                  # 192 MB; reordered from 1.9 M keys
+    n = int(slots * load)
+    idx = torch.arange(2 * n, dtype=torch.int64, device="cuda")
+    if kw == 64:
+        keys = dk.mix63_perm_dev(idx, k)
+    else:
+        d = dk.mix32_perm_dev(idx, k)
+        keys = (d - ((d >> 31) << 32)).to(torch.int32)
+    t = ht.HashTable(slots, "cuckoo", kw, dict(num_hashes=k, cuckoo_chain_h1=h1))
+    vals = (idx[:n] * 3 + 1).to(torch.int32)
+    at = first = 0
+    if kw == 32:
+        at = first = n // 2 + 7
+        t.insert(keys[:at], vals[:at])                  # the rest of the keys get value 0
+    sizes = [1, 31, 33, 700_001]
+    while at < n:
+        m = min(sizes.pop(0) if sizes else 650_000, n - at)
+        rep = torch.randint(0, at, (m // 2,), device="cuda") if at else idx[:0]
+        order = torch.randperm(2 * m + len(rep), device="cuda")
+        f = t.find_or_put(torch.cat([keys[at:at + m], keys[at:at + m], keys[rep]])[order])
+        g = torch.zeros_like(f)
+        g[order] = f
+        assert bool((g[:m] + g[m:2 * m] == 1).all()) and not bool(g[2 * m:].any())
+        at += m
+    found, v = t.lookup(keys)
+    assert torch.equal(found, (idx < n).to(torch.uint8))
+    if kw == 32:
+        want = torch.zeros(2 * n, dtype=torch.int32, device="cuda")
+        want[:first] = vals[:first]
+        assert torch.equal(v, want)
+    assert t.sync() == 0 and t.size() == n
