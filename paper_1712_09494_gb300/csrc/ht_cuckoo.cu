@@ -55,7 +55,6 @@ constexpr int kStage = 96;              // staged winners per warp
 // Resident blocks per SM that the probe with a queue is compiled for (fill of 2^27
 // keys in region order 12.7 ms; 13.3 at 3, 13.5 at 5).
 constexpr int kProbeBlocks = 4;
-constexpr int kFarBlocks = 3;           // fill of 2^26 keys to load 0.5 4.91 ms; 4.96 at 2
 
 // Adds the block's per-warp sums (held by each warp's lane 0) to N table
 // counters with one atomic per counter and block, not per warp: the last
@@ -328,12 +327,12 @@ cuckoo_probe_kernel(const __grid_constant__ DevTable t, const __grid_constant__ 
 // The same with four keys per thread in lock step, one slot of each at a time
 // until all are settled, then their CASes.  For tables past L2 whose batch is not
 // in region order: bound by random lines, read and then claimed, of which it keeps
-// 96 warps' worth in flight per SM (the queue 32).  Fills to load 0.5: 2^26 keys in
-// batches of 2^22 4.91 ms (5.12 with the queue), 2^27 in 2^24 10.4 (10.8); 2^25 to
-// load 0.85 in batches of 2^21 3.47 (3.76 with one more array of words per key
-// in registers and 2 blocks per SM).
-template <int KW, bool VALUES>
-__global__ void __launch_bounds__(kBlock, kFarBlocks)
+// 64 or 96 warps' worth in flight per SM (the queue 32).  Fills to load 0.5: 2^26
+// keys in batches of 2^22 4.96 ms (5.12 with the queue), 2^27 in 2^24 10.53 (10.83).
+// BLOCKS per SM: 3 while a part of the lines is found in L2, 2 past four times L2
+// (cuckoo_probe), where more in flight only queue.
+template <int KW, bool VALUES, int BLOCKS>
+__global__ void __launch_bounds__(kBlock, BLOCKS)
 cuckoo_probe_far_kernel(const __grid_constant__ DevTable t, const __grid_constant__ DevScratch sc, uint32_t parity,
                         const void* __restrict__ keys, const uint32_t* __restrict__ vals, uint64_t n,
                         const unsigned long long* __restrict__ d_n, uint64_t off, uint8_t* __restrict__ out_flag,
@@ -671,10 +670,15 @@ cudaError_t cuckoo_probe(int kw, const DevTable& t, const DevScratch& sc, uint32
                          const unsigned long long* d_n, uint64_t off, uint8_t* is_new, cudaStream_t s,
                          const L2Window& w, bool list_stored, bool local) {
     ProfScope ps(kKCuckooProbe, s);
-    const bool far = !local && t.nslots * 8 > l2_bytes();
+    // Tables past L2 with a batch in its own order.  Blocks per SM, 2 / 3: a map of
+    // 2^24 keys in 170 MB 1.48 / 1.36 ms, 2^25 keys in 320 MB 3.81 / 3.68; 2^26 in 670
+    // MB equal, in 1 GB 5.03 / 5.14, 2^27 in 2.1 GB 10.63 / 10.85.
+    const uint64_t bytes = t.nslots * 8, l2 = l2_bytes();
+    const bool far = !local && bytes > l2, near = bytes <= 4 * l2;
 #define L(KW, V)                                                                                        \
     {                                                                                                   \
-        auto k = far ? cuckoo_probe_far_kernel<KW, V> : cuckoo_probe_kernel<KW, V>;                     \
+        auto k = !far ? cuckoo_probe_kernel<KW, V>                                                      \
+                      : near ? cuckoo_probe_far_kernel<KW, V, 3> : cuckoo_probe_far_kernel<KW, V, 2>;   \
         return launch_win(k, launch_grid((const void*)k, kBlock, n, kBlock), kBlock, 0, s, w, t, sc, parity, keys, vals, \
                           n, d_n, off, is_new, list_stored);                                            \
     }

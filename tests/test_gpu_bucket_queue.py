@@ -206,14 +206,14 @@ def test_reordered_batch_of_one_key_and_reserved_keys():
     assert t.sync() == 1 and t.size() == 1 + 2_000_000 - 2000
 
 
-@pytest.mark.parametrize("k,h1,load", [(2, 0, 0.4), (4, 0, 0.85), (4, 1, 0.85), (8, 0, 0.9)])
+@pytest.mark.parametrize("k,h1,load,slots", [(2, 0, 0.4, 24_000_000), (4, 0, 0.85, 24_000_000), (4, 1, 0.85, 24_000_000),
+                                             (8, 0, 0.9, 24_000_000), (4, 0, 0.1, 80_000_000)])
 @pytest.mark.parametrize("kw", [32, 64])
-def test_cuckoo_table_past_l2_in_the_batchs_order(kw, k, h1, load):
+def test_cuckoo_table_past_l2_in_the_batchs_order(kw, k, h1, load, slots):
     """Cuckoo tables larger than L2 with batches too small to be reordered: each key of a batch is new in exactly one
     of its two places, stored keys are not, and lookups return the stored values."""
     from workloads import device_keys as dk
-    slots = 24_000_000                                  # 192 MB; reordered from 1.9 M keys
-    n = int(slots * load)
+    n = int(slots * load)                               # 192 and 640 MB; reordered from 1.9 and 6.3 M keys
     idx = torch.arange(2 * n, dtype=torch.int64, device="cuda")
     if kw == 64:
         keys = dk.mix63_perm_dev(idx, k)
