@@ -596,7 +596,8 @@ ht_status ht_probe_random_rmw(void* d_buf, uint64_t bytes, uint64_t n_access, ui
  * device array inside the library (8 MiB, held on every GPU that uses the
  * library until the process exits).  No cudaMalloc or cudaFree is called.
  *
- * d_slots   caller-owned device array of nslots uint64 words: the table.
+ * d_slots   caller-owned device array of nslots uint64 words (8-byte
+ *           aligned): the table.
  * d_state   caller-owned device block of HT_NOALLOC_STATE_BYTES bytes,
  *           16-byte aligned: counters, a 101-word stash and a 64-word
  *           overflow area.  After the work completes:

@@ -49,13 +49,20 @@ export_kernel(const DevTable t, typename Keys<KW>::T* __restrict__ keys_out,
     }
 }
 
+// n words of p to v, 16 bytes a store.  p may be 8-byte aligned only (the caller's
+// table of ht_noalloc.cu): the word before the first 16-byte boundary and the one
+// after the last are stored alone.
 __global__ void __launch_bounds__(kBlock) fill_kernel(uint64_t* __restrict__ p, uint64_t n, uint64_t v) {
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-    const uint64_t n2 = n / 2;
-    ulonglong2* q = reinterpret_cast<ulonglong2*>(p);
+    const uint64_t head = min(n, uint64_t(reinterpret_cast<uintptr_t>(p) >> 3) & 1);
+    const uint64_t n2 = (n - head) / 2;
+    ulonglong2* q = reinterpret_cast<ulonglong2*>(p + head);
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n2; i += stride)
         q[i] = make_ulonglong2(v, v);
-    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) p[n - 1] = v;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (head) p[0] = v;
+        if ((n - head) & 1) p[n - 1] = v;
+    }
 }
 
 // Words [0, n) of p to EMPTY by threads [tid] of [nthreads], 32 bytes a store
