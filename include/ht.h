@@ -141,7 +141,8 @@ ht_status ht_default_params(ht_scheme scheme, ht_params* p);
  * clears them on `stream`; use the table on other streams only after work
  * on `stream` is ordered before that use.
  * key_width 32, 64 or 128: 128-bit keys are two 64-bit words (low word
- * first, 16-byte aligned, bit 63 of the high word reserved) for state
+ * first; arrays of them 16-byte aligned, else HT_ERR_INVALID; bit 63 of the
+ * high word reserved) for state
  * vectors wider than 64 bits, in 16-byte slots written with 16-byte atomics
  * (compare-and-swap claims, exchange evictions for Cuckoo); bucket scheme:
  * buckets of 8 slots (bucket_slots must be 8, lanes_per_key 2 or 4; with

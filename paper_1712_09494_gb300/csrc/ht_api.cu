@@ -46,6 +46,10 @@ void derive_seeds(ht_table* t) {
 
 bool is_long(uint32_t kw) { return kw > 128; }
 
+// Arrays of 128-bit keys are read and written 16 bytes at a time; at another
+// address each access would fault.
+bool key_aligned(uint32_t kw, const void* p) { return kw != 128 || (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 BucketCfg bucket_cfg(const ht_table* t) {
     return BucketCfg{int(t->kw), int(t->p.bucket_slots)};
 }
@@ -690,6 +694,7 @@ static ht_status put_common(ht_table* t, const void* keys, const uint32_t* vals,
     if (vals && t->kw != 32) return HT_ERR_INVALID;
     if ((new_out == nullptr) != (new_count == nullptr)) return HT_ERR_INVALID;
     if (is_long(t->kw) && (new_out || (reinterpret_cast<uintptr_t>(keys) & 7))) return HT_ERR_INVALID;
+    if (n && !(key_aligned(t->kw, keys) && key_aligned(t->kw, new_out))) return HT_ERR_INVALID;
     DeviceGuard g(t->device);
     return run_put(t, keys, vals, n, is_new, new_out, new_count, as_stream(stream));
 }
@@ -720,7 +725,7 @@ ht_status ht_lookup(ht_table* t, const void* d_keys, uint64_t n, uint32_t* d_val
         return cuda_status(long_lookup(t->dt, d_keys, n, d_found, s));
     }
     if (t->kw == 128) {
-        if (d_values) return HT_ERR_INVALID;
+        if (d_values || !key_aligned(128, d_keys)) return HT_ERR_INVALID;
         if (t->scheme == HT_CUCKOO) return cuda_status(wide_cuckoo_lookup(t->dt, d_keys, n, d_found, s));
         return cuda_status(wide_lookup(t->dt, d_keys, n, d_found, s));
     }
@@ -986,6 +991,7 @@ ht_status ht_successors(const ht_model* h_model, uint32_t key_width, const void*
         return HT_ERR_INVALID;
     if (!model_max_successors(h_model, key_width)) return HT_ERR_INVALID;
     if (n == 0) return HT_OK;
+    if (!(key_aligned(key_width, d_states) && key_aligned(key_width, d_succ))) return HT_ERR_INVALID;
     const cudaStream_t s = as_stream(stream);
     DevBuf dm;
     const PreparedModel pm = prepare_model(*h_model);
@@ -1003,7 +1009,7 @@ static ht_status bfs_common(ht_table* t, const ht_model* h_model, uint64_t s0, u
     if (!t || !result) return HT_ERR_INVALID;
     if (fused && (t->scheme != HT_BUCKET || t->kw == 128)) return HT_ERR_INVALID;
     const uint64_t msucc = model_max_successors(h_model, t->kw);
-    if (!msucc) return HT_ERR_INVALID;
+    if (!msucc || !key_aligned(t->kw, d_states)) return HT_ERR_INVALID;
     if (t->kw == 32 ? s0 >= 0xFFFFFFFFull : (s0 >> 63) != 0) return HT_ERR_INVALID;
     DeviceGuard g(t->device);
     const cudaStream_t s = as_stream(stream);
