@@ -355,9 +355,11 @@ typedef struct ht_bfs_result {
  * With a 128-bit table (models wider than 63 bits) states are 16-byte
  * pairs (low word first) and s0 is the initial state's low word (its high
  * word is 0).
- * Allocates its work buffers in the order of `stream` (cudaMallocAsync) and
- * frees them there before returning; a table keeps up to 16 MB of them, or as
- * much as its slots take, until it is destroyed, for its next exploration. */
+ * Allocates its work buffers in the order of `stream` (cudaMallocAsync).  Those
+ * of more than 512 MB (the states, where d_states is NULL) are back with the
+ * device when it returns, smaller ones from the next synchronisation on; a
+ * table keeps up to 16 MB of them, or as much as its slots take, until it is
+ * destroyed, for its next exploration. */
 ht_status ht_bfs(ht_table* t, const ht_model* h_model, uint64_t s0, uint32_t max_levels,
                  uint64_t* h_level_sizes, void* d_states, uint64_t states_cap,
                  ht_bfs_result* result, void* stream);

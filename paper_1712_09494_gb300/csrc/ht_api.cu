@@ -965,19 +965,46 @@ struct DevBuf {
     ~DevBuf() { cudaFree(p); }
 };
 
-// Stream-ordered device memory, freed in the stream's order unless it is kept.
+// Stream-ordered device memory, freed when it goes out of scope unless it is kept.
+// Freed memory goes back to the device at the next synchronisation.  A large
+// buffer (the states, where the caller gives none) is followed by one: the caller
+// may want that memory for cudaMalloc next.  A smaller one is not, and the
+// next exploration mostly finds it in the pool again (0.7 M states of 128 bits,
+// 60 MB of work memory: 1.43 ms, 1.68 with the unmapping and mapping).
+constexpr size_t kBfsLarge = 512u << 20;
 struct BfsMem {
     explicit BfsMem(cudaStream_t st) : s(st) {}
     void* p = nullptr;
+    size_t size = 0;
     bool keep = false;
     cudaStream_t s;
-    cudaError_t alloc(size_t bytes) { return cudaMallocAsync(&p, bytes, s); }
+    cudaError_t alloc(size_t bytes) {
+        size = bytes;
+        return cudaMallocAsync(&p, bytes, s);
+    }
     void take(void* q) {
         p = q;
         keep = true;
     }
     ~BfsMem() {
-        if (p && !keep) cudaFreeAsync(p, s);
+        if (!p || keep) return;
+        cudaFreeAsync(p, s);
+        if (size > kBfsLarge) cudaStreamSynchronize(s);
+    }
+};
+
+// The reordering scratch that an exploration leaves its table: none past `most`
+// bytes.
+struct PartTrim {
+    ht_table* t;
+    cudaStream_t s;
+    size_t most;
+    ~PartTrim() {
+        if (t->part_bytes <= most) return;
+        cudaFreeAsync(t->part, s);
+        t->part = nullptr;
+        t->part_bytes = 0;
+        cudaStreamSynchronize(s);
     }
 };
 
@@ -1034,6 +1061,7 @@ static ht_status bfs_common(ht_table* t, const ht_model* h_model, uint64_t s0, u
     const size_t model_bytes = (sizeof(PreparedModel) + 255) / 256 * 256;
     const size_t need = model_bytes + 256 + 256 + succ_cap * ksz;
     BfsMem work(s), states_own(s);
+    const PartTrim trim{t, s, std::max<uint64_t>(256u << 20, slots * 8)};
     if (t->bfs_bytes >= need) {
         work.take(t->bfs_mem);
     } else {
@@ -1138,13 +1166,7 @@ static ht_status bfs_common(ht_table* t, const ht_model* h_model, uint64_t s0, u
     HT_TRY(cudaMemcpyAsync(&gen, c + 2, sizeof(gen), cudaMemcpyDeviceToHost, s));
     HT_TRY(cudaStreamSynchronize(s));
     result->successors = gen;
-    if (t->part_bytes > std::max<uint64_t>(256u << 20, slots * 8)) {     // nor reordering scratch past that size
-        cudaFreeAsync(t->part, s);
-        t->part = nullptr;
-        t->part_bytes = 0;
-    }
-    const ht_status ts = sync_and_status(t, s);
-    return ts;
+    return sync_and_status(t, s);
 }
 
 ht_status ht_bfs(ht_table* t, const ht_model* h_model, uint64_t s0, uint32_t max_levels, uint64_t* h_level_sizes,
