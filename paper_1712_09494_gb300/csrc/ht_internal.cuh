@@ -452,9 +452,10 @@ cudaError_t table_export(int kw, const DevTable& t, void* keys_out, uint32_t* va
                          unsigned long long* count, uint64_t cap, cudaStream_t s);
 cudaError_t fill_words(uint64_t* p, uint64_t n, uint64_t v, cudaStream_t s);
 // Empties a table (its slots and overflow entries are of 1 or 2 words), or n
-// tables of one-word slots whose descriptors are in device memory.
+// tables of one-word slots, the largest of most_slots, whose descriptors are in
+// device memory.
 cudaError_t clear_words(const DevTable& t, uint32_t slot_words, uint32_t ovf_words, cudaStream_t s);
-cudaError_t clear_many(const DevTable* tables, uint32_t n, cudaStream_t s);
+cudaError_t clear_many(const DevTable* tables, uint32_t n, uint64_t most_slots, cudaStream_t s);
 cudaError_t compact(int kw, const void* keys, const uint8_t* flags, uint64_t n, void* out,
                     unsigned long long* count, cudaStream_t s);
 cudaError_t probe_random_read(const void* buf, uint64_t bytes, uint32_t gran, uint64_t n_access,

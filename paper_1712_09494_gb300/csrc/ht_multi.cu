@@ -158,7 +158,9 @@ ht_status reset_multi(ht_multi* m) {
     for (ht_table* t : m->tables) table_forget(t);
     for (auto& g : m->groups) {
         const uint64_t n = g.members.size();
-        if (clear_many(g.dev.tables, uint32_t(n), m->stream) != cudaSuccess) return HT_ERR_CUDA;
+        uint64_t most = 0;
+        for (uint32_t e : g.members) most = std::max(most, table_dev(m->tables[e]).nslots);
+        if (clear_many(g.dev.tables, uint32_t(n), most, m->stream) != cudaSuccess) return HT_ERR_CUDA;
         // Zero every counter array (they sit contiguously at the arena's start).
         const char* first = reinterpret_cast<const char*>(g.dev.total);
         const char* last = reinterpret_cast<const char*>(g.dev.steps) + 256;
