@@ -270,16 +270,19 @@ long_bucket_kernel(const __grid_constant__ DevTable t, const uint64_t* __restric
             old = atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + slot0 + sl), kEmpty, tag | kBusy);
         }
         if (match) touch_l2(t.kstore + (slot0 + __ffs(match) - 1) * RW);
+        // A match whose header is not published yet is left for later: the lanes of
+        // the warp that won a claim publish theirs before any lane waits, so a wait
+        // is for a lane that waits on nothing.
+        uint32_t busy = 0;
         while (match && !found) {
-            const int ms = __ffs(match) - 1;
+            const uint32_t ms = __ffs(match) - 1;
             match &= match - 1;
-            found = slot_holds(t, slot0 + ms, key, W, RW);
+            if (ld_acquire(t.slots + slot0 + ms) & kBusy) busy |= 1u << ms;
+            else found = row_is(t.kstore + (slot0 + ms) * RW, key, W);
         }
-        bool full = act && !found;
-        if (LOOKUP) {
-            full &= empty == 0;                    // an EMPTY slot: the key would sit in this bucket
-        } else {
-            while (empty && full) {
+        // Bounded: busy is empty after the first turn.
+        for (;;) {
+            while (!LOOKUP && empty && !busy && !found && !claimed) {
                 uint64_t* hdr = t.slots + slot0 + sl;
                 if (!sent) {
                     sl = bucket::first_from<kLBS>(empty, uint32_t(d.digest >> 7) % kLBS);
@@ -292,12 +295,20 @@ long_bucket_kernel(const __grid_constant__ DevTable t, const uint64_t* __restric
                     copy_row(t.kstore + (slot0 + sl) * RW, key, W, RW);
                     st_release(hdr, tag);
                     claimed = true;
-                    full = false;
-                } else if ((old & ~kBusy) == tag && slot_holds(t, slot0 + sl, key, W, RW)) {
-                    full = false;
+                } else if ((old & ~kBusy) == tag) {
+                    found = slot_holds(t, slot0 + sl, key, W, RW);
                 }
             }
+            if (!__any_sync(kFullMask, busy != 0)) break;
+            while (busy && !found) {
+                const uint32_t ms = __ffs(busy) - 1;
+                busy &= busy - 1;
+                found = slot_holds(t, slot0 + ms, key, W, RW);
+            }
+            busy = 0;
         }
+        // A lookup's key would sit in a bucket with an EMPTY slot.
+        const bool full = act && !found && !claimed && (!LOOKUP || empty == 0);
         __syncwarp();
         // Still searching: the bucket is full; the next function, if any.
         bool waits = full;

@@ -245,27 +245,29 @@ class LongWarps:
     """The long-key bucket kernel's pass, two or more lanes to a warp (warps: each lane's warp).  A header is EMPTY,
     ("busy", tag) or ("ready", tag); row: the slot's key.  In a pass every lane of a warp reads its bucket's
     headers; lanes without a tag match send their first claim (from a slot that the digest gives, around the
-    bucket); claims won are published; then lanes with a match wait for that header's publish and compare, and
-    the others go on claiming.  The lanes of a warp go through these steps together: a lane may not start a step
-    before its warp's lanes have ended the one before.  late: the former order, in which a claim that was sent is
-    published only after the warp's lanes have checked their matches."""
+    bucket); lanes with matches compare those that are published; the lanes with no unpublished match settle their
+    claims; then the others wait for theirs, compare, and claim.  The lanes of a warp go through these steps together: a
+    lane may not start a step before its warp's lanes have ended the one before.  late: another order, in which
+    unpublished matches are waited for before the claims that were sent are published."""
 
-    RANK = dict(read=0, sent=1, write=2, publish=2, match=3, wait=3, claim=4, lwait=4, lwrite=4, lpublish=4)
-    LATE = dict(RANK, write=4, publish=4)
+    RANK = dict({"read": 0, "sent": 1, "match": 2, "wait": 4}, **{p: 3 for p in ("claim", "lwait", "write", "publish")},
+                **{p + "+": 5 for p in ("claim", "lwait", "write", "publish")})
+    LATE = dict(RANK, wait=2)
 
     def __init__(self, keys, warps, tag, start, seq, S=2, nbuckets=1, late=False):
         self.keys, self.warps, self.tag, self.begin, self.seq, self.S = list(keys), list(warps), tag, start, seq, S
         self.rank = self.LATE if late else self.RANK
         n = S * nbuckets
-        # lane state: (pc, bucket number, headers read, slots left, matches left, slot, result)
-        self.start = (tuple([EMPTY] * n), tuple([None] * n), tuple(("read", 0, (), (), (), None, None) for _ in keys))
+        # lane state: (pc, bucket number, headers read, slots left, matches left, unpublished ones, slot, result)
+        lane = ("read", 0, (), (), (), (), None, None)
+        self.start = (tuple([EMPTY] * n), tuple([None] * n), tuple(lane for _ in keys))
 
     def _held(self, lane):
-        return lane[0] in ("write", "publish", "lwrite", "lpublish")
+        return lane[0].rstrip("+") in ("write", "publish")
 
     def step(self, state, i):
         hdr, row, lanes = state
-        pc, f, seen, empty, match, slot, res = lanes[i]
+        pc, f, seen, empty, match, busy, slot, res = lanes[i]
         if pc == "done":
             return None
         at = (f, self.rank[pc])
@@ -276,52 +278,51 @@ class LongWarps:
         tag = self.tag[key]
         base = self.seq[key][f] * self.S
         hdr, row = list(hdr), list(row)
+        more = "+" if pc == "wait" or pc.endswith("+") else ""      # the second turn of the claims
 
-        def put(*new):
+        def put(pc, empty=(), match=(), busy=(), slot=None, res=None, f=f, seen=()):
             t = list(lanes)
-            t[i] = new
+            t[i] = (pc, f, seen, empty, match, busy, slot, res)
             return (tuple(hdr), tuple(row), tuple(t))
-
-        def claim(slots, won, lost):
-            s = slots[0]
-            old = hdr[s]
-            if old == EMPTY:
-                hdr[s] = ("busy", tag)
-                return put(won, f, (), slots[1:], (), s, None)
-            if old[1] == tag:
-                return put("lwait", f, (), slots[1:], (), s, None)
-            return put(lost, f, (), slots[1:], (), None, None)
 
         if pc == "read":
             seen = seen + (hdr[base + len(seen)],)
             if len(seen) < self.S:
-                return put("read", f, seen, (), (), None, None)
+                return put("read", seen=seen)
             m = tuple(base + s for s, h in enumerate(seen) if h != EMPTY and h[1] == tag)
             e = tuple(base + s for s in _around(self.begin[tag], self.S) if seen[s] == EMPTY)
-            return put("sent" if e and not m else "match", f, (), e, m, None, None)
-        if pc == "sent":
-            return claim(empty, "write", "claim")
-        if pc in ("write", "lwrite"):
-            row[slot] = key
-            return put("publish" if pc == "write" else "lpublish", f, (), (), (), slot, None)
-        if pc in ("publish", "lpublish"):
-            hdr[slot] = ("ready", tag)
-            return put("done", f, (), (), (), None, "claimed")
-        if pc == "match":
-            if match:
-                return put("wait", f, (), empty, match[1:], match[0], None)
-            return put("claim", f, (), empty, (), None, None)
-        if pc in ("wait", "lwait"):
-            if hdr[slot][0] == "busy":
+            return put("sent" if e and not m else "match", e, m)
+        if pc == "match":                     # published matches are compared, the others left for later
+            if not match:
+                return put("wait" if busy else "claim", empty, busy=busy)
+            if hdr[match[0]][0] == "busy":
+                return put("match", empty, match[1:], busy + match[:1])
+            if row[match[0]] == key:
+                return put("done", res="found")
+            return put("match", empty, match[1:], busy)
+        if pc in ("wait", "lwait", "lwait+"):
+            s = busy[0] if pc == "wait" else slot
+            if hdr[s][0] == "busy":
                 return None
-            if row[slot] == key:
-                return put("done", f, (), (), (), None, "found")
-            return put("match" if pc == "wait" else "claim", f, (), empty, match, None, None)
-        if empty:                             # claim
-            return claim(empty, "lwrite", "claim")
+            if row[s] == key:
+                return put("done", res="found")
+            return put("wait" if busy[1:] else "claim" + more, empty, busy=busy[1:])
+        if pc.startswith("write"):
+            row[slot] = key
+            return put("publish" + more, slot=slot)
+        if pc.startswith("publish"):
+            hdr[slot] = ("ready", tag)
+            return put("done", res="claimed")
+        if empty:                             # sent, claim, claim+: a compare-and-swap from EMPTY
+            s = empty[0]
+            old = hdr[s]
+            if old == EMPTY:
+                hdr[s] = ("busy", tag)
+                return put("write" + more, slot=s)
+            return put("lwait" + more, empty[1:], slot=s) if old[1] == tag else put("claim" + more, empty[1:])
         if f + 1 < len(self.seq[key]):
-            return put("read", f + 1, (), (), (), None, None)
-        return put("done", f, (), (), (), None, "full")
+            return put("read", f=f + 1)
+        return put("done", res="full")
 
     def run(self, limit=3_000_000):
         """(wrong final or stuck states, states in which a lane with an unpublished claim is held up by a lane of its
@@ -342,7 +343,7 @@ class LongWarps:
                 stored = [row[s] for s, h in enumerate(hdr) if h != EMPTY]
                 ok = all(x[0] == "done" for x in lanes) and len(stored) == len(set(stored))
                 for k in set(self.keys):
-                    res = sorted(x[6] or "" for j, x in enumerate(lanes) if self.keys[j] == k)
+                    res = sorted(x[7] or "" for j, x in enumerate(lanes) if self.keys[j] == k)
                     ok &= res == (["claimed"] + ["found"] * (len(res) - 1) if k in stored else ["full"] * len(res))
                 if not ok:
                     wrong.append(st)
@@ -367,7 +368,7 @@ def test_a_long_key_claim_waits_on_nothing_before_its_publish(keys, warps, S, nb
 
 
 def test_a_claim_held_while_its_warp_waits_is_caught():
-    """The former order gives the same answers, but a header stays busy while its owner's warp waits for another's."""
+    """The late order gives the same answers, but a header stays busy while its owner's warp waits for another's."""
     keys, warps, S, nb = CASES[0]
     wrong, held_up = LongWarps(keys, warps, TAG, {1: 0, 2: 0, 3: 0}, {k: [0] for k in TAG}, S, nb, late=True).run()
     assert not wrong and held_up
