@@ -178,7 +178,17 @@ ht_status ht_destroy(ht_table* t);
  * d_keys: n keys (uint32 or uint64 by key_width).  d_is_new (nullable): n
  * bytes, 1 where this call stored the key.  Among equal keys of one batch
  * exactly one is flagged (which one is unspecified).  On a map the stored
- * value is 0. */
+ * value is 0.
+ * Memory: a batch with more than 1.25 keys for each 128 bytes of a table's
+ * slots, in a table larger than L2 (keys of up to 128 bits, without values), is
+ * first put in the order of the table's regions.  The scratch for that -- up to
+ * 12 bytes a key, 20 for 128-bit keys, of at most 2^24 keys at a time, and no
+ * more than the slots take -- is allocated in the order of `stream`
+ * (cudaMallocAsync) by this call, ht_find_or_put_append, ht_insert or a Cuckoo
+ * table's part of ht_multi_find_or_put, and kept by the table until it is
+ * destroyed.  Where it cannot be had, or while
+ * `stream` is being captured, the batch goes in its own order: slower, with the
+ * same results. */
 ht_status ht_find_or_put(ht_table* t, const void* d_keys, uint64_t n,
                          uint8_t* d_is_new, void* stream);
 
@@ -359,7 +369,10 @@ typedef struct ht_bfs_result {
  * of more than 512 MB (the states, where d_states is NULL) are back with the
  * device when it returns, smaller ones from the next synchronisation on; a
  * table keeps up to 16 MB of them, or as much as its slots take, until it is
- * destroyed, for its next exploration. */
+ * destroyed, for its next exploration.  The scratch for large levels in the
+ * order of the table's regions (ht_find_or_put) takes as much again as their
+ * successors (at most 2^26 vectors); a table keeps up to 256 MB of it, or as
+ * much as its slots take. */
 ht_status ht_bfs(ht_table* t, const ht_model* h_model, uint64_t s0, uint32_t max_levels,
                  uint64_t* h_level_sizes, void* d_states, uint64_t states_cap,
                  ht_bfs_result* result, void* stream);

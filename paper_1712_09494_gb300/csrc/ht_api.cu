@@ -167,9 +167,20 @@ void* part_scratch(ht_table* t, size_t need, cudaStream_t s) {
     return t->part;
 }
 
-// Keys of one reordered piece: counters fit 32 bits, and its scratch (190 MB
-// with flags) stays a fraction of a table that wants it.
-constexpr uint64_t kPartPiece = 1ull << 24;
+// Keys of one reordered piece of a batch of n: at most 2^24 (its counters take 32
+// bits, its scratch 190 MB of 64-bit keys with flags, 320 MB of 128-bit ones), so
+// a table past 1.7 GB, whose lines get fewer than 1.25 keys each from that many,
+// is filled in the batch's order; and scratch for no more than the table's
+// slots, which leaves 6 keys for each line and more (half of the slots: fills of
+// tables of 140 to 340 MB 1 to 6% slower, replays into them 4 to 10%).
+uint64_t part_piece(const ht_table* t, uint64_t n, bool with_flags) {
+    const uint64_t bytes = t->dt.nslots * (t->kw == 128 ? 16 : 8);
+    // A key, its flag, its place and its share of the tiles' runs; the rest is for
+    // the counters and the alignment of each array.
+    const uint64_t per_key = t->kw / 8 + (with_flags ? 4 : 0), rest = 4096;
+    const uint64_t fit = bytes > rest ? (bytes - rest) / per_key / kPartTile * kPartTile : 0;
+    return std::min({n, uint64_t(1) << 24, fit});
+}
 
 // Runs op(keys, count, flags, local) over a batch: in pieces in region order
 // where that pays (local), with the flags brought back to the batch's order,
@@ -178,7 +189,7 @@ template <class Op>
 ht_status in_region_order(ht_table* t, const void* keys, uint64_t n, const unsigned long long* d_n, uint8_t* flags,
                           cudaStream_t s, Op&& op) {
     const size_t ksz = t->kw / 8;
-    const uint64_t piece = d_n ? n : std::min(n, kPartPiece);
+    const uint64_t piece = d_n ? n : part_piece(t, n, flags != nullptr);
     const int bits = region_bits(t, d_n ? piece / 2 : piece);        // d_n: about half of the bound
     void* p = bits ? part_scratch(t, PartScratch(nullptr, piece, ksz, flags != nullptr, bits).bytes, s) : nullptr;
     if (!p) return op(keys, n, flags, false);

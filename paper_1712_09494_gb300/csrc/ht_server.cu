@@ -74,6 +74,9 @@ struct Slot {
     std::chrono::steady_clock::time_point issued;
 };
 
+// What a table takes when it is created.  Not counted is what a Cuckoo table past L2
+// allocates for a request so large that it is reordered (ht_api.cu): without that
+// memory the request goes in its own order, so no table has to wait for it.
 uint64_t table_bytes(uint64_t capacity, ht_scheme scheme, const ht_params& p) {
     const uint64_t bs = p.bucket_slots ? p.bucket_slots : 16;
     const uint64_t slots = (capacity + bs - 1) / bs * bs;
