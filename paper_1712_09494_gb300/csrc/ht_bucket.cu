@@ -246,7 +246,12 @@ cudaError_t launch_multi(const MultiDev& m, uint64_t max_tiles, bool init, cudaS
 // items and each warp takes a contiguous range of them, finds its first
 // tile's item once and walks the items in order, keeping the item's
 // descriptor in registers and its table's size count until it moves on.
-template <int KW, int BS>
+// WHOLE: buckets are read whole, for launches of few keys, by the single-table
+// kernel's rule and for its reason (batches of 2^15 keys into one table of 32 MB, us
+// by sectors / whole: at load 0.5 56 / 56, at 0.8 63 / 56, at 0.9 80 / 65).  In
+// launches of many keys sectors are the better one to load 0.7, also past L2 (2^19
+// keys into 268 MB at load 0.5 70 / 79, at 0.8 89 / 82).
+template <int KW, int BS, bool WHOLE>
 __global__ void __launch_bounds__(kBlock, 4)
 packed_bucket_kernel(const DevTable* __restrict__ tables, const WorkDesc* __restrict__ items, uint32_t nitems,
                      uint64_t ntiles) {
@@ -297,7 +302,7 @@ packed_bucket_kernel(const DevTable* __restrict__ tables, const WorkDesc* __rest
             p.sec = first_sector<BS / kSec>(p.key, hidx(p.key, t.seed[0], t.nbuckets));
         }
         bool waits;
-        const uint32_t st = put_pass<KW, BS, false, false>(tables[d.table], pend, p, ok, waits);
+        const uint32_t st = put_pass<KW, BS, WHOLE, false>(tables[d.table], pend, p, ok, waits);
         if (mine && !waits && d.flags) d.flags[p.pos] = uint8_t(st);
         stored += __popc(__ballot_sync(kFull, st == kKeyHit));
     }
@@ -445,7 +450,8 @@ cudaError_t packed_bucket_find_or_put(const BucketCfg& c, const DevTable* tables
     ProfScope ps(kKBucketFop, s);
 #define L(KW, BS)                                                                                      \
     {                                                                                                     \
-        auto k = packed_bucket_kernel<KW, BS>;                                                         \
+        auto k = ntiles * 32 < kSectorKeys ? packed_bucket_kernel<KW, BS, true>                           \
+                                           : packed_bucket_kernel<KW, BS, false>;                         \
         const int grid = int(std::min<uint64_t>(launch_blocks((const void*)k, kBlock), (ntiles + 7) / 8)); \
         k<<<grid, kBlock, 0, s>>>(tables, items, nitems, ntiles);                                         \
         return cudaGetLastError();                                                                        \
