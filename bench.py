@@ -792,7 +792,7 @@ def run_batched(ht, torch):
                                                      r["batched_persistent"]["seconds"], 2)
         mx.close()
         # Autotuned: each exploration's capacity class tuned once (bucket:
-        # width, lanes, hash functions; Cuckoo: hash functions, eviction
+        # width, hash functions; Cuckoo: hash functions, eviction
         # bound) for a BFS-like repeat rate, then the persistent run.
         import tempfile
         from paper_1712_09494_gb300 import autotune
@@ -923,9 +923,8 @@ def run_wide(ht, torch, dev, n_log2=26, batch_log2=24, dup=0.25, lf=0.8, reps=3)
     pairs = [torch.stack([b, dk.mix63_perm_dev(b, 92)], dim=1).contiguous() for b in batches]
     issued = sum(p.shape[0] for p in pairs)
     flags = torch.empty(max(p.shape[0] for p in pairs), dtype=torch.uint8, device=dev)
-    for name, sch, params in (("bucket_lanes2", "bucket", dict(lanes_per_key=2)),
-                              ("bucket_lanes4", "bucket", dict(lanes_per_key=4)), ("cuckoo", "cuckoo", None)):
-        t = ht.HashTable(int(np.ceil(n / lf)), sch, 128, params)
+    for name in ("bucket", "cuckoo"):
+        t = ht.HashTable(int(np.ceil(n / lf)), name, 128)
         times = []
         for r in range(reps + 1):
             ht.ht_clear(t.handle)
