@@ -332,7 +332,10 @@ __device__ __forceinline__ void add_size(const DevTable& t, unsigned long long s
 // exploration once and then walks on in order with that exploration's
 // descriptor in registers; each tile runs against exploration e's table
 // (addressed as a 64-bit key table, which a 32-bit set table's words also
-// are) and its new states are appended to e's states.
+// are) and its new states are appended to e's states.  By sectors at every size:
+// most successors are stored already and found in the first one (256 explorations of
+// 440 MB together 18.8 ms; one of 49 M states, 560 MB, by sectors / whole 35.5 / 42.2
+// ms at load 0.7, 41.1 / 44.6 at 0.9, 56.0 / 55.2 at 0.97).
 constexpr int kMultiStage = kStageCap / 2;     // with the queues and tile map, under 48 KB a block
 
 template <int BS>

@@ -210,9 +210,9 @@ struct LongEntry {
     uint32_t f;        // the hash function to try next
     uint32_t pad_;
 };
-// (3 blocks per SM: 3.32 ms per fill of 2^25 256-bit keys; 3.36 at 4, 4.33 with
-// eight-lane reads of the buckets and the key's words held in registers, whose
-// lookups ran at 8.4 G/s; now 23.)
+// (3 blocks per SM: 3.27 ms per fill of 2^25 256-bit keys; 3.36 at 4, 4.33 with
+// eight-lane reads of the buckets and the key's words held in registers.  Lookups
+// in that table, half absent, run at 17.7 G/s.)
 template <bool LOOKUP>
 __global__ void __launch_bounds__(kBlock, 3)
 long_bucket_kernel(const __grid_constant__ DevTable t, const uint64_t* __restrict__ keys, uint64_t n,

@@ -3,7 +3,8 @@
 //
 // A slot is 16 bytes: the key's low word, then its high word.  EMPTY is all
 // ones in both; a key's top bit (bit 63 of the high word) is reserved, so no
-// key is EMPTY.  A bucket is 8 slots (one 128-byte line) read by G lanes.
+// key is EMPTY.  A bucket is 8 slots (one 128-byte line), read whole by two
+// lanes or, in large batches where the table's lines are in L2, half by one lane.
 // A claim is one 16-byte compare-and-swap (atom.cas.b128), so a slot goes
 // from EMPTY to a key at once and never changes again.
 //
@@ -13,9 +14,11 @@
 // at least one all-ones word.  So a slot read with neither word all ones is
 // a complete key (and stays so); a slot with both all ones, or exactly one,
 // is a claim candidate whose true content the claiming CAS returns.  Claims
-// go in slot order over the candidates (the slot-order argument of the
-// 64-bit kernels: a key is claimed in at most one slot), and only the CAS
-// result decides, so stale or torn reads cannot duplicate a key.
+// go over the candidates in an order that the key gives: half after half of
+// the bucket from one of them, and in each half from one of its slots (the
+// 64-bit kernels' argument, by halves instead of sectors: a key is claimed in
+// at most one slot), and only the CAS result decides, so stale or torn reads
+// cannot duplicate a key.
 #include "ht_bucket_tile.cuh"
 
 namespace ht {
