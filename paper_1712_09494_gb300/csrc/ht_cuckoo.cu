@@ -463,9 +463,9 @@ cuckoo_probe_far_kernel(const __grid_constant__ DevTable t, const __grid_constan
 // kernel's queue, 246 here, 32-bit keys with values 380, 265; past L2 at load 0.5
 // (2^24 lookups) 662 us, 605 here in 1 GB, 32-bit keys with values 502, 385 in 270
 // MB.  Touching the next round's first slots ahead gives nothing (605, 411 us).
-// Past L2 bound by random lines, in L2 by instruction issue: 2^24 lookups of stored
-// keys in 10 MB take 198 us, 193 with all functions unrolled, which costs other
-// lookups more (32-bit ones at load 0.5 past L2 433 us, 446).
+// Past L2 bound by random lines.  In L2 2^24 lookups of stored keys (10 MB) take 198
+// us, 193 with the kernel before it, which held all k words of a key and is
+// slower on others (2^22 32-bit ones 56 us, 51 here; past L2 at load 0.5 446, 433).
 template <int KW>
 __global__ void __launch_bounds__(kBlock, 3)
 cuckoo_lookup_kernel(const __grid_constant__ DevTable t, const void* __restrict__ keys, uint64_t n,
