@@ -365,10 +365,11 @@ typedef struct ht_bfs_result {
  * With a 128-bit table (models wider than 63 bits) states are 16-byte
  * pairs (low word first) and s0 is the initial state's low word (its high
  * word is 0).
- * Allocates its work buffers in the order of `stream` (cudaMallocAsync).  Those
- * of more than 512 MB (the states, where d_states is NULL) are back with the
- * device when it returns, smaller ones from the next synchronisation on; a
- * table keeps up to 16 MB of them, or as much as its slots take, until it is
+ * Allocates its work buffers in the order of `stream` (cudaMallocAsync).  A
+ * buffer for the states (where d_states is NULL) of more than 512 MB is back
+ * with the device when it returns; the rest, at most 2^26 successors, is from
+ * the next synchronisation on, except that a table keeps up to 16 MB of
+ * successors, or as much as its slots take, until it is
  * destroyed, for its next exploration.  The scratch for large levels in the
  * order of the table's regions (ht_find_or_put) takes as much again as their
  * successors (at most 2^26 vectors); a table keeps up to 256 MB of it, or as

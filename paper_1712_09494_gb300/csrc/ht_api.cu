@@ -980,18 +980,16 @@ struct DevBuf {
 };
 
 // Stream-ordered device memory, freed when it goes out of scope unless it is kept.
-// Freed memory goes back to the device at the next synchronisation.  A large
-// buffer (the states, where the caller gives none) is followed by one: the caller
-// may want that memory for cudaMalloc next.  A smaller one is not, and the
-// next exploration mostly finds it in the pool again (0.7 M states of 128 bits,
-// 60 MB of work memory: 1.43 ms, 1.68 with the unmapping and mapping).
-constexpr size_t kBfsLarge = 512u << 20;
+// Freed memory goes back to the device at the next synchronisation.  A buffer of
+// more than `most` bytes is followed by one: the caller may want that memory for
+// cudaMalloc next.
 struct BfsMem {
-    explicit BfsMem(cudaStream_t st) : s(st) {}
+    BfsMem(cudaStream_t st, size_t most) : s(st), most(most) {}
     void* p = nullptr;
     size_t size = 0;
     bool keep = false;
     cudaStream_t s;
+    size_t most;
     cudaError_t alloc(size_t bytes) {
         size = bytes;
         return cudaMallocAsync(&p, bytes, s);
@@ -1003,7 +1001,7 @@ struct BfsMem {
     ~BfsMem() {
         if (!p || keep) return;
         cudaFreeAsync(p, s);
-        if (size > kBfsLarge) cudaStreamSynchronize(s);
+        if (size > most) cudaStreamSynchronize(s);
     }
 };
 
@@ -1074,7 +1072,10 @@ static ht_status bfs_common(ht_table* t, const ht_model* h_model, uint64_t s0, u
     // 1800 and, with the reordering scratch, 2 ms of a large one's 50.
     const size_t model_bytes = (sizeof(PreparedModel) + 255) / 256 * 256;
     const size_t need = model_bytes + 256 + 256 + succ_cap * ksz;
-    BfsMem work(s), states_own(s);
+    // The states can be most of the device's memory.  The work block is 2^26 successors
+    // at most, and the next exploration mostly finds it in the pool again (0.7 M and 29
+    // M states of 128 bits 1.43 and 36.1 ms; 1.68 and 37.9 where it is unmapped).
+    BfsMem work(s, ~size_t(0)), states_own(s, 512u << 20);
     const PartTrim trim{t, s, std::max<uint64_t>(256u << 20, slots * 8)};
     if (t->bfs_bytes >= need) {
         work.take(t->bfs_mem);

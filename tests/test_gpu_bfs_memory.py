@@ -1,5 +1,5 @@
-"""Device memory of an exploration: what it allocates for itself, but for two buffers of up to 512 MB, is free again
-when it returns, without a synchronisation by the caller, whether it ends, is stopped or cannot be run."""
+"""Device memory of an exploration: the states it keeps for itself, where they are large, are free again when it
+returns, without a synchronisation by the caller, whether it ends, is stopped or cannot be run."""
 import math
 
 import numpy as np
